@@ -59,9 +59,9 @@ extern "C" {
 
 /* ---- precision modes ------------------------------------------------------------- */
 #define DG_FP64 0     /* everything in float64                                             */
-#define DG_MIXED 1    /* bracket and viscous term in double-float on the float32 pipe (see  */
-                      /* dg_bracket_mixed), inner CG in float32, float64 refinement, state  */
-#define DG_MIXED64 2  /* bracket in float64, inner CG in float32, float64 refinement, state  */
+#define DG_MIXED 1    /* inner CG in float32, float64 refinement and state; the bracket and  */
+                      /* viscous term as in DG_FP64 (dg_bracket_mixed)                      */
+#define DG_MIXED64 2  /* the same as DG_MIXED (they differed in the bracket's arithmetic)   */
 #define DG_FP64_PC32 3 /* float64 everywhere except the CG preconditioner, applied in float32 */
                        /* (a float32 copy of the cell block solve and the coarse DFT solve)   */
 
@@ -209,10 +209,7 @@ int dg_bracket_parts(dg_grid* g, const double* psi, const double* omega, double*
 
 /*
  * dg_bracket_mixed -- the bracket of dg_bracket (Eq. J) as the DG_MIXED time stepper evaluates
- * it: the same operations in double-float arithmetic on the float32 pipe (each value the
- * unevaluated sum of two floats, about 48 significant bits; Dekker's TwoProduct and Knuth's
- * TwoSum), read from and written to float64 arrays.  Products are rounded one by one, so
- * J(f, f) = 0 holds bitwise as in float64.  Arguments and errors as dg_bracket.
+ * it: the same arithmetic as dg_bracket.  Arguments and errors as dg_bracket.
  */
 int dg_bracket_mixed(dg_grid* g, const double* psi, const double* omega, double* J, void* stream);
 
@@ -320,8 +317,7 @@ int dg_sim_get(dg_sim* s, double* omega, double* psi, void* stream);
 /*
  * dg_sim_get_state / dg_sim_set_state -- the full stepper state (device pointers, all
  * required): omega^k, psi^k, psi^{k-1}, R^{k-1}, R^{k-2} and the step index k.  Setting the
- * state lets a caller (e.g. a checkpoint or a parity test) resume bit-exactly.  For
- * DG_MIXED the R history is stored in float32 and is converted on get/set.
+ * state lets a caller (e.g. a checkpoint or a parity test) resume bit-exactly.
  */
 int dg_sim_get_state(dg_sim* s, long long* step, double* omega, double* psi, double* psi_prev,
                      double* R1, double* R2, void* stream);

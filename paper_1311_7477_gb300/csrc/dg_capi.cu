@@ -176,6 +176,34 @@ int alloc_ws_mixed(Workspace& w) {
   return DG_OK;
 }
 
+// ---- fixed-point tables (dg_fixed.cuh) ----------------------------------------------------
+
+fx fx_coef(double c, int k) { return fx_split(llrint(std::ldexp(c, k))); }
+
+// The smallest e with v < 2^e, with a little room for the rounding of the coefficients.
+int exp_above(double v) {
+  int e = 0;
+  std::frexp(v * (1.0 + 1e-6), &e);
+  return e;
+}
+
+template <int N>
+FxRhs<N> make_fx_rhs(const RefTables& t, double hx, double hy, double tau) {
+  FxRhs<N> F{};
+  double big = 0.0;
+  for (int j = 0; j < N; ++j) big = std::max(big, 1.0 / t.w[j]);
+  F.ei = exp_above(big);
+  for (int k = 0; k < N * N; ++k) F.isw[k] = fx_coef(1.0 / std::sqrt(t.w[k / N] * t.w[k % N]), 60 - F.ei);
+  F.cj = 1.0 / (hx * hy);
+  F.cp = 2.0 / std::sqrt(hx * hy);
+  F.clx = 1.0 / (hx * hx);
+  F.cly = 1.0 / (hy * hy);
+  auto mid = [](double v) { return v > 1e-80 && v < 1e80; };
+  F.ok = mid(F.cj) && mid(F.cp) && mid(F.cj * F.cp);
+  F.lap_ok = tau == 0.0 && mid(F.clx) && mid(F.cly);
+  return F;
+}
+
 // Gershgorin bound on the largest eigenvalue of the CG operator Ahat = I (x) kx + ky (x) I:
 // the largest row sum of |kx| plus that of |ky| (a row of a 1D operator couples the cell's own
 // nodes through M and the neighbours' face traces through a r^T and d s^T).
@@ -215,8 +243,8 @@ template <int N>
 void build_ops(dg_grid* g) {
   new (g->ops.d) Ops2D<double, N>(make_ops<double, N>(g->rt, g->hx, g->hy));
   new (g->ops.f) Ops2D<float, N>(make_ops<float, N>(g->rt, g->hx, g->hy));
+  new (g->ops.x) FxRhs<N>(make_fx_rhs<N>(g->rt, g->hx, g->hy, g->tau));
   const Ops2D<df, N> x = make_ops<df, N>(g->rt, g->hx, g->hy);
-  new (g->ops.x) Ops2D<df, N>(x);
   new (g->ops.k) OpsK<df, N>(OpsK<df, N>{x.kx, x.ky});
   const Ops2D<double, N>& Od = *reinterpret_cast<const Ops2D<double, N>*>(g->ops.d);
   g->precise_auto = precise_apply_needed<N>(Od, g->Lx, g->Ly, g->bc) ? 2 : 0;
@@ -669,13 +697,13 @@ int dg_bracket(dg_grid* g, const double* psi, const double* omega, double* J, vo
   if (!g || !psi || !omega || !J) return fail(DG_ERR_ARG, "NULL argument");
   if (!aligned8(psi) || !aligned8(omega) || !aligned8(J)) return fail(DG_ERR_ARG, "misaligned pointer");
   if (J == psi || J == omega) return fail(DG_ERR_ARG, "J must not alias psi or omega");
-  RhsArgs<double> A{};
+  RhsArgs A{};
   A.psi = psi;
   A.omega_in = omega;
   A.omega_base = omega;
   A.omega_out = J;
   A.bracket_only = 1;
-  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<double, decltype(nc)::value>(g, A, as_stream(stream)); });
+  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<decltype(nc)::value>(g, A, as_stream(stream)); });
 }
 
 int dg_bracket_parts(dg_grid* g, const double* psi, const double* omega, double* J, int parts, void* stream) {
@@ -683,27 +711,27 @@ int dg_bracket_parts(dg_grid* g, const double* psi, const double* omega, double*
   if (parts < 1 || parts > 7) return fail(DG_ERR_ARG, "parts must be a non-empty subset of {1, 2, 4}");
   if (!aligned8(psi) || !aligned8(omega) || !aligned8(J)) return fail(DG_ERR_ARG, "misaligned pointer");
   if (J == psi || J == omega) return fail(DG_ERR_ARG, "J must not alias psi or omega");
-  RhsArgs<double> A{};
+  RhsArgs A{};
   A.psi = psi;
   A.omega_in = omega;
   A.omega_base = omega;
   A.omega_out = J;
   A.bracket_only = 1;
   A.parts = parts;
-  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<double, decltype(nc)::value>(g, A, as_stream(stream)); });
+  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<decltype(nc)::value>(g, A, as_stream(stream)); });
 }
 
 int dg_bracket_mixed(dg_grid* g, const double* psi, const double* omega, double* J, void* stream) {
   if (!g || !psi || !omega || !J) return fail(DG_ERR_ARG, "NULL argument");
   if (!aligned8(psi) || !aligned8(omega) || !aligned8(J)) return fail(DG_ERR_ARG, "misaligned pointer");
   if (J == psi || J == omega) return fail(DG_ERR_ARG, "J must not alias psi or omega");
-  RhsArgs<df> A{};
+  RhsArgs A{};
   A.psi = psi;
   A.omega_in = omega;
   A.omega_base = omega;
   A.omega_out = J;
   A.bracket_only = 1;
-  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<df, decltype(nc)::value>(g, A, as_stream(stream)); });
+  return dispatch_n(g->n, [&](auto nc) { return launch_rhs<decltype(nc)::value>(g, A, as_stream(stream)); });
 }
 
 int dg_laplace_apply(dg_grid* g, const double* x, double* y, int mode, void* stream) {
@@ -863,37 +891,27 @@ int sim_solve(dg_sim* s, const double* omega, const double* xa, double ca, const
 }
 
 // R = -J(psi, omega_in) + D Delta_h omega_in;  omega_out = omega_base + dt (c_new R + sum c_m hist_m).
-// R and the history are float64; the RHS is evaluated in float64 or, for DG_MIXED, in
-// double-float arithmetic on the float32 pipe.
-template <typename T>
-int sim_rhs_t(dg_sim* s, const double* psi, const double* om_in, const double* om_base, double* om_out, void* R_out,
-              double c_new, int nhist, void* const* hist, const double* c_hist, cudaStream_t st) {
-  RhsArgs<T> A{};
+int sim_rhs(dg_sim* s, const double* psi, const double* om_in, const double* om_base, double* om_out, double* R_out,
+            double c_new, int nhist, double* const* hist, const double* c_hist, cudaStream_t st) {
+  int rc;
+  if (s->timing && (rc = record_event(s->ev_rhs, s->n_ev_rhs, st))) return rc;
+  RhsArgs A{};
   A.psi = psi;
   A.omega_in = om_in;
   A.omega_base = om_base;
   A.omega_out = om_out;
-  A.R_out = static_cast<hist_t<T>*>(R_out);
+  A.R_out = R_out;
   A.c_new = c_new;
   A.nhist = nhist;
   for (int m = 0; m < nhist; ++m) {
-    A.hist[m] = static_cast<const hist_t<T>*>(hist[m]);
+    A.hist[m] = hist[m];
     A.c_hist[m] = c_hist[m];
   }
   A.dt = s->dt;
   A.visc = s->D;
   A.psi_scaled = 1;
   A.parts = s->parts;
-  return dispatch_n(s->g->n, [&](auto nc) { return launch_rhs<T, decltype(nc)::value>(s->g, A, st); });
-}
-
-int sim_rhs(dg_sim* s, const double* psi, const double* om_in, const double* om_base, double* om_out, void* R_out,
-            double c_new, int nhist, void* const* hist, const double* c_hist, cudaStream_t st) {
-  int rc;
-  if (s->timing && (rc = record_event(s->ev_rhs, s->n_ev_rhs, st))) return rc;
-  rc = (s->precision == DG_MIXED)
-           ? sim_rhs_t<df>(s, psi, om_in, om_base, om_out, R_out, c_new, nhist, hist, c_hist, st)
-           : sim_rhs_t<double>(s, psi, om_in, om_base, om_out, R_out, c_new, nhist, hist, c_hist, st);
+  rc = dispatch_n(s->g->n, [&](auto nc) { return launch_rhs<decltype(nc)::value>(s->g, A, st); });
   if (rc) return rc;
   if (s->timing && (rc = record_event(s->ev_rhs, s->n_ev_rhs, st))) return rc;
   s->launches += 1;
@@ -933,7 +951,7 @@ int sim_solve_slots(dg_sim* s, const double* omega, int a, double ca, int b, dou
 int sim_rk4_step(dg_sim* s, cudaStream_t st) {
   const double* w0 = s->omega[s->oc];
   double* w1 = s->omega[s->oc ^ 1];
-  void* k1 = s->R[s->rfree];
+  double* k1 = s->R[s->rfree];
   const int sA = s->p2, sB = s->p1;
   double* PA = s->psi[sA];
   double* PB = s->psi[sB];
@@ -945,7 +963,7 @@ int sim_rk4_step(dg_sim* s, cudaStream_t st) {
   if ((rc = sim_solve_slots(s, s->stB, sA, 1.0, -1, 0.0, sB, st))) return rc;
   if ((rc = sim_rhs(s, PB, s->stB, w0, s->stA, s->k3, 1.0, 0, nullptr, nullptr, st))) return rc;
   if ((rc = sim_solve_slots(s, s->stA, sB, 1.0, -1, 0.0, sA, st))) return rc;
-  void* const hist[3] = {k1, s->k2, s->k3};
+  double* const hist[3] = {k1, s->k2, s->k3};
   const double ch[3] = {1.0 / 6.0, 2.0 / 6.0, 2.0 / 6.0};
   if ((rc = sim_rhs(s, PA, s->stA, w0, w1, nullptr, 1.0 / 6.0, 3, hist, ch, st))) return rc;
   if ((rc = sim_solve_slots(s, w1, sA, 1.0, -1, 0.0, sB, st))) return rc;
@@ -963,8 +981,8 @@ int sim_rk4_step(dg_sim* s, cudaStream_t st) {
 int sim_ab3_step(dg_sim* s, cudaStream_t st) {
   const double* w0 = s->omega[s->oc];
   double* w1 = s->omega[s->oc ^ 1];
-  void* Rk = s->R[s->rfree];
-  void* const hist[3] = {s->R[s->r1], s->R[s->r2], s->R[s->r3]};
+  double* Rk = s->R[s->rfree];
+  double* const hist[3] = {s->R[s->r1], s->R[s->r2], s->R[s->r3]};
   const int K = s->K;
   const double ch[3] = {kAB[K][1], kAB[K][2], kAB[K][3]};
   int rc;
@@ -1590,7 +1608,7 @@ BatchSim make_batch_sim(const dg_batch* bt, dg_sim* s) {
   batch_geoms(bt, g, &b.Gr, &b.Gc);
   b.ops_d = g->d_opsd;
   b.ops_f = g->d_opsf;
-  b.ops_df = g->d_opsx;
+  b.ops_rhs = g->d_opsx;
   b.ops_k = g->d_opsk;
   b.precise_apply = g->precise_apply;
   b.keep_mean = g->bc;
@@ -1647,7 +1665,7 @@ size_t batch_smem_for(const dg_batch* b, const dg_sim* s) {
   size_t out = 0;
   dispatch_n(g->n, [&](auto nc) {
     constexpr int N = decltype(nc)::value;
-    const size_t rhs = rhs_smem_values<double, N>(Gr.TY, Gr.TX) * sizeof(double);  // double or double-float
+    const size_t rhs = rhs_smem_bytes<N>(Gr.TY, Gr.TX);
     const size_t sol = s->precision == DG_FP64 ? cg_smem_bytes<double, N>(Gc.TY, Gc.TX, Lmax, g->precond, pow2_grid(g))
                                                : mixed_smem_bytes<N>(Gc.TY, Gc.TX, Lmax, g->precond, pow2_grid(g));
     out = batch_ops_bytes<N>() + std::max(rhs, sol);

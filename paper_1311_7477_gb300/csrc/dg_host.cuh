@@ -45,11 +45,11 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 inline bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
 
-// Host copies of the device operator tables for one n, in float64 and float32.
+// Host copies of the device operator tables for one n.
 struct OpsHost {
   alignas(16) unsigned char d[sizeof(Ops2D<double, kMaxN>)];
   alignas(16) unsigned char f[sizeof(Ops2D<float, kMaxN>)];
-  alignas(16) unsigned char x[sizeof(Ops2D<df, kMaxN>)];  // double-float (RHS of DG_MIXED)
+  alignas(16) unsigned char x[sizeof(FxRhs<kMaxN>)];      // fixed point (right-hand side)
   alignas(16) unsigned char k[sizeof(OpsK<df, kMaxN>)];   // double-float CG operator
 };
 
@@ -68,7 +68,7 @@ NodeWeights<N> make_weights(const RefTables& t, double hx, double hy) {
 
 // Built-in tiles (cells per block, TY x TX) for the RHS kernel and the CG kernel.
 inline void default_tiles(int n, int& rty, int& rtx, int& cty, int& ctx) {
-  static const int R[6][2] = {{0, 0}, {16, 16}, {8, 16}, {8, 8}, {4, 8}, {4, 8}};
+  static const int R[6][2] = {{0, 0}, {16, 16}, {16, 16}, {8, 16}, {8, 8}, {8, 8}};
   static const int Cg[6][2] = {{0, 0}, {16, 16}, {16, 16}, {8, 16}, {8, 8}, {8, 8}};
   rty = R[n][0];
   rtx = R[n][1];
@@ -93,11 +93,9 @@ inline void fit_tile(int Nx, int Ny, int sms, int& ty, int& tx) {
 
 inline void choose_tiles(int n, int Nx, int Ny, int sms, int& rty, int& rtx, int& cty, int& ctx) {
   default_tiles(n, rty, rtx, cty, ctx);
-  // a single simulation's RHS kernel at n = 5 is faster on 8 x 8 tiles (1024^2 cells:
-  // 5.5 against 6.6 ms per bracket), whose ~200 KB of shared memory a batch, sizing its
-  // kernel for every member, would pay in resident blocks: batches keep 4 x 8
-  if (n == 5) rty = 8;
-  fit_tile(Nx, Ny, sms, rty, rtx);
+  // two or more RHS blocks share an SM, so the RHS tiles shrink until there are two per SM
+  // (100^2 cells: n = 4 16.9 us on 325 tiles of 4 x 8, 19.1 on 169 of 8 x 8; n = 5 23.6 and 27.2)
+  fit_tile(Nx, Ny, 2 * sms, rty, rtx);
   fit_tile(Nx, Ny, sms, cty, ctx);
 }
 
@@ -165,7 +163,7 @@ struct dg_grid {
   PcTables pc;
   void* d_opsd = nullptr;  // device copies of the operator tables (batched kernel)
   void* d_opsf = nullptr;
-  void* d_opsx = nullptr;  // Ops2D<df, n>
+  void* d_opsx = nullptr;  // FxRhs<n>
   void* d_opsk = nullptr;  // OpsK<df, n>
   // a float32 evaluation of the CG operator is too inexact on the smoothest modes of this grid
   // (see precise_apply_needed): mixed solves apply it in double-float
@@ -191,12 +189,12 @@ struct dg_sim {
   // initial residual b - Ahat (2 psi^k - psi^{k-1}) needs no operator application
   double* apsi[3] = {nullptr, nullptr, nullptr};
   bool apsi_ok[3] = {false, false, false};
-  void* R[4];      // history ring: float64 (DG_FP64) or float32 (DG_MIXED)
+  double* R[4];    // history ring
   int r1, r2, r3, rfree;  // R^{k-1}, R^{k-2}, R^{k-3}, free slot
   int K = 3;              // steps of the Adams-Bashforth method (1..4)
   int parts = 0;          // bracket parts (0: J of Eq. J; 1: J++ alone, the naive bracket)
   double *stA, *stB;  // RK stage vorticities
-  void *k2, *k3;      // RK stage slopes (same type as R)
+  double *k2, *k3;    // RK stage slopes
   double tol_in;      // inner relative tolerance of the float32 sweeps (DG_MIXED)
   int max_sweeps;
   Workspace ws;
@@ -226,8 +224,12 @@ inline Geom geom_of(const dg_grid* g, int TY, int TX) {
 template <typename T, int N>
 const Ops2D<T, N>& ops_of(const dg_grid* g) {
   if constexpr (std::is_same<T, double>::value) return *reinterpret_cast<const Ops2D<T, N>*>(g->ops.d);
-  else if constexpr (std::is_same<T, float>::value) return *reinterpret_cast<const Ops2D<T, N>*>(g->ops.f);
-  else return *reinterpret_cast<const Ops2D<T, N>*>(g->ops.x);
+  else return *reinterpret_cast<const Ops2D<T, N>*>(g->ops.f);
+}
+
+template <int N>
+const FxRhs<N>& fxrhs_of(const dg_grid* g) {
+  return *reinterpret_cast<const FxRhs<N>*>(g->ops.x);
 }
 
 template <int N>
@@ -333,8 +335,8 @@ inline Geom solve_geom(const dg_grid* g, bool allow_cluster, bool* cluster) {
 inline int co_resident_cap(const dg_grid* g) { return std::max(64, 8 * g->num_sms); }
 
 // ---- per-n kernel launchers (dg_launch.cuh; instantiated in dg_inst_n<N>.cu) -------------
-template <typename T, int N>
-int launch_rhs(const dg_grid* g, const RhsArgs<T>& A, cudaStream_t st);
+template <int N>
+int launch_rhs(const dg_grid* g, const RhsArgs& A, cudaStream_t st);
 template <typename T, int N>
 int launch_apply(const dg_grid* g, const double* x, double* y, int mode, cudaStream_t st);
 template <typename T, int N, typename TP = T>

@@ -1,7 +1,8 @@
 // The hot-path kernels, templated on the arithmetic type T (double or float) and the
 // number of nodes per cell and dimension N (1..5).
 //
-//   rhs_kernel       bracket J(psi, omega) (Eq. J) + viscous term + multistep update, fused
+//   rhs_kernel       bracket J(psi, omega) (Eq. J) + viscous term + multistep update, fused, in
+//                    fixed point on the integer pipe
 //   apply_kernel     the LDG operator A or Delta_h on a field
 //   cg_kernel        persistent cooperative conjugate-gradient Poisson solve (Sec. 6)
 //   mixed_cg_kernel  float64 residual / float32 inner CG iterative refinement
@@ -12,17 +13,22 @@
 
 #include "dg_device.cuh"
 #include "dg_df.cuh"
+#include "dg_fixed_tables.cuh"
 
 namespace dgk {
 
 constexpr int kThreads = 256;
-// Threads of a standalone RHS block: its tile's staging (up to about 190 KB at n = 5) leaves
-// room for one or two blocks per SM, so the block itself must carry the SM's warps (measured on
-// the 1024^2, n = 5 step: 6.56 / 5.47 / 5.07 ms per RHS with 256 / 512 / 1024 threads; on
-// 512^2, n = 4: 1.01 / 0.88 / 1.12 ms).
+// Threads of a standalone RHS block and the blocks per SM its registers are sized for (two tiles of
+// 100 KB at n = 5, three of 68 KB at n = 4 fill an SM's shared memory; measured on 1000^2 cells:
+// n = 5 1223 us with 320 threads, 1286 / 1282 with 416 / 512; n = 4 695 us with 256 threads and three
+// blocks, 823 with 320 / 352 and two).
 template <int N>
 __host__ __device__ constexpr int rhs_threads() {
-  return N == 5 ? 1024 : 512;
+  return N == 5 ? 320 : 256;
+}
+template <int N>
+__host__ __device__ constexpr int rhs_blocks() {
+  return N == 5 ? 2 : 3;
 }
 
 // Copies an operator table (a kernel parameter or a global array) to shared memory: the
@@ -45,24 +51,7 @@ __host__ __device__ constexpr size_t table_bytes() {
 
 
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ df mul_rn(df a, df b) { return a * b; }
-__device__ __forceinline__ df sub_rn(df a, df b) { return a - b; }
-
-// Storage type of the right-hand-side history for an RHS evaluated in T: float64 for the
-// float64 and the double-float bracket (a double-float value converts to float64 exactly).
-template <typename T>
-struct HistType {
-  using type = double;
-};
-template <>
-struct HistType<float> {
-  using type = float;
-};
-template <typename T>
-using hist_t = typename HistType<T>::type;
 
 // a*b - c*d with both products rounded separately (never contracted into an FMA), so that
 // the bracket's antisymmetry J(f, g) = -J(g, f) and J(f, f) = 0 hold bitwise.
@@ -79,14 +68,13 @@ __device__ __forceinline__ T prod_diff(T a, T b, T c, T d) {
 // included: the second derivatives of J+x and Jx+ reach the diagonal neighbours) are staged
 // in shared memory, all intermediate products stay there.
 // =========================================================================================
-template <typename T>
 struct RhsArgs {
   const double* psi;        // stream function; times sqrt(W) if psi_scaled
   const double* omega_in;   // vorticity at which R is evaluated (halo reads)
   const double* omega_base; // omega^k of the update (own nodes only; may alias omega_out)
   double* omega_out;        // updated vorticity, or J in bracket-only mode
-  hist_t<T>* R_out;         // fresh R (may alias one hist buffer); may be null
-  const hist_t<T>* hist[3];
+  double* R_out;            // fresh R (may alias one hist buffer); may be null
+  const double* hist[3];
   double c_new;
   double c_hist[3];
   int nhist;
@@ -102,14 +90,13 @@ __host__ __device__ constexpr size_t rhs_smem_values(int TY, int TX) {
   return (size_t)(TY + 2) * (TX + 2) * (7 * (N * N + 1) + 12 * N);
 }
 
-// One tile of the right-hand side (smem: rhs_smem_values<T, N>(G.TY, G.TX) values of T).
+// One box of the right-hand side in float64 (smem: rhs_smem_values<double, N>(G.TY, G.TX) values).
 template <typename T, int N>
-__device__ __forceinline__ void rhs_tile(const Ops2D<T, N>& C, const Geom& G, const RhsArgs<T>& A, int tile,
-                                         unsigned char* smem_raw) {
+__device__ __forceinline__ void rhs_box_float(const Ops2D<T, N>& C, const Geom& G, const RhsArgs& A, const TileBox& B,
+                                              unsigned char* smem_raw) {
   constexpr int NN = N * N;
   constexpr int CS = NN + 1;  // padded cell stride in shared memory
   T* sm = reinterpret_cast<T*>(smem_raw);
-  const TileBox B = make_box(G, tile);
   const int boxc = (G.TY + 2) * (G.TX + 2);
   T* sPsi = sm;
   T* sOm = sPsi + boxc * CS;
@@ -245,17 +232,326 @@ __device__ __forceinline__ void rhs_tile(const Ops2D<T, N>& C, const Geom& G, co
     }
     double incr = A.c_new * double(R);
     for (int m = 0; m < A.nhist; ++m) incr = fma(A.c_hist[m], double(A.hist[m][g]), incr);
-    if (A.R_out) A.R_out[g] = hist_t<T>(R);
+    if (A.R_out) A.R_out[g] = double(R);
     A.omega_out[g] = fma(A.dt, incr, A.omega_base[g]);
   }
   __syncthreads();
 }
 
-template <typename T, int N>
-__global__ void __launch_bounds__(rhs_threads<N>()) rhs_kernel(const __grid_constant__ Ops2D<T, N> C, const Geom G,
-                                                      const __grid_constant__ RhsArgs<T> A) {
+// What the fixed-point right-hand side (dg_fixed.cuh) takes from the grid.  The derivative and the
+// Laplacian are tables of n on the reference cell, so every term of J carries the same factor
+// 1 / (hx hy), applied once to the finished sum; likewise 1 / sqrt(W) is 1 / sqrt(w_a w_b) times
+// one factor.
+template <int N>
+struct FxRhs {
+  fx isw[N * N];   // 1 / sqrt(w_a w_b) = 2^(ei - 60) isw
+  int ei;
+  int ok;          // the factors lie in the range the fixed-point path covers
+  int lap_ok;      // ... and the Laplacian's (its table holds for the penalty tau = 0)
+  double cj, cp;   // 1 / (hx hy), 2 / sqrt(hx hy)
+  double clx, cly; // 1 / hx^2, 1 / hy^2
+};
+
+// Cell stride of the fixed-point staging: odd, so that the lanes of a warp, which read the same
+// node of consecutive cells, fall on distinct pairs of banks.
+template <int N>
+__host__ __device__ constexpr int fx_cell() {
+  return (N * N) | 1;
+}
+
+// Shared memory of one right-hand-side tile: five arrays over the box, or the float64 fallback on
+// single cells, whichever is larger.
+template <int N>
+__host__ __device__ constexpr size_t rhs_smem_bytes(int TY, int TX) {
+  const size_t a = (size_t)(TY + 2) * (TX + 2) * 5 * fx_cell<N>() * 8;
+  const size_t b = rhs_smem_values<double, N>(1, 1) * 8;
+  return a > b ? a : b;
+}
+
+// The tile in float64: for tiles whose values the fixed-point scale cannot hold (infinities, NaN,
+// products near the ends of the float64 range).  It needs more shared memory per cell than the
+// fixed-point tile, so it runs on sub-tiles that fit.
+template <int N>
+__device__ __noinline__ void rhs_tile_float(const Ops2D<double, N>& C, const Geom& G, const RhsArgs& A, int tile,
+                                            unsigned char* smem) {
+  const TileBox B = make_box(G, tile);
+  const size_t avail = rhs_smem_bytes<N>(G.TY, G.TX);
+  Geom S = G;
+  while (rhs_smem_values<double, N>(S.TY, S.TX) * 8 > avail) {
+    if (S.TX >= S.TY)
+      S.TX = (S.TX + 1) / 2;
+    else
+      S.TY = (S.TY + 1) / 2;
+  }
+  for (int y = 0; y < B.TYe; y += S.TY)
+    for (int x = 0; x < B.TXe; x += S.TX) {
+      TileBox b;
+      b.ty0 = B.ty0 + y;
+      b.tx0 = B.tx0 + x;
+      b.TYe = min(S.TY, B.TYe - y);
+      b.TXe = min(S.TX, B.TXe - x);
+      b.BW = S.TX + 2;
+      b.mTXe = magic_of(b.TXe);
+      rhs_box_float<double, N>(C, S, A, b, smem);
+    }
+}
+
+// One tile of the right-hand side in fixed point (smem: rhs_smem_bytes<N>(G.TY, G.TX)).
+//
+// What bounds it: the integer pipe (60% busy with the multiply-adds on 512^2 cells, n = 5) and the
+// synchronisations between phases; the float64 pipe only does the update (8%).  Per bracket, before
+// (the same phases in float64) and now: 1000^2 cells, n = 4 2396 and 695 us; 1000^2, n = 5 4.8 ms and
+// 1223 us; 100^2, n = 4 38.9 and 16.4 us; 501 x 373, n = 3 158 (in double-float) and 72 us.  A thread computes a whole line of a cell (its n nodes along x or y):
+// it reads the n values of the line and the neighbours' once, evaluates their face traces itself
+// (as many multiply-adds as evaluating each trace once and storing it, one phase and 12 n arrays
+// less), and takes its coefficients from the constant bank.  Phases (a block synchronisation after
+// each):
+//   stage f = psi and g = omega with their halo ring, find the tile's largest magnitudes,
+//   convert to fixed point;
+//   x-lines of rows [-1, TYe]:  f_x, g_x, h2 = f_x g - f g_x;
+//   y-lines of columns [-1, TXe]:  f_y, g_y, J++ = f_x g_y - f_y g_x, h1 = f g_y - f_y g;
+//   x-lines of the tile: D_x h1 (over f); y-lines: J++ + D_y h2;   [viscous: lx g, ly g]
+//   nodes: J, the update.
+// J(f, f) = 0 and J(f, g) = -J(g, f) hold bitwise: equal and opposite products cancel exactly in
+// the accumulators, and every rounding is odd.
+//
+// Gen: Dirichlet boundaries or a part of J only.  The common case (periodic, all of J) is compiled
+// without either: the selects they put around every trace and product took 40% of its time.
+template <int N, bool Gen>
+__device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, N>& C, const Geom& G,
+                                         const RhsArgs& A, int tile, unsigned char* smem) {
+  constexpr int NN = N * N;
+  constexpr int CS = fx_cell<N>();
+  __shared__ unsigned s_mag[2][32];
+  __shared__ fx s_isw[NN];
+  constexpr FxTable<N> D = fx_deriv<N>();
+  constexpr FxTable<N> Lp = fx_lap<N>();
+  const TileBox B = make_box(G, tile);
+  const int BW = B.BW;
+  const int boxc = (G.TY + 2) * BW;
+  fx* sF = reinterpret_cast<fx*>(smem);
+  fx* sG = sF + boxc * CS;
+  fx* sA = sG + boxc * CS;  // f_x, then J++ (+ D_y h2)
+  fx* sB = sA + boxc * CS;  // g_x, then h1, then lx g
+  fx* sC = sB + boxc * CS;  // h2, then ly g
+
+  // stage the two fields and their largest magnitudes
+  {
+    double* rF = reinterpret_cast<double*>(sF);
+    double* rG = reinterpret_cast<double*>(sG);
+    unsigned mf = 0, mg = 0;
+    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+    const int rowlen = BWe * NN, total = BHe * rowlen;
+    const unsigned mrow = magic_of(rowlen);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int br = quot(i, mrow);
+      const int j = i - br * rowlen;
+      const int bc = j / NN, k = j - bc * NN;
+      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+      const int o = (br * BW + bc) * CS + k;
+      if (Gen && G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)) {
+        rF[o] = 0.0;
+        rG[o] = 0.0;
+        continue;
+      }
+      const size_t g = ((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k;
+      const double f = A.psi[g], w = A.omega_in[g];
+      rF[o] = f;
+      rG[o] = w;
+      mf = max(mf, fx_mag(f));
+      mg = max(mg, fx_mag(w));
+    }
+    mf = __reduce_max_sync(0xffffffffu, mf);
+    mg = __reduce_max_sync(0xffffffffu, mg);
+    if (A.psi_scaled && threadIdx.x < NN) s_isw[threadIdx.x] = F.isw[threadIdx.x];
+    if ((threadIdx.x & 31) == 0) {
+      s_mag[0][threadIdx.x >> 5] = mf;
+      s_mag[1][threadIdx.x >> 5] = mg;
+    }
+  }
+  __syncthreads();
+  const int nw = int(blockDim.x >> 5), lane = threadIdx.x & 31;
+  const unsigned mf = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[0][lane] : 0u);
+  const unsigned mg = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[1][lane] : 0u);
+  const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
+  // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any)
+  const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
+  const int uj = uf + ug + 2 * D.e + 60, ul = ug + Lp.e;
+  const bool viscous = A.visc != 0.0 && !A.bracket_only;
+  // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
+  const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.lap_ok && abs(ul) <= 600));
+  if (!covered) {
+    __syncthreads();  // the staging is reused
+    rhs_tile_float<N>(C, G, A, tile, smem);
+    return;
+  }
+  for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
+    const fx f = sF[i], w = sG[i];  // raw bits: {low, high} words
+    long long x = fx_from_bits(unsigned(f.l), unsigned(f.h), ef);
+    if (A.psi_scaled) {
+      const int k = i % CS;
+      FxAcc s;
+      fx_mac(s, s_isw[k < NN ? k : 0], fx_split(x));
+      x = fx_round(s);
+    }
+    sF[i] = fx_split(x);
+    sG[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), eg));
+  }
+  __syncthreads();
+
+  // Which parts enter (Eq. J): J = s (c0 J++ + J+x + Jx+) with J+x = D_x(f g_y) - D_y(f g_x),
+  // Jx+ = D_y(f_x g) - D_x(f_y g).
+  const int parts = A.parts ? A.parts : 7;
+  const int mpp = !Gen || (parts & 1) ? -1 : 0, mpx = !Gen || (parts & 2) ? -1 : 0, mxp = !Gen || (parts & 4) ? -1 : 0;
+  const bool bc = Gen && G.bc;
+
+  // x-lines of rows [-1, TYe]
+  {
+    const int nc = (B.TYe + 2) * B.TXe;
+    const unsigned mnc = magic_of(nc);
+    for (int u = threadIdx.x; u < nc * N; u += blockDim.x) {
+      const int a = quot(u, mnc), c = u - a * nc;
+      const int br = quot(c, B.mTXe), rx = c - br * B.TXe;
+      const int o = (br * BW + rx + 1) * CS + a * N;
+      fx fd[N];
+      auto keep = [&](int i, long long y) { fd[i] = fx_split(y); };
+      auto store = [&](int i, long long y) {
+        const fx gd = fx_split(y);
+        sA[o + i] = fd[i];
+        sB[o + i] = gd;
+        sC[o + i] = fx_split(fx_prod_diff(fd[i], fx_and(sG[o + i], mxp), fx_and(sF[o + i], mpx), gd));
+      };
+      if constexpr (Gen) {
+        const bool first = bc && B.tx0 + rx == 0, last = bc && B.tx0 + rx == G.Nx - 1;
+        fx_line_bounded<N>(D, sF + o, 1, CS, first, last, keep);
+        fx_line_bounded<N>(D, sG + o, 1, CS, first, last, store);
+      } else {
+        fx_line<N>(D, sF + o, 1, CS, keep);
+        fx_line<N>(D, sG + o, 1, CS, store);
+      }
+    }
+  }
+  __syncthreads();
+  // y-lines of columns [-1, TXe]
+  {
+    const int w = B.TXe + 2, nc = B.TYe * w;
+    const unsigned mnc = magic_of(nc), mw = magic_of(w);
+    for (int u = threadIdx.x; u < nc * N; u += blockDim.x) {
+      const int b = quot(u, mnc), c = u - b * nc;
+      const int ry = quot(c, mw), bc_ = c - ry * w;
+      const int o = ((ry + 1) * BW + bc_) * CS + b, dn = BW * CS;
+      const bool inner = bc_ > 0 && bc_ <= B.TXe;
+      fx fd[N];
+      auto keep = [&](int i, long long y) { fd[i] = fx_split(y); };
+      auto store = [&](int i, long long y) {
+        const fx gd = fx_split(y);
+        const int oi = o + i * N;
+        if (inner)
+          reinterpret_cast<long long*>(sA)[oi] = fx_prod_diff(fx_and(sA[oi], mpp), gd, fd[i], fx_and(sB[oi], mpp));
+        sB[oi] = fx_split(fx_prod_diff(fx_and(sF[oi], mpx), gd, fd[i], fx_and(sG[oi], mxp)));
+      };
+      if constexpr (Gen) {
+        const bool first = bc && B.ty0 + ry == 0, last = bc && B.ty0 + ry == G.Ny - 1;
+        fx_line_bounded<N>(D, sF + o, N, dn, first, last, keep);
+        fx_line_bounded<N>(D, sG + o, N, dn, first, last, store);
+      } else {
+        fx_line<N>(D, sF + o, N, dn, keep);
+        fx_line<N>(D, sG + o, N, dn, store);
+      }
+    }
+  }
+  __syncthreads();
+  // D_x h1 over f, J++ + D_y h2
+  const int nc = B.TYe * B.TXe;
+  const unsigned mnc = magic_of(nc);
+  for (int u = threadIdx.x; u < 2 * nc * N; u += blockDim.x) {
+    const bool alongx = u < nc * N;
+    const int v = alongx ? u : u - nc * N;
+    const int ln = quot(v, mnc), c = v - ln * nc;
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const int cell = ((ry + 1) * BW + rx + 1) * CS;
+    if (alongx) {
+      const int o = cell + ln * N;
+      auto put = [&](int i, long long y) { reinterpret_cast<long long*>(sF)[o + i] = y; };
+      if constexpr (Gen)
+        fx_line_bounded<N>(D, sB + o, 1, CS, bc && B.tx0 + rx == 0, bc && B.tx0 + rx == G.Nx - 1, put);
+      else
+        fx_line<N>(D, sB + o, 1, CS, put);
+    } else {
+      const int o = cell + ln;
+      auto add = [&](int i, long long y) { reinterpret_cast<long long*>(sA)[o + i * N] += y; };
+      if constexpr (Gen)
+        fx_line_bounded<N>(D, sC + o, N, BW * CS, bc && B.ty0 + ry == 0, bc && B.ty0 + ry == G.Ny - 1, add);
+      else
+        fx_line<N>(D, sC + o, N, BW * CS, add);
+    }
+  }
+  __syncthreads();
+  if (viscous) {  // lx g over h1, ly g over h2
+    for (int u = threadIdx.x; u < 2 * nc * N; u += blockDim.x) {
+      const bool alongx = u < nc * N;
+      const int v = alongx ? u : u - nc * N;
+      const int ln = quot(v, mnc), c = v - ln * nc;
+      const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+      const int cell = ((ry + 1) * BW + rx + 1) * CS;
+      if (alongx) {
+        const int o = cell + ln * N;
+        auto put = [&](int i, long long y) { reinterpret_cast<long long*>(sB)[o + i] = y; };
+        if constexpr (Gen)
+          fx_ldg_bounded<N>(Lp, sG + o, 1, CS, bc ? B.tx0 + rx : 2, put);
+        else
+          fx_line<N>(Lp, sG + o, 1, CS, put);
+      } else {
+        const int o = cell + ln;
+        auto put = [&](int i, long long y) { reinterpret_cast<long long*>(sC)[o + i * N] = y; };
+        if constexpr (Gen)
+          fx_ldg_bounded<N>(Lp, sG + o, N, BW * CS, bc ? B.ty0 + ry : 2, put);
+        else
+          fx_line<N>(Lp, sG + o, N, BW * CS, put);
+      }
+    }
+    __syncthreads();
+  }
+  // nodes: J and the update
+  const double cJ = (parts == 7 ? 1.0 / 3.0 : 1.0) * F.cj * (A.psi_scaled ? F.cp : 1.0) * fx_pow2(uj);
+  const double cLx = A.visc * F.clx * fx_pow2(ul), cLy = A.visc * F.cly * fx_pow2(ul);
+  const bool square = F.clx == F.cly;
+  const int nin = nc * NN;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < nin; i += blockDim.x) {
+    const int c = i / NN, k = i - (i / NN) * NN;
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const int o = ((ry + 1) * BW + rx + 1) * CS + k;
+    const size_t g = ((size_t)(B.ty0 + ry) * G.Nx + (B.tx0 + rx)) * NN + k;
+    const double J =
+        fx_to_double(reinterpret_cast<const long long*>(sA)[o] + reinterpret_cast<const long long*>(sF)[o]) * cJ;
+    if (A.bracket_only) {
+      A.omega_out[g] = J;
+      continue;
+    }
+    double R = -J;
+    if (viscous) {  // + D Delta_h omega, since -Delta_h = lx + ly
+      const long long lx = reinterpret_cast<const long long*>(sB)[o], ly = reinterpret_cast<const long long*>(sC)[o];
+      if (square)
+        R = fma(-cLx, fx_to_double(lx + ly), R);
+      else
+        R = fma(-cLx, fx_to_double(lx), fma(-cLy, fx_to_double(ly), R));
+    }
+    double incr = A.c_new * R;
+    for (int m = 0; m < A.nhist; ++m) incr = fma(A.c_hist[m], A.hist[m][g], incr);
+    if (A.R_out) A.R_out[g] = R;
+    A.omega_out[g] = fma(A.dt, incr, A.omega_base[g]);
+  }
+  __syncthreads();
+}
+
+template <int N, bool Gen>
+__global__ void __launch_bounds__(rhs_threads<N>(), rhs_blocks<N>()) rhs_kernel(const __grid_constant__ FxRhs<N> F,
+                                                               const __grid_constant__ Ops2D<double, N> C, const Geom G,
+                                                               const __grid_constant__ RhsArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rhs_tile<T, N>(stage_table(C, smem_raw), G, A, blockIdx.x, smem_raw + table_bytes<Ops2D<T, N>>());
+  rhs_tile<N, Gen>(F, C, G, A, blockIdx.x, smem_raw);
 }
 
 // =========================================================================================
@@ -1719,19 +2015,19 @@ __global__ void __launch_bounds__(kThreads, MinB) mixed_cg_kernel(const __grid_c
 // simulations queued on it, one after the other.  Groups run concurrently.
 // =========================================================================================
 struct BatchSim {
-  int n, precision, precond;       // precision: 0 float64, 1 mixed (double-float RHS), 2 mixed (float64 RHS)
+  int n, precision, precond;       // precision: 0 float64, else mixed
   int precise_apply;               // mixed: the inner solve applies Ahat in double-float
   int keep_mean;                   // homogeneous Dirichlet grid: no mean removed from omega
   Geom Gr, Gc;                     // tiles of the RHS and of the solve
   const void* ops_d;               // device copy of Ops2D<double, n>
   const void* ops_f;               // device copy of Ops2D<float, n>
-  const void* ops_df;              // device copy of Ops2D<df, n> (double-float RHS)
+  const void* ops_rhs;             // device copy of FxRhs<n> (fixed-point RHS)
   const void* ops_k;               // device copy of OpsK<df, n> (double-float CG operator)
   double* omega[2];
   double* psi[3];                  // sqrt(W) psi
   double* apsi[3];                 // Ahat psi of each slot, valid where apsi_ok (see dg_sim)
   int apsi_ok[3];
-  void* R[4];                      // right-hand-side history (float64)
+  double* R[4];                    // right-hand-side history
   int oc, p0, p1, p2, r1, r2, r3, rfree;  // ring indices, advanced by the kernel
   long long step;
   long long limit;                 // no batched step once step == limit (0: no limit)
@@ -1762,17 +2058,17 @@ struct BatchArgs {
   int* error;                // first error flag of any group
 };
 
-template <typename T, int N>
-__device__ __noinline__ void batch_rhs(const BatchSim& S, const Ops2D<T, N>& C, int oc, int p0, int r1, int r2,
-                                          int rfree, int vrank, int vsize, unsigned char* smem) {
-  RhsArgs<T> A{};
+template <int N>
+__device__ __noinline__ void batch_rhs(const BatchSim& S, const FxRhs<N>& F, int oc, int p0, int r1, int r2, int rfree,
+                                       int vrank, int vsize, unsigned char* smem) {
+  RhsArgs A{};
   A.psi = S.psi[p0];
   A.omega_in = S.omega[oc];
   A.omega_base = S.omega[oc];
   A.omega_out = S.omega[oc ^ 1];
-  A.R_out = static_cast<hist_t<T>*>(S.R[rfree]);
-  A.hist[0] = static_cast<const hist_t<T>*>(S.R[r1]);
-  A.hist[1] = static_cast<const hist_t<T>*>(S.R[r2]);
+  A.R_out = S.R[rfree];
+  A.hist[0] = S.R[r1];
+  A.hist[1] = S.R[r2];
   A.c_new = 23.0 / 12.0;
   A.c_hist[0] = -16.0 / 12.0;
   A.c_hist[1] = 5.0 / 12.0;
@@ -1781,15 +2077,19 @@ __device__ __noinline__ void batch_rhs(const BatchSim& S, const Ops2D<T, N>& C, 
   A.visc = S.D;
   A.psi_scaled = 1;
   const int nt = S.Gr.tilesX * S.Gr.tilesY;
-  for (int t = vrank; t < nt; t += vsize) rhs_tile<T, N>(C, S.Gr, A, t, smem);
+  const Ops2D<double, N>& C = *static_cast<const Ops2D<double, N>*>(S.ops_d);
+  if (S.Gr.bc)
+    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, true>(F, C, S.Gr, A, t, smem);
+  else
+    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, false>(F, C, S.Gr, A, t, smem);
 }
 
 // One AB3 step of simulation S on a group.  Returns false after a barrier timeout.
-// Shared-memory tables of a batched step: the float64 operators (the double-float RHS
-// operators during a DG_MIXED member's RHS pass: same size), float32, double-float CG operator.
+// Shared-memory tables of a batched step: the float64 operators (the fixed-point tables during
+// the RHS pass), float32, double-float CG operator.
 template <int N>
 __host__ __device__ constexpr size_t batch_ops_bytes() {
-  static_assert(sizeof(Ops2D<df, N>) == sizeof(Ops2D<double, N>), "table sizes");
+  static_assert(sizeof(FxRhs<N>) <= sizeof(Ops2D<double, N>), "table sizes");
   return table_bytes<Ops2D<double, N>>() + table_bytes<Ops2D<float, N>>() + table_bytes<OpsK<df, N>>();
 }
 
@@ -1806,13 +2106,8 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
   // this simulation's operator tables, staged in shared memory (the previous step's last
   // barrier has synchronised the block)
   unsigned char* smem = smem_all + batch_ops_bytes<N>();
-  if (S.precision == 1) {
-    const Ops2D<df, N>& Cr = stage_table(*static_cast<const Ops2D<df, N>*>(S.ops_df), smem_all);
-    batch_rhs<df, N>(S, Cr, oc, p0, r1, r2, rfree, vrank, grp.nblocks, smem);
-  } else {
-    const Ops2D<double, N>& Cr = stage_table(*static_cast<const Ops2D<double, N>*>(S.ops_d), smem_all);
-    batch_rhs<double, N>(S, Cr, oc, p0, r1, r2, rfree, vrank, grp.nblocks, smem);
-  }
+  const FxRhs<N>& Fr = stage_table(*static_cast<const FxRhs<N>*>(S.ops_rhs), smem_all);
+  batch_rhs<N>(S, Fr, oc, p0, r1, r2, rfree, vrank, grp.nblocks, smem);
   if (!grid_barrier(grp.sync, s_flag, grp.nblocks)) return false;
   // the solve's tables (the barrier has synchronised the block: the RHS table is no longer read)
   const Ops2D<double, N>& Cd = stage_table(*static_cast<const Ops2D<double, N>*>(S.ops_d), smem_all);

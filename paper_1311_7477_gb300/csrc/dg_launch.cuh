@@ -6,12 +6,14 @@
 
 namespace dgk {
 
-template <typename T, int N>
-int launch_rhs(const dg_grid* g, const RhsArgs<T>& A, cudaStream_t st) {
+template <int N>
+int launch_rhs(const dg_grid* g, const RhsArgs& A, cudaStream_t st) {
   const Geom G = geom_of(g, g->rTY, g->rTX);
-  const size_t smem = table_bytes<Ops2D<T, N>>() + rhs_smem_values<T, N>(G.TY, G.TX) * sizeof(T);
-  if (int rc = set_smem(rhs_kernel<T, N>, smem)) return rc;
-  rhs_kernel<T, N><<<G.tilesX * G.tilesY, rhs_threads<N>(), smem, st>>>(ops_of<T, N>(g), G, A);
+  const size_t smem = rhs_smem_bytes<N>(G.TY, G.TX);
+  const bool gen = G.bc || (A.parts && A.parts != 7);
+  auto kern = gen ? rhs_kernel<N, true> : rhs_kernel<N, false>;
+  if (int rc = set_smem(kern, smem)) return rc;
+  kern<<<G.tilesX * G.tilesY, rhs_threads<N>(), smem, st>>>(fxrhs_of<N>(g), ops_of<double, N>(g), G, A);
   CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
@@ -184,8 +186,7 @@ int launch_scale(const dg_grid* g, const double* x, double* y, int inverse, cuda
 // Explicit instantiation of every launcher for one n (in namespace dgk).
 #define DGK_INSTANTIATE_LAUNCHERS(N)                                                                           \
   namespace dgk {                                                                                             \
-  template int launch_rhs<double, N>(const dg_grid*, const RhsArgs<double>&, cudaStream_t);                   \
-  template int launch_rhs<df, N>(const dg_grid*, const RhsArgs<df>&, cudaStream_t);                           \
+  template int launch_rhs<N>(const dg_grid*, const RhsArgs&, cudaStream_t);                                   \
   template int launch_apply<double, N>(const dg_grid*, const double*, double*, int, cudaStream_t);            \
   template int launch_cg<double, N, double>(const dg_grid*, CgArgs<double, double>, const Workspace&,         \
                                             cudaStream_t, dg_sim*);                                           \

@@ -257,7 +257,7 @@ def dg_bracket(grid, psi, omega, J, stream=None):
 
 
 def dg_bracket_mixed(grid, psi, omega, J, stream=None):
-    """The bracket as DG_MIXED evaluates it: double-float arithmetic on the float32 pipe."""
+    """The bracket as DG_MIXED evaluates it (the same arithmetic as dg_bracket)."""
     _check(_lib.dg_bracket_mixed(grid.h, _ptr(psi), _ptr(omega), _ptr(J), _stream(stream)))
 
 

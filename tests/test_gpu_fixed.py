@@ -1,0 +1,73 @@
+"""The fixed-point right-hand side where it can go wrong: tile edges and remainders for every n,
+anisotropic cells, the parts the tables do not cover (a jump penalty), and values outside the
+fixed-point range, which the float64 tile takes.
+
+Bars: 1e-12 in relative L2 against the float64 oracle, as for the float64 evaluation: one rounding of
+2^-60 of a tile's largest value per term against the oracle's own 2^-53.  Fields are i.i.d. normal,
+so no value is more than a few bits below its tile's largest.
+"""
+import numpy as np
+import pytest
+
+from oracle.operators import Operators
+from oracle.tables import Grid as OGrid
+from tests.test_gpu_parity import bracket_scale, dev, host, rel_l2
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+# default tiles are 16 x 16 (n = 1, 2), 8 x 16 (n = 3), 8 x 8 (n = 4, 5), smaller on small grids
+SHAPES = [(33, 17, 1), (17, 35, 2), (40, 41, 3), (9, 70, 4), (41, 33, 5), (2, 3, 5)]
+
+
+@pytest.fixture(scope="module")
+def dg(native):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    return native
+
+
+@pytest.mark.parametrize("Nx,Ny,n", SHAPES)
+@pytest.mark.parametrize("bc,tau", [("periodic", 0.0), ("periodic", 0.3), ("dirichlet", 0.0)])
+def test_rhs(dg, Nx, Ny, n, bc, tau):
+    """R = -J(psi, omega) + D Delta_h omega of one Adams-Bashforth step, read back from the state."""
+    Lx, Ly, D = 1.5, 2.0, 0.05
+    g = dg.Grid(Nx, Ny, n, Lx, Ly, tau, bc=bc)
+    o = Operators(OGrid(Nx, Ny, n, Lx, Ly), tau=tau, bc=bc)
+    psi, w, z = np.random.default_rng(Nx + n).standard_normal((3, Ny, Nx, n, n))
+    s = dg.Sim(g, dev(np.zeros(g.shape)), D=D, dt=1e-6)
+    s.set_state(5, dev(w), dev(psi), dev(psi), dev(z), dev(z))
+    s.set_cg(1e-30, 10, fixed_iters=1)
+    s.step(1)
+    b = [torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(5)]
+    s.get_state(*b)
+    R = host(b[3])
+    lap = D * o.laplacian(w)
+    ref = -o.bracket(psi, w) + lap
+    assert rel_l2(R, ref, bracket_scale(o, psi, w) + np.linalg.norm(lap.ravel())) < 1e-12
+    assert rel_l2(host(b[0]), w + 1e-6 * (23 * ref - 16 * z + 5 * z) / 12) < 1e-12
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+def test_bracket_outside_the_fixed_point_range(dg, n):
+    Nx, Ny = 21, 19
+    g = dg.Grid(Nx, Ny, n)
+    o = Operators(OGrid(Nx, Ny, n))
+    f, h = np.random.default_rng(n).standard_normal((2, Ny, Nx, n, n))
+    J = torch.empty(g.shape, dtype=torch.float64, device="cuda")
+    ref = o.bracket(f, h)
+    scale = bracket_scale(o, f, h)
+    for a, b in ((1e250, 1e-80), (1e-150, 1e-150), (1e150, 1e150), (0.0, 1e200)):
+        dg.dg_bracket(g, dev(a * f), dev(b * h), J)
+        assert rel_l2(host(J) / a / b if a else host(J), ref if a else 0.0 * ref, scale) < 1e-12, (a, b)
+    # a value that is not finite spoils exactly the nodes whose stencils reach it
+    for bad in (np.nan, np.inf):
+        f2 = f.copy()
+        f2[9, 10, n // 2, 0] = bad
+        dg.dg_bracket(g, dev(f2), dev(h), J)
+        with np.errstate(invalid="ignore"):
+            want = o.bracket(f2, h)
+        got = host(J)
+        assert np.array_equal(np.isfinite(got), np.isfinite(want))
+        ok = np.isfinite(want)
+        assert rel_l2(got[ok], ref[ok], scale) < 1e-12
