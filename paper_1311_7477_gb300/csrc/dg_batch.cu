@@ -5,11 +5,10 @@ namespace dgk {
 
 __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__ BatchArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[32];
-  __shared__ double bcd;
-  __shared__ float redf[32];
-  __shared__ float bcf;
-  __shared__ int s_flag;
+  __shared__ double redd[96];
+  __shared__ float redf[96];
+  __shared__ BarrierState bs;
+  if (threadIdx.x == 0) bs = BarrierState{0, 0};
   int gi = 0;
   while (gi + 1 < A.ngroups && (int)blockIdx.x >= A.groups[gi + 1].first_block) ++gi;
   const BatchGroup grp = A.groups[gi];
@@ -19,11 +18,11 @@ __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__
     for (int j = 0; j < grp.count && ok; ++j) {
       BatchSim* S = A.sims + A.order[grp.first + j];
       switch (S->n) {
-        case 1: ok = batch_step<1>(S, grp, vrank, smem_raw, redd, &bcd, redf, &bcf, &s_flag); break;
-        case 2: ok = batch_step<2>(S, grp, vrank, smem_raw, redd, &bcd, redf, &bcf, &s_flag); break;
-        case 3: ok = batch_step<3>(S, grp, vrank, smem_raw, redd, &bcd, redf, &bcf, &s_flag); break;
-        case 4: ok = batch_step<4>(S, grp, vrank, smem_raw, redd, &bcd, redf, &bcf, &s_flag); break;
-        case 5: ok = batch_step<5>(S, grp, vrank, smem_raw, redd, &bcd, redf, &bcf, &s_flag); break;
+        case 1: ok = batch_step<1>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 2: ok = batch_step<2>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 3: ok = batch_step<3>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 4: ok = batch_step<4>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 5: ok = batch_step<5>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
         default: ok = false;
       }
     }
@@ -32,6 +31,13 @@ __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__
 }
 
 int batch_kernel_occupancy(size_t smem, int* per_sm) {
+  int dev = 0, optin = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  cudaFuncAttributes fa;
+  CUDA_TRY(cudaFuncGetAttributes(&fa, batch_kernel));
+  if (smem + fa.sharedSizeBytes > (size_t)optin)
+    return fail(DG_ERR_ARG, "batch needs %zu B of shared memory per block (max %d)", smem + fa.sharedSizeBytes, optin);
   if (int rc = set_smem(batch_kernel, smem)) return rc;
   CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, batch_kernel, kThreads, smem));
   return DG_OK;

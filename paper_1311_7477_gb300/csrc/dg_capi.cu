@@ -1680,11 +1680,6 @@ int batch_plan(dg_batch* b, int dev_sms, cudaStream_t st) {
   const int ns = (int)b->sims.size();
   size_t smem = 0;
   for (dg_sim* s : b->sims) smem = std::max(smem, batch_smem_for(b, s));
-  int optin = 0;
-  int dev = 0;
-  CUDA_TRY(cudaGetDevice(&dev));
-  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (smem > (size_t)optin) return fail(DG_ERR_ARG, "batch needs %zu B of shared memory per block (max %d)", smem, optin);
   int per_sm = 0;
   if (int rc = batch_kernel_occupancy(smem, &per_sm)) return rc;
   if (per_sm < 1) return fail(DG_ERR_CUDA, "batch kernel does not fit on an SM");

@@ -341,28 +341,20 @@ __device__ __forceinline__ T sum_partials(const T* p, int G, int stride, T* bcas
   return r;
 }
 
-// The same with the whole block: thread t adds the partials t, t + blockDim.x, ... in
-// order, then a fixed-shape block reduction.  Every block computes the bit-identical value
-// (the order depends only on G and blockDim.x); one round of loads instead of G / 32.
-template <typename T>
-__device__ __forceinline__ T sum_partials_block(const T* p, int G, int stride, T* red, T* bcast) {
-  T v = T(0);
-  for (int i = threadIdx.x; i < G; i += blockDim.x) v += __ldcg(p + (size_t)i * stride);
-  v = block_sum(v, red);
-  if (threadIdx.x == 0) *bcast = v;
-  __syncthreads();
-  const T r = *bcast;
-  __syncthreads();
-  return r;
-}
-
 // ---- grid barrier for persistent cooperative kernels -----------------------------------
 
-struct SyncState {
-  unsigned int count;
-  unsigned int gen;
-  int error;
+struct alignas(8) SyncState {
+  unsigned int count;   // arrivals since the launch, modulo 2^32
+  int error;            // read together with count (one 64-bit load)
   unsigned int ticket;  // work-unit tickets of the dynamically scheduled phases (next_unit)
+  unsigned int pad;
+};
+
+// A block's part of a grid barrier, in shared memory: {error of the last barrier, arrivals that
+// complete it}.  Start it at {0, 0} on every launch, as SyncState.
+struct BarrierState {
+  int error;
+  unsigned int target;
 };
 
 // Waits of a block at the barrier give up after this many polls (~1 s with the sleep
@@ -371,34 +363,33 @@ constexpr unsigned long long kSpinCap = 1ull << 23;
 
 // The nblk blocks of a (virtual) grid meet here: all blocks of a cooperative launch, or the
 // blocks of one group of a batched launch.  Returns false if any block raised an error.
-__device__ __forceinline__ bool grid_barrier(SyncState* s, int* s_flag, unsigned int nblk) {
+// One release-add per block on a counter that only grows, and acquire-polls of the counter itself
+// with the error word beside it: a barrier costs one trip to L2 for the add and one for the poll that sees the
+// last arrival (a counter that the last block resets before it opens a second word cost three
+// more, and the full fences around them).
+__device__ __forceinline__ bool grid_barrier(SyncState* s, BarrierState* bs, unsigned int nblk) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned int* vgen = &s->gen;
-    volatile int* verr = &s->error;
-    const unsigned int gen0 = *vgen;
-    __threadfence();
-    const unsigned int arrived = atomicAdd(&s->count, 1u) + 1u;
-    if (arrived == nblk) {
-      atomicExch(&s->count, 0u);
-      __threadfence();
-      atomicAdd(&s->gen, 1u);
-    } else {
-      unsigned long long spins = 0;
-      while (*vgen == gen0) {
-        if (*verr) break;
-        if (++spins > kSpinCap) {
-          atomicCAS(&s->error, 0, kFlagTimeout);
-          break;
-        }
-        if (spins > 4096) __nanosleep(100);  // poll tightly first: most waits are short
+    const unsigned int target = bs->target + nblk;
+    bs->target = target;
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&s->count), "r"(1u) : "memory");
+    unsigned long long spins = 0, v;
+    int err;
+    while (true) {
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(s) : "memory");
+      err = int(v >> 32);
+      if (err || int(unsigned(v) - target) >= 0) break;
+      if (++spins > kSpinCap) {
+        atomicCAS(&s->error, 0, kFlagTimeout);
+        err = kFlagTimeout;
+        break;
       }
+      if (spins > 4096) __nanosleep(100);  // poll tightly first: most waits are short
     }
-    __threadfence();
-    *s_flag = *verr;
+    bs->error = err;
   }
   __syncthreads();
-  return *s_flag == 0;
+  return bs->error == 0;
 }
 
 // All threads of all blocks of this thread-block cluster meet here: the hardware cluster

@@ -76,26 +76,27 @@ inline void default_tiles(int n, int& rty, int& rtx, int& cty, int& ctx) {
   ctx = Cg[n][1];
 }
 
-// Small grids: halve the larger tile side until the grid has at least one tile per SM (or
-// the tile is down to 4 cells), so that the few cells are spread over many blocks -- the
-// solves' phases are then short chains of work rather than long loops in a few blocks.
-inline void fit_tile(int Nx, int Ny, int sms, int& ty, int& tx) {
-  auto tiles = [&]() { return (long long)((Nx + tx - 1) / tx) * ((Ny + ty - 1) / ty); };
-  while (tiles() < sms && ty * tx > 4) {
-    if (tx >= ty && tx > 1)
-      tx /= 2;
-    else if (ty > 1)
-      ty /= 2;
-    else
-      break;
+// Small grids: halve the larger tile side while the grid then has at most `most` tiles (or the tile
+// is down to 4 cells), so that the few cells are spread over the SMs -- the phases are then short
+// chains of work rather than long loops in a few blocks.
+inline void fit_tile(int Nx, int Ny, int most, int& ty, int& tx) {
+  auto tiles = [&](int y, int x) { return (long long)((Nx + x - 1) / x) * ((Ny + y - 1) / y); };
+  while (ty * tx > 4) {
+    const int y = tx >= ty ? ty : (ty + 1) / 2, x = tx >= ty ? (tx + 1) / 2 : tx;
+    if (tiles(y, x) > most) break;
+    ty = y;
+    tx = x;
   }
 }
 
 inline void choose_tiles(int n, int Nx, int Ny, int sms, int& rty, int& rtx, int& cty, int& ctx) {
   default_tiles(n, rty, rtx, cty, ctx);
-  // two or more RHS blocks share an SM, so the RHS tiles shrink until there are two per SM
-  // (100^2 cells: n = 4 16.9 us on 325 tiles of 4 x 8, 19.1 on 169 of 8 x 8; n = 5 23.6 and 27.2)
-  fit_tile(Nx, Ny, 2 * sms, rty, rtx);
+  // two or three RHS blocks share an SM (100^2 cells: n = 4 16.6 us on 325 tiles of 4 x 8, 18.8 on
+  // 169 of 8 x 8; n = 5 22.8 and 26.9)
+  fit_tile(Nx, Ny, 3 * sms, rty, rtx);
+  // a solve's barriers and partial sums want few blocks: at most one per SM (us per iteration, n = 3,
+  // W^-1, with one tile per SM at most and with at least one: 32^2 cells 16.8 and 20.9, 48^2 17.6
+  // and 21.5, 64^2 18.2 and 21.4; n = 5, 64^2 23.2 and 24.9)
   fit_tile(Nx, Ny, sms, cty, ctx);
 }
 

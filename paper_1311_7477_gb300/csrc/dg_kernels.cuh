@@ -696,8 +696,7 @@ struct SolveCtx {
   Cplx<T>* line1;
   const T* Bs;                    // Bt staged in shared memory (null without preconditioner)
   T* red;
-  T* bcast;
-  int* s_flag;
+  BarrierState* bs;
   SyncState* sync;
   T* part;                        // 6 * vsize: two alternating halves of up to 3 sums
   int phase;
@@ -719,7 +718,7 @@ __device__ __forceinline__ bool solve_barrier(SolveCtx<T>& X) {
     cluster_barrier();
     return true;
   }
-  return grid_barrier(X.sync, X.s_flag, X.vsize);
+  return grid_barrier(X.sync, X.bs, X.vsize);
 }
 
 // Dynamic distribution of a phase's work units over the blocks of a solve: each block takes
@@ -747,46 +746,81 @@ __device__ __forceinline__ unsigned int read_ticket(const SyncState* s) {
   return *reinterpret_cast<const volatile unsigned int*>(&s->ticket);
 }
 
-// Block partials of one or two sums -> grid barrier -> the sums in every block (fixed order).
-template <typename T>
-__device__ __forceinline__ bool reduce_all(SolveCtx<T>& X, T v0, T& out0) {
+// Block partials of K sums -> grid barrier -> the sums in every block, in a fixed order that depends
+// only on the block count.  red: 32 K values.
+template <int K, typename T>
+__device__ __forceinline__ bool reduce_sums(SolveCtx<T>& X, T (&v)[K], T (&out)[K]) {
   T* ph = X.part + (X.phase & 1) * 3 * X.vsize;
   ++X.phase;
-  v0 = block_sum(v0, X.red);
-  if (threadIdx.x == 0) __stcg(ph + X.vrank, v0);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = int(blockDim.x >> 5);
+#pragma unroll
+  for (int j = 0; j < K; ++j) v[j] = warp_sum_down(v[j]);
+  __syncthreads();  // the previous use of red has been read
+  if (lane == 0) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) X.red[32 * j + w] = v[j];
+  }
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const T t = warp_sum_down(lane < nw ? X.red[32 * j + lane] : T(0));
+      if (lane == 0) __stcg(ph + K * X.vrank + j, t);
+    }
+  }
   if (!solve_barrier(X)) return false;
-  out0 = sum_partials_block(ph, X.vsize, 1, X.red, X.bcast);
+  if (X.vsize <= 128) {
+    // few blocks: every warp adds all partials itself, without another block synchronisation
+    T t[K] = {};
+    for (int i = lane; i < X.vsize; i += 32)
+#pragma unroll
+      for (int j = 0; j < K; ++j) t[j] += __ldcg(ph + K * i + j);
+#pragma unroll
+    for (int j = 0; j < K; ++j) out[j] = __shfl_sync(0xffffffffu, warp_sum_down(t[j]), 0);
+    return true;
+  }
+  T t[K] = {};
+  for (int i = threadIdx.x; i < X.vsize; i += blockDim.x)
+#pragma unroll
+    for (int j = 0; j < K; ++j) t[j] += __ldcg(ph + K * i + j);
+#pragma unroll
+  for (int j = 0; j < K; ++j) t[j] = warp_sum_down(t[j]);
+  if (lane == 0) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) X.red[32 * j + w] = t[j];
+  }
+  __syncthreads();
+  // every warp adds the warps' sums itself
+#pragma unroll
+  for (int j = 0; j < K; ++j)
+    out[j] = __shfl_sync(0xffffffffu, warp_sum_down(lane < nw ? X.red[32 * j + lane] : T(0)), 0);
+  return true;
+}
+
+template <typename T>
+__device__ __forceinline__ bool reduce_all(SolveCtx<T>& X, T v0, T& out0) {
+  T v[1] = {v0}, o[1];
+  if (!reduce_sums<1>(X, v, o)) return false;
+  out0 = o[0];
   return true;
 }
 
 template <typename T>
 __device__ __forceinline__ bool reduce_all2(SolveCtx<T>& X, T v0, T v1, T& out0, T& out1) {
-  T* ph = X.part + (X.phase & 1) * 3 * X.vsize;
-  ++X.phase;
-  v0 = block_sum(v0, X.red);
-  if (threadIdx.x == 0) __stcg(ph + 2 * X.vrank, v0);
-  v1 = block_sum(v1, X.red);
-  if (threadIdx.x == 0) __stcg(ph + 2 * X.vrank + 1, v1);
-  if (!solve_barrier(X)) return false;
-  out0 = sum_partials_block(ph, X.vsize, 2, X.red, X.bcast);
-  out1 = sum_partials_block(ph + 1, X.vsize, 2, X.red, X.bcast);
+  T v[2] = {v0, v1}, o[2];
+  if (!reduce_sums<2>(X, v, o)) return false;
+  out0 = o[0];
+  out1 = o[1];
   return true;
 }
 
 template <typename T>
 __device__ __forceinline__ bool reduce_all3(SolveCtx<T>& X, T v0, T v1, T v2, T& out0, T& out1, T& out2) {
-  T* ph = X.part + (X.phase & 1) * 3 * X.vsize;
-  ++X.phase;
-  v0 = block_sum(v0, X.red);
-  if (threadIdx.x == 0) __stcg(ph + 3 * X.vrank, v0);
-  v1 = block_sum(v1, X.red);
-  if (threadIdx.x == 0) __stcg(ph + 3 * X.vrank + 1, v1);
-  v2 = block_sum(v2, X.red);
-  if (threadIdx.x == 0) __stcg(ph + 3 * X.vrank + 2, v2);
-  if (!solve_barrier(X)) return false;
-  out0 = sum_partials_block(ph, X.vsize, 3, X.red, X.bcast);
-  out1 = sum_partials_block(ph + 1, X.vsize, 3, X.red, X.bcast);
-  out2 = sum_partials_block(ph + 2, X.vsize, 3, X.red, X.bcast);
+  T v[3] = {v0, v1, v2}, o[3];
+  if (!reduce_sums<3>(X, v, o)) return false;
+  out0 = o[0];
+  out1 = o[1];
+  out2 = o[2];
   return true;
 }
 
@@ -1710,15 +1744,14 @@ template <typename T, int N, typename TP = T, int MinB = (N == 5 ? 4 : 3)>
 __global__ void __launch_bounds__(kThreads, MinB) cg_kernel(const __grid_constant__ Ops2D<T, N> C, const Geom G,
                                                         const __grid_constant__ CgArgs<T, TP> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ T red[32];
-  __shared__ T bcast;
-  __shared__ int s_flag;
+  __shared__ T red[96];
+  __shared__ BarrierState bs;
+  if (threadIdx.x == 0) bs = BarrierState{0, 0};
   const Ops2D<T, N>& Cs = stage_table(C, smem_raw);
   SolveCtx<T> X;
   init_ctx<T, N, TP>(X, smem_raw + table_bytes<Ops2D<T, N>>(), G, A.pc.Bt, A.precond == 1, max(G.Nx, G.Ny));
   X.red = red;
-  X.bcast = &bcast;
-  X.s_flag = &s_flag;
+  X.bs = &bs;
   X.vrank = blockIdx.x;
   X.vsize = gridDim.x;
   X.cluster = A.cluster;
@@ -1977,11 +2010,10 @@ __global__ void __launch_bounds__(kThreads, MinB) mixed_cg_kernel(const __grid_c
                                                            const __grid_constant__ MixedArgs A) {
   constexpr int NN = N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[32];
-  __shared__ double bcd;
-  __shared__ float redf[32];
-  __shared__ float bcf;
-  __shared__ int s_flag;
+  __shared__ double redd[96];
+  __shared__ float redf[96];
+  __shared__ BarrierState bs;
+  if (threadIdx.x == 0) bs = BarrierState{0, 0};
   const bool pc = A.precond == kPrecondTwoLevel;  // the cell blocks are staged
   const int Lmax = max(G.Nx, G.Ny);
   const Ops2D<double, N>& Cds = stage_table(Cd, smem_raw);
@@ -1992,15 +2024,13 @@ __global__ void __launch_bounds__(kThreads, MinB) mixed_cg_kernel(const __grid_c
   SolveCtx<float> Xf;
   init_ctx<float, N>(Xf, smem, G, A.pc.Bt, pc, Lmax);
   Xf.red = redf;
-  Xf.bcast = &bcf;
-  Xf.s_flag = &s_flag;
+  Xf.bs = &bs;
   Xf.vrank = blockIdx.x;
   Xf.vsize = gridDim.x;
   SolveCtx<double> Xd;
   init_ctx<double, N>(Xd, smem + (pc ? align16(sizeof(float) * NN * NN) : 0), G, (const double*)nullptr, false, Lmax);
   Xd.red = redd;
-  Xd.bcast = &bcd;
-  Xd.s_flag = &s_flag;
+  Xd.bs = &bs;
   Xd.vrank = blockIdx.x;
   Xd.vsize = gridDim.x;
   Xf.cluster = Xd.cluster = A.cluster;
@@ -2095,7 +2125,7 @@ __host__ __device__ constexpr size_t batch_ops_bytes() {
 
 template <int N>
 __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int vrank, unsigned char* smem_all,
-                                           double* redd, double* bcd, float* redf, float* bcf, int* s_flag) {
+                                           double* redd, float* redf, BarrierState* bs) {
   constexpr int NN = N * N;
   const BatchSim& S = *Sp;
   // a simulation that has reached its step limit sits the step out (every block of the
@@ -2108,7 +2138,7 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
   unsigned char* smem = smem_all + batch_ops_bytes<N>();
   const FxRhs<N>& Fr = stage_table(*static_cast<const FxRhs<N>*>(S.ops_rhs), smem_all);
   batch_rhs<N>(S, Fr, oc, p0, r1, r2, rfree, vrank, grp.nblocks, smem);
-  if (!grid_barrier(grp.sync, s_flag, grp.nblocks)) return false;
+  if (!grid_barrier(grp.sync, bs, grp.nblocks)) return false;
   // the solve's tables (the barrier has synchronised the block: the RHS table is no longer read)
   const Ops2D<double, N>& Cd = stage_table(*static_cast<const Ops2D<double, N>*>(S.ops_d), smem_all);
   const Ops2D<float, N>& Cf =
@@ -2146,8 +2176,7 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     SolveCtx<double> X;
     init_ctx<double, N>(X, smem, S.Gc, S.pc.Bt, pc, Lmax);
     X.red = redd;
-    X.bcast = bcd;
-    X.s_flag = s_flag;
+    X.bs = bs;
     X.vrank = vrank;
     X.vsize = grp.nblocks;
     cg_solve<double, N>(Cd, S.Gc, A, X);
@@ -2183,21 +2212,19 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     SolveCtx<float> Xf;
     init_ctx<float, N>(Xf, smem, S.Gc, S.pcf.Bt, pc, Lmax);
     Xf.red = redf;
-    Xf.bcast = bcf;
-    Xf.s_flag = s_flag;
+    Xf.bs = bs;
     Xf.vrank = vrank;
     Xf.vsize = grp.nblocks;
     SolveCtx<double> Xd;
     init_ctx<double, N>(Xd, smem + (pc ? align16(sizeof(float) * NN * NN) : 0), S.Gc, (const double*)nullptr, false, Lmax);
     Xd.red = redd;
-    Xd.bcast = bcd;
-    Xd.s_flag = s_flag;
+    Xd.bs = bs;
     Xd.vrank = vrank;
     Xd.vsize = grp.nblocks;
     mixed_solve<N>(Cd, Cf, Ck, S.Gc, A, Xf, Xd);
   }
   // every block has finished the solve before the rings move
-  if (!grid_barrier(grp.sync, s_flag, grp.nblocks)) return false;
+  if (!grid_barrier(grp.sync, bs, grp.nblocks)) return false;
   if (vrank == 0 && threadIdx.x == 0) {
     Sp->apsi_ok[p2] = S.fixed_iters == 0 ? 1 : 0;
     Sp->oc = oc ^ 1;
@@ -2211,7 +2238,7 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     Sp->step = S.step + 1;
     __threadfence();
   }
-  return grid_barrier(grp.sync, s_flag, grp.nblocks);
+  return grid_barrier(grp.sync, bs, grp.nblocks);
 }
 
 

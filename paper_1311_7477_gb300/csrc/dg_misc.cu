@@ -18,9 +18,10 @@ __global__ void invariants_final_kernel(const double* __restrict__ part, int npa
 // Self-test of the capped grid barrier: block 0 never arrives, so every other block's wait
 // runs out after kSpinCap polls and raises kFlagTimeout; nothing faults or hangs.
 __global__ void barrier_selftest_kernel(SyncState* s, int* out) {
-  __shared__ int f;
+  __shared__ BarrierState bs;
   if (blockIdx.x == 0) return;
-  const bool ok = grid_barrier(s, &f, gridDim.x);
+  if (threadIdx.x == 0) bs = BarrierState{0, 0};
+  const bool ok = grid_barrier(s, &bs, gridDim.x);
   if (threadIdx.x == 0 && !ok) atomicOr(out, kFlagTimeout);
 }
 
