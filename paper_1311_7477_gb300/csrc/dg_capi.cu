@@ -188,7 +188,7 @@ int exp_above(double v) {
 }
 
 template <int N>
-FxRhs<N> make_fx_rhs(const RefTables& t, double hx, double hy, double tau) {
+FxRhs<N> make_fx_rhs(const RefTables& t, double hx, double hy) {
   FxRhs<N> F{};
   double big = 0.0;
   for (int j = 0; j < N; ++j) big = std::max(big, 1.0 / t.w[j]);
@@ -196,12 +196,76 @@ FxRhs<N> make_fx_rhs(const RefTables& t, double hx, double hy, double tau) {
   for (int k = 0; k < N * N; ++k) F.isw[k] = fx_coef(1.0 / std::sqrt(t.w[k / N] * t.w[k % N]), 60 - F.ei);
   F.cj = 1.0 / (hx * hy);
   F.cp = 2.0 / std::sqrt(hx * hy);
-  F.clx = 1.0 / (hx * hx);
-  F.cly = 1.0 / (hy * hy);
   auto mid = [](double v) { return v > 1e-80 && v < 1e80; };
   F.ok = mid(F.cj) && mid(F.cp) && mid(F.cj * F.cp);
-  F.lap_ok = tau == 0.0 && mid(F.clx) && mid(F.cly);
+  F.l = FxScale{1.0 / (hx * hx), 1.0 / (hy * hy), 0, nullptr, nullptr};
+  F.l.ok = mid(F.l.cx) && mid(F.l.cy);
   return F;
+}
+
+// An operator on the reference cell as a table in memory (grids with a jump penalty).
+template <int N>
+FxTable<N> make_fx_table(const Op1D<double, N>& o) {
+  FxTable<N> t{};
+  double r = 0.0, s = 0.0, row = 0.0;
+  for (int j = 0; j < N; ++j) {
+    r += std::fabs(o.r[j]);
+    s += std::fabs(o.s[j]);
+  }
+  for (int i = 0; i < N; ++i) {
+    double v = std::fabs(o.a[i]) * r + std::fabs(o.d[i]) * s;
+    for (int j = 0; j < N; ++j) v += std::fabs(o.M[i][j]);
+    row = std::max(row, v);
+  }
+  t.e = exp_above(row);
+  t.er = exp_above(r);
+  t.es = exp_above(s);
+  // the lifts' high parts, |a| 2^(er - e + 30) and |d| 2^(es - e + 30), must fit in an int
+  for (int i = 0; i < N; ++i)
+    while (std::ldexp(std::fabs(o.a[i]), t.er - t.e) > 1.9 || std::ldexp(std::fabs(o.d[i]), t.es - t.e) > 1.9) ++t.e;
+  for (int i = 0; i < N; ++i) {
+    for (int j = 0; j < N; ++j) t.M[i][j] = fx_coef(o.M[i][j], 60 - t.e);
+    t.a[i] = fx_coef(o.a[i], 60 - t.e + t.er);
+    t.r[i] = fx_coef(o.r[i], 60 - t.er);
+    t.d[i] = fx_coef(o.d[i], 60 - t.e + t.es);
+    t.s[i] = fx_coef(o.s[i], 60 - t.es);
+  }
+  return t;
+}
+
+// The grid's fixed-point tables for a jump penalty: {stiffness, Laplacian} to tab.
+void fill_fx_tables(const dg_grid* g, unsigned char* tab) {
+  dispatch_n(g->n, [&](auto nc) {
+    constexpr int N = decltype(nc)::value;
+    const Ops2D<double, N> O = make_ops<double, N>(g->rt, 1.0, 1.0);
+    const FxTable<N> t[2] = {make_fx_table<N>(O.kx), make_fx_table<N>(O.lx)};
+    std::memcpy(tab, t, sizeof(t));
+    return DG_OK;
+  });
+}
+
+// Points the grid's operators at its tables in device memory.
+void set_fx_tables(dg_grid* g, void* dev) {
+  dispatch_n(g->n, [&](auto nc) {
+    constexpr int N = decltype(nc)::value;
+    const FxTable<N>* t = static_cast<const FxTable<N>*>(dev);
+    g->ks.stiff = t;
+    g->ks.lap = t + 1;
+    reinterpret_cast<FxRhs<N>*>(g->ops.x)->l = g->ks;
+    return DG_OK;
+  });
+}
+
+constexpr size_t kFxTabBytes = 2 * sizeof(FxTable<kMaxN>);
+
+int upload_fx_tables(dg_grid* g) {
+  if (g->tau == 0.0) return DG_OK;
+  unsigned char tab[kFxTabBytes] = {};
+  fill_fx_tables(g, tab);
+  CUDA_TRY(cudaMalloc(&g->d_fxtab, kFxTabBytes));
+  CUDA_TRY(cudaMemcpy(g->d_fxtab, tab, kFxTabBytes, cudaMemcpyHostToDevice));
+  set_fx_tables(g, g->d_fxtab);
+  return DG_OK;
 }
 
 // Gershgorin bound on the largest eigenvalue of the CG operator Ahat = I (x) kx + ky (x) I:
@@ -243,7 +307,8 @@ template <int N>
 void build_ops(dg_grid* g) {
   new (g->ops.d) Ops2D<double, N>(make_ops<double, N>(g->rt, g->hx, g->hy));
   new (g->ops.f) Ops2D<float, N>(make_ops<float, N>(g->rt, g->hx, g->hy));
-  new (g->ops.x) FxRhs<N>(make_fx_rhs<N>(g->rt, g->hx, g->hy, g->tau));
+  new (g->ops.x) FxRhs<N>(make_fx_rhs<N>(g->rt, g->hx, g->hy));
+  g->ks = fxrhs_of<N>(g).l;
   const Ops2D<df, N> x = make_ops<df, N>(g->rt, g->hx, g->hy);
   new (g->ops.k) OpsK<df, N>(OpsK<df, N>{x.kx, x.ky});
   const Ops2D<double, N>& Od = *reinterpret_cast<const Ops2D<double, N>*>(g->ops.d);
@@ -595,11 +660,10 @@ int dg_grid_create_bc(dg_grid** gp, int Nx, int Ny, int n, double Lx, double Ly,
   int rc = alloc_ws(g->ws, ndof_of(g), co_resident_cap(g), true);
   if (!rc) rc = alloc_ws_precond(g->ws, Nx, Ny, n, false);
   if (!rc) rc = build_pc(g);
+  if (!rc) rc = upload_fx_tables(g);
   if (!rc) rc = upload_ops(g);
   if (rc) {
-    free_ws(g->ws);
-    free_pc(g->pc);
-    delete g;
+    dg_grid_destroy(g);
     return rc;
   }
   *gp = g;
@@ -614,6 +678,7 @@ int dg_grid_destroy(dg_grid* g) {
   cudaFree(g->d_opsf);
   cudaFree(g->d_opsx);
   cudaFree(g->d_opsk);
+  cudaFree(g->d_fxtab);
   delete g;
   return DG_OK;
 }
@@ -740,7 +805,7 @@ int dg_laplace_apply(dg_grid* g, const double* x, double* y, int mode, void* str
   if (!aligned8(x) || !aligned8(y)) return fail(DG_ERR_ARG, "misaligned pointer");
   if (x == y) return fail(DG_ERR_ARG, "y must not alias x");
   return dispatch_n(g->n,
-                    [&](auto nc) { return launch_apply<double, decltype(nc)::value>(g, x, y, mode, as_stream(stream)); });
+                    [&](auto nc) { return launch_apply<decltype(nc)::value>(g, x, y, mode, as_stream(stream)); });
 }
 
 int dg_poisson_solve(dg_grid* g, const double* omega, double* psi, double tol, int maxit, int fixed_iters,
@@ -1451,6 +1516,7 @@ struct StaticScratch {
   double part[6 * kStaticMaxBlocks];
   SyncState sync;
   SolveStatus status;
+  alignas(16) unsigned char tab[kFxTabBytes];  // fixed-point tables of a grid with a jump penalty
 };
 
 static __device__ __align__(256) StaticScratch g_static_scratch;
@@ -1504,6 +1570,12 @@ extern "C" int dg_poisson_solve_static(int Nx, int Ny, int n, double Lx, double 
     build_ops<decltype(nc)::value>(&g);
     return DG_OK;
   });
+  if (tau != 0.0) {
+    unsigned char tab[kFxTabBytes] = {};
+    fill_fx_tables(&g, tab);
+    CUDA_TRY(cudaMemcpyAsync(sc->tab, tab, kFxTabBytes, cudaMemcpyHostToDevice, st));
+    set_fx_tables(&g, sc->tab);
+  }
   Workspace w{};
   w.ndof = (size_t)ndof;
   w.grid_cap = kStaticMaxBlocks;
@@ -1638,6 +1710,7 @@ BatchSim make_batch_sim(const dg_batch* bt, dg_sim* s) {
   b.max_sweeps = s->max_sweeps;
   b.fixed_iters = s->fixed_iters;
   b.sumW = g->Lx * g->Ly;
+  b.ks = g->ks;
   b.r = s->ws.r;
   b.p0v = s->ws.p0;
   b.p1v = s->ws.p1;

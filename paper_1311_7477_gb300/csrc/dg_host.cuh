@@ -158,6 +158,8 @@ struct dg_grid {
   int rTY, rTX, cTY, cTX;
   int num_sms;
   OpsHost ops;
+  FxScale ks{};  // factors (and, with a jump penalty, tables) of the fixed-point LDG operators
+  void* d_fxtab = nullptr;  // the tables: FxTable<n> of the stiffness and of the Laplacian
   Workspace ws;
   int precond = 0;  // DG_PRECOND_JACOBI, DG_PRECOND_TWOLEVEL or DG_PRECOND_SPECTRAL
   bool cluster_ok = true;  // small solves may run as one thread-block cluster
@@ -338,7 +340,7 @@ inline int co_resident_cap(const dg_grid* g) { return std::max(64, 8 * g->num_sm
 // ---- per-n kernel launchers (dg_launch.cuh; instantiated in dg_inst_n<N>.cu) -------------
 template <int N>
 int launch_rhs(const dg_grid* g, const RhsArgs& A, cudaStream_t st);
-template <typename T, int N>
+template <int N>
 int launch_apply(const dg_grid* g, const double* x, double* y, int mode, cudaStream_t st);
 template <typename T, int N, typename TP = T>
 int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_t st, dg_sim* timed = nullptr);

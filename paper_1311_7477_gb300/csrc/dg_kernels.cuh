@@ -238,6 +238,43 @@ __device__ __forceinline__ void rhs_box_float(const Ops2D<T, N>& C, const Geom& 
   __syncthreads();
 }
 
+// Cell stride of the fixed-point staging: odd, so that the lanes of a warp, which read the same
+// node of consecutive cells, fall on distinct pairs of banks.
+template <int N>
+__host__ __device__ constexpr int fx_cell() {
+  return (N * N) | 1;
+}
+
+// The factors of the fixed-point LDG operators, 1 / hx^2 and 1 / hy^2.  ok: they lie in the range the
+// fixed-point path covers.  stiff, lap: device tables (FxTable<n>) that replace fx_stiff and fx_lap
+// on grids with a jump penalty tau != 0, else null.
+struct FxScale {
+  double cx, cy;
+  int ok;
+  const void *stiff, *lap;
+};
+
+// One LDG operator on all lines of a tile with a table in memory: x-lines to qx, y-lines to qy, cell
+// (ry, rx) of the results at (ry * orow + rx + ooff).  Periodic grids (a penalty needs one).
+template <int N>
+__device__ __noinline__ void fx_lines_table(const FxTable<N>* O, const TileBox& B, const fx* sU, long long* qx,
+                                            long long* qy, int orow, int ooff) {
+  constexpr int CS = fx_cell<N>();
+  const int nc = B.TYe * B.TXe;
+  const unsigned mnc = magic_of(nc);
+  for (int u = threadIdx.x; u < 2 * nc * N; u += blockDim.x) {
+    asm volatile("" : "+l"(O));  // keeps the table out of registers across the lines
+    const bool alongx = u < nc * N;
+    const int v = alongx ? u : u - nc * N;
+    const int ln = quot(v, mnc), c = v - ln * nc;
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const int st = alongx ? 1 : N, first = alongx ? ln * N : ln;
+    long long* q = (alongx ? qx : qy) + (ry * orow + rx + ooff) * CS + first;
+    fx_line<N>(*O, sU + ((ry + 1) * B.BW + rx + 1) * CS + first, st, alongx ? CS : B.BW * CS,
+               [&](int i, long long y) { q[i * st] = y; });
+  }
+}
+
 // What the fixed-point right-hand side (dg_fixed.cuh) takes from the grid.  The derivative and the
 // Laplacian are tables of n on the reference cell, so every term of J carries the same factor
 // 1 / (hx hy), applied once to the finished sum; likewise 1 / sqrt(W) is 1 / sqrt(w_a w_b) times
@@ -247,17 +284,9 @@ struct FxRhs {
   fx isw[N * N];   // 1 / sqrt(w_a w_b) = 2^(ei - 60) isw
   int ei;
   int ok;          // the factors lie in the range the fixed-point path covers
-  int lap_ok;      // ... and the Laplacian's (its table holds for the penalty tau = 0)
   double cj, cp;   // 1 / (hx hy), 2 / sqrt(hx hy)
-  double clx, cly; // 1 / hx^2, 1 / hy^2
+  FxScale l;       // the Laplacian's
 };
-
-// Cell stride of the fixed-point staging: odd, so that the lanes of a warp, which read the same
-// node of consecutive cells, fall on distinct pairs of banks.
-template <int N>
-__host__ __device__ constexpr int fx_cell() {
-  return (N * N) | 1;
-}
 
 // Shared memory of one right-hand-side tile: five arrays over the box, or the float64 fallback on
 // single cells, whichever is larger.
@@ -377,10 +406,10 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
   const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
   // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any)
   const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
-  const int uj = uf + ug + 2 * D.e + 60, ul = ug + Lp.e;
+  const int uj = uf + ug + 2 * D.e + 60, ul = ug + (F.l.lap ? static_cast<const FxTable<N>*>(F.l.lap)->e : Lp.e);
   const bool viscous = A.visc != 0.0 && !A.bracket_only;
   // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
-  const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.lap_ok && abs(ul) <= 600));
+  const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.l.ok && abs(ul) <= 600));
   if (!covered) {
     __syncthreads();  // the staging is reused
     rhs_tile_float<N>(C, G, A, tile, smem);
@@ -488,7 +517,11 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
     }
   }
   __syncthreads();
-  if (viscous) {  // lx g over h1, ly g over h2
+  if (viscous && F.l.lap) {  // lx g over h1, ly g over h2
+    fx_lines_table<N>(static_cast<const FxTable<N>*>(F.l.lap), B, sG, reinterpret_cast<long long*>(sB),
+                      reinterpret_cast<long long*>(sC), BW, BW + 1);
+    __syncthreads();
+  } else if (viscous) {
     for (int u = threadIdx.x; u < 2 * nc * N; u += blockDim.x) {
       const bool alongx = u < nc * N;
       const int v = alongx ? u : u - nc * N;
@@ -515,8 +548,8 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
   }
   // nodes: J and the update
   const double cJ = (parts == 7 ? 1.0 / 3.0 : 1.0) * F.cj * (A.psi_scaled ? F.cp : 1.0) * fx_pow2(uj);
-  const double cLx = A.visc * F.clx * fx_pow2(ul), cLy = A.visc * F.cly * fx_pow2(ul);
-  const bool square = F.clx == F.cly;
+  const double cLx = A.visc * F.l.cx * fx_pow2(ul), cLy = A.visc * F.l.cy * fx_pow2(ul);
+  const bool square = F.l.cx == F.l.cy;
   const int nin = nc * NN;
 #pragma unroll 2
   for (int i = threadIdx.x; i < nin; i += blockDim.x) {
@@ -555,48 +588,163 @@ __global__ void __launch_bounds__(rhs_threads<N>(), rhs_blocks<N>()) rhs_kernel(
 }
 
 // =========================================================================================
+// One tile of an LDG operator on a float64 field in fixed point (dg_fixed.cuh).
+// =========================================================================================
+
+// Shared memory of the pass: the staged box and the two directions' results on the tile.
+template <int N>
+__host__ __device__ constexpr size_t fx_apply_bytes(int TY, int TX) {
+  return ((size_t)(TY + 2) * (TX + 2) + 2 * (size_t)TY * TX) * fx_cell<N>() * 8;
+}
+
+// The lines of the tile in float64, for tiles the fixed-point scale cannot hold.
+template <int N>
+__device__ __noinline__ void apply_lines_float(const Op1D<double, N>& ox, const Op1D<double, N>& oy, const Geom& G,
+                                               const TileBox& B, const double* sU, double* qx, double* qy) {
+  constexpr int CS = fx_cell<N>();
+  const int nc = B.TYe * B.TXe;
+  for (int u = threadIdx.x; u < 2 * nc * N; u += blockDim.x) {
+    const bool alongx = u < nc * N;
+    const int v = alongx ? u : u - nc * N;
+    const int ln = v / nc, c = v - ln * nc;
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const Op1D<double, N>& o = alongx ? ox : oy;
+    const int st = alongx ? 1 : N, dc = alongx ? CS : B.BW * CS, first = alongx ? ln * N : ln;
+    const double* w = sU + ((ry + 1) * B.BW + rx + 1) * CS + first;
+    double* q = (alongx ? qx : qy) + (ry * G.TX + rx) * CS + first;
+    const int pos = G.bc ? (alongx ? B.tx0 + rx : B.ty0 + ry) : 2;
+    double tr = 0.0, tl = 0.0;
+    for (int j = 0; j < N; ++j) {
+      tr = fma(o.r[j], w[dc + j * st], tr);
+      tl = fma(pos == 1 ? o.sf[j] : o.s[j], w[j * st - dc], tl);
+    }
+    for (int i = 0; i < N; ++i) {
+      double acc = (pos == 0 ? o.af[i] : o.a[i]) * tr;
+      acc = fma(o.d[i], tl, acc);
+      for (int j = 0; j < N; ++j) acc = fma(pos == 0 ? o.Mf[i][j] : o.M[i][j], w[j * st], acc);
+      q[i * st] = acc;
+    }
+  }
+}
+
+// Stages u = load(g, k, interior) on the tile and its plus-shaped halo, applies the operator (Lap:
+// -Delta_h, else W^-1/2 A W^-1/2; ox, oy its float64 form) and hands (g, k, q) of the tile's nodes
+// to out.  smem: fx_apply_bytes<N>(G.TY, G.TX).
+template <int N, bool Lap, class LoadF, class OutF>
+__device__ __forceinline__ void fx_tile_apply(const Op1D<double, N>& ox, const Op1D<double, N>& oy, const FxScale& S,
+                                              const Geom& G, int tile, void* smem, LoadF&& load, OutF&& out) {
+  constexpr int NN = N * N;
+  constexpr int CS = fx_cell<N>();
+  constexpr FxTable<N> O = Lap ? fx_lap<N>() : fx_stiff<N>();
+  __shared__ unsigned s_mag[32];
+  const TileBox B = make_box(G, tile);
+  const int BW = B.BW, boxc = (G.TY + 2) * BW;
+  fx* sU = static_cast<fx*>(smem);
+  long long* qx = reinterpret_cast<long long*>(sU + boxc * CS);
+  long long* qy = qx + G.TY * G.TX * CS;
+  unsigned m = 0;
+  {
+    double* rU = reinterpret_cast<double*>(sU);
+    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+    const int rowlen = BWe * NN, total = BHe * rowlen;
+    const unsigned mrow = magic_of(rowlen);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int br = quot(i, mrow);
+      const int j = i - br * rowlen;
+      const int bc = j / NN, k = j - bc * NN;
+      const bool rowhalo = (br == 0) || (br == BHe - 1), colhalo = (bc == 0) || (bc == BWe - 1);
+      if (rowhalo && colhalo) continue;  // the 5-cell operators never read the corners
+      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+      const int o = (br * BW + bc) * CS + k;
+      double v = 0.0;  // Dirichlet: zero outside
+      if (!(G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)))
+        v = load(((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k, k, !(rowhalo || colhalo));
+      rU[o] = v;
+      m = max(m, fx_mag(v));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) s_mag[threadIdx.x >> 5] = m;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  m = __reduce_max_sync(0xffffffffu, lane < int(blockDim.x >> 5) ? s_mag[lane] : 0u);
+  const FxTable<N>* tab = static_cast<const FxTable<N>*>(Lap ? S.lap : S.stiff);
+  const int em = max(1, int(m >> 20)), uq = m ? em - 1082 + (tab ? tab->e : O.e) : 0;
+  const bool covered = S.ok && em < 2047 && abs(uq) <= 600;
+  const int nc = B.TYe * B.TXe;
+  if (covered) {
+    for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
+      const fx w = sU[i];  // raw bits: {low, high} words
+      sU[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), em));
+    }
+    __syncthreads();
+    const unsigned mnc = magic_of(nc);
+    if (tab) fx_lines_table<N>(tab, B, sU, qx, qy, G.TX, 0);
+    for (int u = threadIdx.x; u < (tab ? 0 : 2 * nc * N); u += blockDim.x) {
+      const bool alongx = u < nc * N;
+      const int v = alongx ? u : u - nc * N;
+      const int ln = quot(v, mnc), c = v - ln * nc;
+      const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+      const fx* w = sU + ((ry + 1) * BW + rx + 1) * CS;
+      const int t = (ry * G.TX + rx) * CS;
+      if (alongx) {
+        auto put = [&](int i, long long y) { qx[t + ln * N + i] = y; };
+        if (G.bc && B.tx0 + rx < 2)
+          fx_ldg_bounded<N>(O, w + ln * N, 1, CS, B.tx0 + rx, put);
+        else
+          fx_line<N>(O, w + ln * N, 1, CS, put);
+      } else {
+        auto put = [&](int i, long long y) { qy[t + ln + i * N] = y; };
+        if (G.bc && B.ty0 + ry < 2)
+          fx_ldg_bounded<N>(O, w + ln, N, BW * CS, B.ty0 + ry, put);
+        else
+          fx_line<N>(O, w + ln, N, BW * CS, put);
+      }
+    }
+  } else {
+    apply_lines_float<N>(ox, oy, G, B, reinterpret_cast<const double*>(sU), reinterpret_cast<double*>(qx),
+                         reinterpret_cast<double*>(qy));
+  }
+  __syncthreads();
+  const double cx = S.cx * fx_pow2(uq), cy = S.cy * fx_pow2(uq);
+  const bool square = S.cx == S.cy;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < nc * NN; i += blockDim.x) {
+    const int c = i / NN, k = i - c * NN;
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const int t = (ry * G.TX + rx) * CS + k;
+    const long long a = qx[t], b = qy[t];
+    double q;
+    if (!covered)
+      q = __longlong_as_double(a) + __longlong_as_double(b);
+    else if (square)
+      q = fx_to_double(a + b) * cx;
+    else
+      q = fma(fx_to_double(a), cx, fx_to_double(b) * cy);
+    out(((size_t)(B.ty0 + ry) * G.Nx + (B.tx0 + rx)) * NN + k, k, q);
+  }
+  __syncthreads();
+}
+
+// =========================================================================================
 // Operator application: mode 0  y = A x = W^1/2 (W^-1/2 A W^-1/2) W^1/2 x,
 //                       mode 1  y = Delta_h x = -(lx + ly) x.
 // =========================================================================================
-template <typename T, int N>
-__host__ __device__ constexpr size_t apply_smem_values(int TY, int TX) {
-  return (size_t)(TY + 2) * (TX + 2) * (N * N + 1 + 4 * N);
-}
-
-template <typename T, int N>
-__global__ void __launch_bounds__(kThreads) apply_kernel(const __grid_constant__ Ops2D<T, N> Cp, const Geom G,
-                                                        const double* __restrict__ x, double* __restrict__ y,
-                                                        int mode) {
-  constexpr int NN = N * N;
+template <int N, bool Lap>
+__global__ void __launch_bounds__(kThreads, 4) apply_kernel(const __grid_constant__ Ops2D<double, N> C,
+                                                         const FxScale S, const Geom G, const double* __restrict__ x,
+                                                         double* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const Ops2D<T, N>& C = stage_table(Cp, smem_raw);
-  T* sU = reinterpret_cast<T*>(smem_raw + table_bytes<Ops2D<T, N>>());
-  const int boxc = (G.TY + 2) * (G.TX + 2);
-  T *tXR = sU + boxc * (NN + 1), *tXL = tXR + boxc * N, *tYR = tXL + boxc * N, *tYL = tYR + boxc * N;
-  const TileBox B = make_box(G, blockIdx.x);
-  const Op1D<T, N>& ox = mode == 0 ? C.kx : C.lx;
-  const Op1D<T, N>& oy = mode == 0 ? C.ky : C.ly;
-  stage_box<T, N>(G, B, sU, false, [&](size_t g, int k, bool) {
-    return mode == 0 ? T(x[g]) * C.sw[k] : T(x[g]);
-  });
-  __syncthreads();
-  line_traces<T, N>(B, sU, sU, ox, oy, tXR, tXL, tYR, tYL, false);
-  __syncthreads();
-  if (G.bc) {
-    dirichlet_first_traces<T, N>(B, sU, sU, ox, oy, tXL, tYL);
+  __shared__ double s_sw[N * N];
+  if constexpr (!Lap) {
+    if (threadIdx.x < N * N) s_sw[threadIdx.x] = C.sw[threadIdx.x];
     __syncthreads();
   }
-  const int nin = B.TYe * B.TXe * NN;
-  for (int i = threadIdx.x; i < nin; i += blockDim.x) {
-    const int c = i / NN, k = i - (i / NN) * NN;
-    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
-    const int lc = (ry + 1) * B.BW + rx + 1;
-    const int a = k / N, b = k - (k / N) * N;
-    const bool fx = G.bc && B.tx0 + rx == 0, fy = G.bc && B.ty0 + ry == 0;
-    const T q = op_x_at<T, N>(sU, tXR, tXL, ox, lc, a, b, fx) + op_y_at<T, N>(sU, tYR, tYL, oy, lc, B.BW, a, b, fy);
-    const size_t g = ((size_t)(B.ty0 + ry) * G.Nx + (B.tx0 + rx)) * NN + k;
-    y[g] = mode == 0 ? double(q * C.sw[k]) : -double(q);
-  }
+  fx_tile_apply<N, Lap>(
+      Lap ? C.lx : C.kx, Lap ? C.ly : C.ky, S, G, blockIdx.x, smem_raw,
+      [&](size_t g, int k, bool) { return Lap ? x[g] : x[g] * s_sw[k]; },
+      [&](size_t g, int k, double q) { y[g] = Lap ? -q : q * s_sw[k]; });
 }
 
 // =========================================================================================
@@ -708,6 +856,7 @@ struct SolveCtx {
   // buffers wU, wXR, wXL, wYR, wYL (the float64 context's staging region)
   const void* kdf;
   df *wU, *wXR, *wXL, *wYR, *wYL;
+  FxScale ks;                     // factors of the fixed-point operator (float64 solves)
 };
 
 // The barrier between the phases of a solve: the hardware cluster barrier when the solve's
@@ -824,8 +973,8 @@ __device__ __forceinline__ bool reduce_all3(SolveCtx<T>& X, T v0, T v1, T v2, T&
   return true;
 }
 
-// One CG tile pass: stage u = load(...) (plus-shaped halo), apply Ahat, hand (g, k, u, q)
-// to out(...).
+// One CG tile pass in float32 or double-float: stage u = load(...) (plus-shaped halo), apply Ahat,
+// hand (g, k, u, q) to out(...).
 template <typename T, int N, class Tab, class LoadF, class OutF>
 __device__ __forceinline__ void cg_tile_apply(const Tab& C, const Geom& G, int tile, SolveCtx<T>& X, LoadF&& load,
                                               OutF&& out) {
@@ -912,16 +1061,18 @@ __device__ __forceinline__ void cg_tile_apply(const Tab& C, const Geom& G, int t
   __syncthreads();
 }
 
-// One tile pass of the solve's operator: cg_tile_apply in T, or -- for a float32 solve with
-// the compensated apply enabled -- in double-float arithmetic on the same float32 values, the
-// result rounded to float32.  A float32 evaluation of Ahat u has an absolute error of about
+// One tile pass of the solve's operator, (g, k, q) handed to out: a float64 solve in fixed point
+// (fx_tile_apply), a float32 one in float32 or -- with the compensated apply enabled -- in
+// double-float arithmetic on the same float32 values, the result rounded to float32.  A float32 evaluation of Ahat u has an absolute error of about
 // eps32 |Ahat| |u|, which on the smoothest modes of a fine grid (eigenvalue ~1 against
 // |Ahat| ~ 1e7 at 1024^2 cells, n = 5) is as large as Ahat u itself; the double-float apply
 // brings it down to ~eps32^2 |Ahat| |u|.
 template <typename T, int N, class LoadF, class OutF>
 __device__ __forceinline__ void solve_apply(const Ops2D<T, N>& C, const Geom& G, int tile, SolveCtx<T>& X,
                                             LoadF&& load, OutF&& out) {
-  if constexpr (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, double>::value) {
+    fx_tile_apply<N, false>(C.kx, C.ky, X.ks, G, tile, X.sU, load, out);
+  } else {
     if (X.kdf) {
       SolveCtx<df> W;
       W.sU = X.wU;
@@ -932,11 +1083,11 @@ __device__ __forceinline__ void solve_apply(const Ops2D<T, N>& C, const Geom& G,
       cg_tile_apply<df, N>(
           *static_cast<const OpsK<df, N>*>(X.kdf), G, tile, W,
           [&](size_t g, int k, bool interior) { return df(load(g, k, interior)); },
-          [&](size_t g, int k, df u, df q) { out(g, k, u.hi, to_float(q)); });
+          [&](size_t g, int k, df, df q) { out(g, k, to_float(q)); });
       return;
     }
+    cg_tile_apply<T, N>(C, G, tile, X, load, [&](size_t g, int k, T, T q) { out(g, k, q); });
   }
-  cg_tile_apply<T, N>(C, G, tile, X, load, out);
 }
 
 // Where the tile's residual is staged for the preconditioner's cell part: X.sU itself, or,
@@ -1360,7 +1511,8 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
       for (int t = X.vrank; t < ntiles; t += X.vsize) {
         solve_apply<T, N>(
             C, G, t, X, [&](size_t g, int, bool) { return __ldcg(V.y + g); },
-            [&](size_t g, int k, T yv, T qv) {
+            [&](size_t g, int k, T qv) {
+              const T yv = __ldcg(V.y + g);
               const T r = rhs_at<T, N>(C, Bsrc, g, k) - qv;
               __stcg(V.r + g, r);
               if (ay) __stcg(ay + g, qv);
@@ -1415,9 +1567,9 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
             if (interior) __stcg(pout + g, pv);
             return pv;
           },
-          [&](size_t g, int, T pv, T qv) {
+          [&](size_t g, int, T qv) {  // p of the tile: written above, by this block
             __stcg(V.q + g, qv);
-            pq = fma(pv, qv, pq);
+            pq = fma(__ldcg(pout + g), qv, pq);
           });
     }
     T pqs = T(0);
@@ -1562,6 +1714,7 @@ struct CgArgs {
   double sumW;
   int cluster;          // launched as one thread-block cluster (cluster barriers)
   int keep_mean;        // homogeneous Dirichlet: A is definite, b = sqrt(W) omega (no mean removed)
+  FxScale ks;           // factors of the fixed-point operator
 };
 
 // Dynamic shared memory of the persistent solves: [Bt (with the preconditioner)] then one
@@ -1571,6 +1724,16 @@ __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) & ~size
 template <typename T, int N>
 __host__ __device__ constexpr size_t cg_tile_values(int TY, int TX) {
   return (size_t)(TY + 2) * (TX + 2) * (N * N + 1 + 4 * N);
+}
+
+// Bytes of the tile staging of a solve: float32 (and, in 8-byte values, double-float) operator
+// applications use cg_tile_values, float64 ones the fixed-point pass; the two-level
+// preconditioner's cell part stages a box of values with, in float64, a float32 copy beside it.
+template <typename T, int N>
+__host__ __device__ constexpr size_t cg_tile_bytes(int TY, int TX) {
+  if (sizeof(T) == 4) return cg_tile_values<T, N>(TY, TX) * sizeof(T);
+  const size_t a = fx_apply_bytes<N>(TY, TX), b = (size_t)(TY + 2) * (TX + 2) * (N * N + 1) * 12;
+  return a > b ? a : b;
 }
 
 // Bytes of the DFT line buffers of a preconditioner (kind: PrecondArgs): two lines for the
@@ -1586,8 +1749,8 @@ __host__ __device__ constexpr size_t pc_line_bytes(int kind, int Lmax, bool pow2
 template <typename T, int N>
 __host__ __device__ constexpr size_t cg_smem_bytes(int TY, int TX, int Lmax, int kind, bool pow2) {
   return (kind == kPrecondTwoLevel ? align16(sizeof(T) * N * N * N * N) : 0) +
-         align16(cg_tile_values<T, N>(TY, TX) * sizeof(T) > pc_line_bytes<T, N>(kind, Lmax, pow2)
-                     ? cg_tile_values<T, N>(TY, TX) * sizeof(T)
+         align16(cg_tile_bytes<T, N>(TY, TX) > pc_line_bytes<T, N>(kind, Lmax, pow2)
+                     ? cg_tile_bytes<T, N>(TY, TX)
                      : pc_line_bytes<T, N>(kind, Lmax, pow2));
 }
 
@@ -1628,6 +1791,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
   X.sync = A.sync;
   X.part = A.part;
   X.phase = 0;
+  X.ks = A.ks;
   X.tbase = read_ticket<T>(A.sync);  // before the first barrier: no block has drawn yet
   const int ntiles = G.tilesX * G.tilesY;
   const size_t ndof = (size_t)G.Nx * G.Ny * NN;
@@ -1681,7 +1845,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
   } else {
     T rrb = T(0), bbb = T(0);
     for (int t = X.vrank; t < ntiles; t += X.vsize) {
-      cg_tile_apply<T, N>(
+      solve_apply<T, N>(
           C, G, t, X,
           [&](size_t g, int k, bool interior) {
             double v = 0.0;
@@ -1691,7 +1855,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
             if (interior) __stcg(A.v.y + g, tv);
             return tv;
           },
-          [&](size_t g, int k, T, T qv) {
+          [&](size_t g, int k, T qv) {
             const T b = rhs_at<T, N>(C, RhsSource<T>{A.omega, A.rhs, wbar}, g, k);
             const T r = b - qv;
             __stcg(A.v.r + g, r);
@@ -1795,6 +1959,7 @@ struct MixedArgs {
   // (too inexact on this problem's smoothest modes), double-float from then on
   int precise_apply;
   int keep_mean;       // homogeneous Dirichlet: b = sqrt(W) omega (no mean removed)
+  FxScale ks;          // factors of the fixed-point operator (float64 residuals)
 };
 
 // The operator tables a mixed solve stages in shared memory: float64 (residuals), float32
@@ -1806,10 +1971,10 @@ __host__ __device__ constexpr size_t mixed_ops_bytes() {
 
 template <int N>
 __host__ __device__ constexpr size_t mixed_smem_bytes(int TY, int TX, int Lmax, int kind, bool pow2) {
-  return (kind == kPrecondTwoLevel ? align16(sizeof(float) * N * N * N * N) : 0) +
-         align16(cg_tile_values<double, N>(TY, TX) * sizeof(double) > pc_line_bytes<float, N>(kind, Lmax, pow2)
-                     ? cg_tile_values<double, N>(TY, TX) * sizeof(double)
-                     : pc_line_bytes<float, N>(kind, Lmax, pow2));
+  size_t t = cg_tile_bytes<double, N>(TY, TX);
+  const size_t w = cg_tile_values<df, N>(TY, TX) * 8, l = pc_line_bytes<float, N>(kind, Lmax, pow2);
+  t = t > w ? t : w;
+  return (kind == kPrecondTwoLevel ? align16(sizeof(float) * N * N * N * N) : 0) + align16(t > l ? t : l);
 }
 
 // One float64 residual pass: r = b - Ahat y (y staged with halo; pass 0: y = y0), rf =
@@ -1848,7 +2013,7 @@ __device__ __forceinline__ void mixed_residual(const Ops2D<double, N>& Cd, const
   }
   const int ntiles = G.tilesX * G.tilesY;
   for (int t = X.vrank; t < ntiles; t += X.vsize) {
-    cg_tile_apply<double, N>(
+    solve_apply<double, N>(
         Cd, G, t, X,
         [&](size_t g, int k, bool interior) {
           if (!from_x0) return __ldcg(A.y + g);
@@ -1859,7 +2024,8 @@ __device__ __forceinline__ void mixed_residual(const Ops2D<double, N>& Cd, const
           if (interior) __stcg(A.y + g, v);
           return v;
         },
-        [&](size_t g, int k, double yv, double qv) {
+        [&](size_t g, int k, double qv) {
+          const double yv = __ldcg(A.y + g);
           const double b = Cd.sw[k] * (A.omega[g] - wbar);
           const double r = b - qv;
           if (A.ay) __stcg(A.ay + g, qv);
@@ -1895,6 +2061,7 @@ __device__ __forceinline__ void mixed_solve(const Ops2D<double, N>& Cd, const Op
   Xd.sync = A.sync;
   Xd.part = A.partd;
   Xd.phase = 0;
+  Xd.ks = A.ks;
   Xf.tbase = Xd.tbase = read_ticket<float>(A.sync);  // before the first barrier
   const size_t ndof = (size_t)G.Nx * G.Ny * NN;
   const size_t stride = (size_t)Xd.vsize * blockDim.x;
@@ -2064,6 +2231,7 @@ struct BatchSim {
   double D, dt, tol2, tol_in2, floor2;
   int maxit, max_sweeps, fixed_iters;
   double sumW;
+  FxScale ks;
   // float64 solve
   double *r, *p0v, *p1v, *q, *part;
   // mixed solve
@@ -2173,6 +2341,7 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     A.maxit = S.fixed_iters > 0 ? max(S.maxit, S.fixed_iters) : S.maxit;
     A.fixed_iters = S.fixed_iters;
     A.sumW = S.sumW;
+    A.ks = S.ks;
     SolveCtx<double> X;
     init_ctx<double, N>(X, smem, S.Gc, S.pc.Bt, pc, Lmax);
     X.red = redd;
@@ -2208,6 +2377,7 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     A.max_sweeps = S.max_sweeps;
     A.maxit_in = S.maxit;
     A.sumW = S.sumW;
+    A.ks = S.ks;
     A.precise_apply = S.precise_apply;
     SolveCtx<float> Xf;
     init_ctx<float, N>(Xf, smem, S.Gc, S.pcf.Bt, pc, Lmax);

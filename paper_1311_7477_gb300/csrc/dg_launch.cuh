@@ -18,12 +18,13 @@ int launch_rhs(const dg_grid* g, const RhsArgs& A, cudaStream_t st) {
   return DG_OK;
 }
 
-template <typename T, int N>
+template <int N>
 int launch_apply(const dg_grid* g, const double* x, double* y, int mode, cudaStream_t st) {
   const Geom G = geom_of(g, g->cTY, g->cTX);
-  const size_t smem = table_bytes<Ops2D<T, N>>() + apply_smem_values<T, N>(G.TY, G.TX) * sizeof(T);
-  if (int rc = set_smem(apply_kernel<T, N>, smem)) return rc;
-  apply_kernel<T, N><<<G.tilesX * G.tilesY, kThreads, smem, st>>>(ops_of<T, N>(g), G, x, y, mode);
+  const size_t smem = fx_apply_bytes<N>(G.TY, G.TX);
+  auto kern = mode == 0 ? apply_kernel<N, false> : apply_kernel<N, true>;
+  if (int rc = set_smem(kern, smem)) return rc;
+  kern<<<G.tilesX * G.tilesY, kThreads, smem, st>>>(ops_of<double, N>(g), g->ks, G, x, y);
   CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
@@ -83,6 +84,7 @@ int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_
   int grid = std::min(per_sm * g->num_sms, G.tilesX * G.tilesY);
   grid = std::min(grid, w.grid_cap);
   A.part = reinterpret_cast<T*>(w.part);
+  A.ks = g->ks;
   A.sync = w.sync;
   A.status = w.status;
   if constexpr (std::is_same<TP, double>::value)
@@ -134,6 +136,7 @@ int launch_mixed(const dg_grid* g, MixedArgs A, const Workspace& w, cudaStream_t
   A.v = CgVectors<float>{w.fe, w.fr, w.fp0, w.fp1, w.fq};
   A.pc = pc_args_f(g, w);
   A.partd = w.part;
+  A.ks = g->ks;
   A.partf = w.partf;
   A.sync = w.sync;
   A.status = w.status;
@@ -187,7 +190,7 @@ int launch_scale(const dg_grid* g, const double* x, double* y, int inverse, cuda
 #define DGK_INSTANTIATE_LAUNCHERS(N)                                                                           \
   namespace dgk {                                                                                             \
   template int launch_rhs<N>(const dg_grid*, const RhsArgs&, cudaStream_t);                                   \
-  template int launch_apply<double, N>(const dg_grid*, const double*, double*, int, cudaStream_t);            \
+  template int launch_apply<N>(const dg_grid*, const double*, double*, int, cudaStream_t);                    \
   template int launch_cg<double, N, double>(const dg_grid*, CgArgs<double, double>, const Workspace&,         \
                                             cudaStream_t, dg_sim*);                                           \
   template int launch_cg<double, N, float>(const dg_grid*, CgArgs<double, float>, const Workspace&,           \
