@@ -43,7 +43,10 @@ def _headers():
 
 
 def _compile(src, obj, verbose, ptxas_verbose):
-    cmd = [_nvcc()] + ARCH + NVCC_FLAGS + ["-c", src, "-o", obj]
+    # the batched kernel calls device functions of other units: relocatable, 128 registers (two
+    # blocks of 256 threads per SM)
+    batch = ["-rdc=true", "-maxrregcount=128"] if os.path.basename(src).startswith("dg_batch") else []
+    cmd = [_nvcc()] + ARCH + NVCC_FLAGS + batch + ["-c", src, "-o", obj]
     if ptxas_verbose and src.endswith(".cu"):
         cmd += ["-Xptxas", "-v"]
     p = subprocess.run(cmd, capture_output=True, text=True)

@@ -3,10 +3,15 @@
 
 namespace dgk {
 
+// One step of a simulation on a group of blocks, compiled per n (dg_batch_n<N>.cu, in parallel).
+template <int N>
+__device__ bool batch_step_n(BatchSim* S, const BatchGroup& grp, int vrank, unsigned char* smem, double* redd, float* redf,
+                             BarrierState* bs);
+
 __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__ BatchArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[96];
-  __shared__ float redf[96];
+  __shared__ double redd[112];
+  __shared__ float redf[128];
   __shared__ BarrierState bs;
   if (threadIdx.x == 0) bs = BarrierState{0, 0};
   int gi = 0;
@@ -18,11 +23,11 @@ __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__
     for (int j = 0; j < grp.count && ok; ++j) {
       BatchSim* S = A.sims + A.order[grp.first + j];
       switch (S->n) {
-        case 1: ok = batch_step<1>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
-        case 2: ok = batch_step<2>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
-        case 3: ok = batch_step<3>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
-        case 4: ok = batch_step<4>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
-        case 5: ok = batch_step<5>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 1: ok = batch_step_n<1>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 2: ok = batch_step_n<2>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 3: ok = batch_step_n<3>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 4: ok = batch_step_n<4>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
+        case 5: ok = batch_step_n<5>(S, grp, vrank, smem_raw, redd, redf, &bs); break;
         default: ok = false;
       }
     }

@@ -1,0 +1,4 @@
+// The batched step for n = 4 nodes per cell and dimension.
+#include "dg_batch_step.cuh"
+
+DGK_INSTANTIATE_BATCH(4)

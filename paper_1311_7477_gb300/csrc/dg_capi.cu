@@ -119,6 +119,7 @@ void free_ws(Workspace& w) {
   cudaFree(w.pCf);
   cudaFree(w.pS);
   cudaFree(w.pSf);
+  cudaFree(w.pE);
   if (w.host_out) cudaFreeHost(w.host_out);
   w = Workspace{};
 }
@@ -132,7 +133,7 @@ int alloc_ws(Workspace& w, size_t ndof, int grid_cap, bool with_y) {
   CUDA_TRY(cudaMalloc(&w.p1, bytes));
   CUDA_TRY(cudaMalloc(&w.q, bytes));
   if (with_y) CUDA_TRY(cudaMalloc(&w.y, bytes));
-  CUDA_TRY(cudaMalloc(&w.part, 6 * (size_t)grid_cap * sizeof(double)));
+  CUDA_TRY(cudaMalloc(&w.part, 8 * (size_t)grid_cap * sizeof(double)));
   CUDA_TRY(cudaMalloc(&w.sync, sizeof(SyncState)));
   CUDA_TRY(cudaMalloc(&w.status, sizeof(SolveStatus)));
   CUDA_TRY(cudaMemset(w.sync, 0, sizeof(SyncState)));
@@ -154,6 +155,7 @@ int alloc_ws_precond(Workspace& w, int Nx, int Ny, int n, bool mixed) {
   CUDA_TRY(cudaMalloc(&w.puc, ncell * sizeof(double)));
   CUDA_TRY(cudaMalloc(&w.pC, ncell * sizeof(Cplx<double>)));
   CUDA_TRY(cudaMalloc(&w.pS, nspec * sizeof(Cplx<double>)));
+  CUDA_TRY(cudaMalloc(&w.pE, ((size_t)(Nx / 2 + 1) + (Ny + 1) / 2) * n * sizeof(int2)));
   if (mixed) {
     CUDA_TRY(cudaMalloc(&w.pzf, w.ndof * sizeof(float)));
     CUDA_TRY(cudaMalloc(&w.prcf, ncell * sizeof(float)));
@@ -172,7 +174,7 @@ int alloc_ws_mixed(Workspace& w) {
   CUDA_TRY(cudaMalloc(&w.fp0, fb));
   CUDA_TRY(cudaMalloc(&w.fp1, fb));
   CUDA_TRY(cudaMalloc(&w.fq, fb));
-  CUDA_TRY(cudaMalloc(&w.partf, 6 * (size_t)w.grid_cap * sizeof(float)));
+  CUDA_TRY(cudaMalloc(&w.partf, 8 * (size_t)w.grid_cap * sizeof(float)));
   return DG_OK;
 }
 
@@ -339,6 +341,10 @@ void free_pc(PcTables& t) {
   cudaFree(t.Vyf);
   cudaFree(t.lxf);
   cudaFree(t.lyf);
+  cudaFree(t.fVx);
+  cudaFree(t.fVy);
+  cudaFree(t.ftwx);
+  cudaFree(t.ftwy);
   t = PcTables{};
 }
 
@@ -452,7 +458,7 @@ int build_spectral(dg_grid* g) {
   const Ops2D<double, N>& O = *reinterpret_cast<const Ops2D<double, N>*>(g->ops.d);
   PcTables& P = g->pc;
   auto line = [&](const Op1D<double, N>& o, int Nc, int kcount, Cplx<double>** V, double** lam, Cplx<float>** Vf,
-                  float** lamf) {
+                  float** lamf, Cfx** fV, Cfx** ftw, double* lmin) {
     std::vector<Cplx<double>> vh((size_t)kcount * N * N);
     std::vector<Cplx<float>> vf((size_t)kcount * N * N);
     std::vector<double> lh((size_t)kcount * N);
@@ -465,15 +471,44 @@ int build_spectral(dg_grid* g) {
       }
       for (int i = 0; i < N; ++i) lh[(size_t)k * N + i] = l[i];
     }
+    if (lmin) {
+      lmin[0] = lmin[1] = HUGE_VAL;
+      for (double l : lh) {
+        lmin[0] = std::min(lmin[0], l);
+        if (l != 0.0) lmin[1] = std::min(lmin[1], l);
+      }
+      if (lmin[1] == HUGE_VAL) lmin[1] = 1.0;
+    }
     CUDA_TRY(cudaMalloc(V, vh.size() * sizeof(Cplx<double>)));
     CUDA_TRY(cudaMemcpy(*V, vh.data(), vh.size() * sizeof(Cplx<double>), cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMalloc(Vf, vf.size() * sizeof(Cplx<float>)));
     CUDA_TRY(cudaMemcpy(*Vf, vf.data(), vf.size() * sizeof(Cplx<float>), cudaMemcpyHostToDevice));
+    if (fV) {  // fixed point, with the line's twiddles exp(-2 pi i m / Nc)
+      std::vector<Cfx> vx(vh.size()), tw(Nc);
+      for (int k = 0; k < kcount; ++k)  // entry by entry, the wave numbers innermost
+        for (int i = 0; i < N * N; ++i) {
+          const Cplx<double> v = vh[(size_t)k * N * N + i];
+          vx[(size_t)i * kcount + k] = Cfx{fx_coef(v.re, 60), fx_coef(v.im, 60)};
+        }
+      for (int m = 0; m < Nc; ++m) {
+        const long double ang = 2.0L * 3.141592653589793238462643383279502884L * m / Nc;
+        // units of 2^-62, split at 32 bits (the low word signed)
+        auto words = [](long double v) {
+          const long long w = llrintl(std::ldexp(v, 62));
+          return fx{int((w + (1ll << 31)) >> 32), int(unsigned(w))};
+        };
+        tw[m] = Cfx{words(std::cos(ang)), words(-std::sin(ang))};
+      }
+      if (int rc = upload(fV, vx)) return rc;
+      if (int rc = upload(ftw, tw)) return rc;
+    }
     if (int rc = upload(lam, lh)) return rc;
     return upload(lamf, lh);
   };
-  if (int rc = line(O.kx, g->Nx, g->Nx / 2 + 1, &P.Vx, &P.lx, &P.Vxf, &P.lxf)) return rc;
-  return line(O.ky, g->Ny, g->Ny, &P.Vy, &P.ly, &P.Vyf, &P.lyf);
+  const bool fixed = P.log2x >= 0 && P.log2y >= 0;
+  if (int rc = line(O.kx, g->Nx, g->Nx / 2 + 1, &P.Vx, &P.lx, &P.Vxf, &P.lxf, fixed ? &P.fVx : nullptr, &P.ftwx, nullptr))
+    return rc;
+  return line(O.ky, g->Ny, g->Ny, &P.Vy, &P.ly, &P.Vyf, &P.lyf, fixed ? &P.fVy : nullptr, &P.ftwy, P.lymin);
 }
 
 // The cell block A_cc = W_y (x) A1_cc/hx + A1_cc/hy (x) W_x (node index a*n + b), its inverse
@@ -1513,7 +1548,7 @@ struct StaticScratch {
   double p0[kStaticMaxDof];
   double p1[kStaticMaxDof];
   double q[kStaticMaxDof];
-  double part[6 * kStaticMaxBlocks];
+  double part[8 * kStaticMaxBlocks];
   SyncState sync;
   SolveStatus status;
   alignas(16) unsigned char tab[kFxTabBytes];  // fixed-point tables of a grid with a jump penalty

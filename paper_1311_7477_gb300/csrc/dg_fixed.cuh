@@ -31,6 +31,10 @@ struct fx {
   int h, l;
 };
 
+struct Cfx {
+  fx re, im;
+};
+
 struct FxAcc {
   long long a1 = 0, a0 = 0;
 };
@@ -76,8 +80,8 @@ __host__ __device__ __forceinline__ long long fx_from_bits(unsigned hi, unsigned
   return int(hi) < 0 ? -x : x;
 }
 
-// An integer as a float64, rounded to nearest (halves away from zero).
-__host__ __device__ __forceinline__ double fx_to_double(long long y) {
+// y 2^e as a float64, rounded to nearest (halves away from zero); the result is a normal number.
+__host__ __device__ __forceinline__ double fx_to_double(long long y, int e = 0) {
   const long long s = y >> 63;
   unsigned long long v = (unsigned long long)((y ^ s) - s);
 #ifdef __CUDA_ARCH__
@@ -89,7 +93,7 @@ __host__ __device__ __forceinline__ double fx_to_double(long long y) {
   v = (v << lz);
   // the leading one adds to the exponent field, and a carry out of the rounding does too
   const unsigned long long r = (v >> 11) + ((v >> 10) & 1u);
-  const unsigned long long bits = ((unsigned long long)(1085 - lz) << 52) + r + ((unsigned long long)s << 63);
+  const unsigned long long bits = ((unsigned long long)(1085 - lz + e) << 52) + r + ((unsigned long long)s << 63);
 #ifdef __CUDA_ARCH__
   return __longlong_as_double((long long)bits);
 #else

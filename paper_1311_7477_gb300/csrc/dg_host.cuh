@@ -112,7 +112,7 @@ struct Workspace {
   size_t ndof = 0;
   int grid_cap = 0;  // capacity of the partials (blocks)
   double *r = nullptr, *p0 = nullptr, *p1 = nullptr, *q = nullptr, *y = nullptr;
-  double* part = nullptr;  // 6 * grid_cap
+  double* part = nullptr;  // 8 * grid_cap
   // float32 inner-solve vectors of the mixed precision path
   float *rf = nullptr, *fr = nullptr, *fe = nullptr, *fp0 = nullptr, *fp1 = nullptr, *fq = nullptr;
   float* partf = nullptr;
@@ -124,6 +124,7 @@ struct Workspace {
   // spectrum of the spectral preconditioner, (Nx/2 + 1) x Ny x n x n (float64 and float32)
   Cplx<double>* pS = nullptr;
   Cplx<float>* pSf = nullptr;
+  int2* pE = nullptr;  // scales of the fixed-point spectrum's (Nx/2 + 1) n column and (Ny/2) n row units
   SyncState* sync = nullptr;
   SolveStatus* status = nullptr;
   double* inv_part = nullptr;  // 3 * kInvBlocks
@@ -147,6 +148,9 @@ struct PcTables {
   double *lx = nullptr, *ly = nullptr;
   Cplx<float>*Vxf = nullptr, *Vyf = nullptr;
   float *lxf = nullptr, *lyf = nullptr;
+  // ... and in fixed point, with the DFTs' twiddles (power-of-two cell counts only)
+  Cfx *fVx = nullptr, *fVy = nullptr, *ftwx = nullptr, *ftwy = nullptr;
+  double lymin[2] = {0.0, 1.0};  // the smallest ly, the smallest non-zero ly
   int spectral_rc = DG_ERR_ARG;  // DG_OK once the spectral tables are built
 };
 
@@ -282,6 +286,13 @@ inline PrecondArgs<double> pc_args(const dg_grid* g, const Workspace& w) {
   P.rc = w.prc;
   P.uc = w.puc;
   P.C = w.pC;
+  P.fVx = g->pc.fVx;
+  P.fVy = g->pc.fVy;
+  P.ftwx = g->pc.ftwx;
+  P.ftwy = g->pc.ftwy;
+  P.EU = w.pE;
+  P.lymin[0] = g->pc.lymin[0];
+  P.lymin[1] = g->pc.lymin[1];
   return P;
 }
 

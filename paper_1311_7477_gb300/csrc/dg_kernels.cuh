@@ -581,10 +581,10 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
 
 template <int N, bool Gen>
 __global__ void __launch_bounds__(rhs_threads<N>(), rhs_blocks<N>()) rhs_kernel(const __grid_constant__ FxRhs<N> F,
-                                                               const __grid_constant__ Ops2D<double, N> C, const Geom G,
+                                                               const Ops2D<double, N>* __restrict__ C, const Geom G,
                                                                const __grid_constant__ RhsArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  rhs_tile<N, Gen>(F, C, G, A, blockIdx.x, smem_raw);
+  rhs_tile<N, Gen>(F, *C, G, A, blockIdx.x, smem_raw);
 }
 
 // =========================================================================================
@@ -732,17 +732,17 @@ __device__ __forceinline__ void fx_tile_apply(const Op1D<double, N>& ox, const O
 //                       mode 1  y = Delta_h x = -(lx + ly) x.
 // =========================================================================================
 template <int N, bool Lap>
-__global__ void __launch_bounds__(kThreads, 4) apply_kernel(const __grid_constant__ Ops2D<double, N> C,
+__global__ void __launch_bounds__(kThreads, 4) apply_kernel(const Ops2D<double, N>* __restrict__ C,
                                                          const FxScale S, const Geom G, const double* __restrict__ x,
                                                          double* __restrict__ y) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_sw[N * N];
   if constexpr (!Lap) {
-    if (threadIdx.x < N * N) s_sw[threadIdx.x] = C.sw[threadIdx.x];
+    if (threadIdx.x < N * N) s_sw[threadIdx.x] = C->sw[threadIdx.x];
     __syncthreads();
   }
   fx_tile_apply<N, Lap>(
-      Lap ? C.lx : C.kx, Lap ? C.ly : C.ky, S, G, blockIdx.x, smem_raw,
+      Lap ? C->lx : C->kx, Lap ? C->ly : C->ky, S, G, blockIdx.x, smem_raw,
       [&](size_t g, int k, bool) { return Lap ? x[g] : x[g] * s_sw[k]; },
       [&](size_t g, int k, double q) { y[g] = Lap ? -q : q * s_sw[k]; });
 }
@@ -834,6 +834,11 @@ struct PrecondArgs {
   const Cplx<T>* Vy;    // Vy[ky][a][i], ky < Ny
   const T* ly;          // ly[ky][i]
   Cplx<T>* S;           // spectrum, (Nx/2 + 1) x Ny x N x N
+  // fixed-point spectral path (float64, power-of-two cell counts; null elsewhere): the same tables
+  // in units of 2^-60, and the units' scales {top, exponent}: |value| < 2^top, value = integer 2^exponent
+  const Cfx *fVx, *fVy, *ftwx, *ftwy;
+  int2* EU;
+  double lymin[2];      // the smallest ly, the smallest non-zero ly
 };
 
 // Shared memory and synchronisation of one persistent solve.
@@ -846,7 +851,7 @@ struct SolveCtx {
   T* red;
   BarrierState* bs;
   SyncState* sync;
-  T* part;                        // 6 * vsize: two alternating halves of up to 3 sums
+  T* part;                        // 8 * vsize: two alternating halves of up to 3 sums and a magnitude
   int phase;
   unsigned int tbase;             // first ticket of the next dynamically scheduled phase
   int vrank, vsize;               // this block's rank and the block count of the (virtual) grid
@@ -896,10 +901,12 @@ __device__ __forceinline__ unsigned int read_ticket(const SyncState* s) {
 }
 
 // Block partials of K sums -> grid barrier -> the sums in every block, in a fixed order that depends
-// only on the block count.  red: 32 K values.
+// only on the block count.  red: 112 values.
+// mag: also the largest magnitude word (fx_mag) of all blocks.
 template <int K, typename T>
-__device__ __forceinline__ bool reduce_sums(SolveCtx<T>& X, T (&v)[K], T (&out)[K]) {
-  T* ph = X.part + (X.phase & 1) * 3 * X.vsize;
+__device__ __forceinline__ bool reduce_sums(SolveCtx<T>& X, T (&v)[K], T (&out)[K], unsigned* mag = nullptr) {
+  T* ph = X.part + (X.phase & 1) * 4 * X.vsize;
+  unsigned* pm = reinterpret_cast<unsigned*>(ph + 3 * X.vsize);
   ++X.phase;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = int(blockDim.x >> 5);
 #pragma unroll
@@ -909,8 +916,17 @@ __device__ __forceinline__ bool reduce_sums(SolveCtx<T>& X, T (&v)[K], T (&out)[
 #pragma unroll
     for (int j = 0; j < K; ++j) X.red[32 * j + w] = v[j];
   }
+  unsigned m = 0;
+  if (mag) {
+    m = __reduce_max_sync(0xffffffffu, *mag);
+    if (lane == 0) reinterpret_cast<unsigned*>(X.red + 96)[w] = m;
+  }
   __syncthreads();
   if (w == 0) {
+    if (mag) {
+      m = __reduce_max_sync(0xffffffffu, lane < nw ? reinterpret_cast<unsigned*>(X.red + 96)[lane] : 0u);
+      if (lane == 0) __stcg(pm + X.vrank, m);
+    }
 #pragma unroll
     for (int j = 0; j < K; ++j) {
       const T t = warp_sum_down(lane < nw ? X.red[32 * j + lane] : T(0));
@@ -918,6 +934,11 @@ __device__ __forceinline__ bool reduce_sums(SolveCtx<T>& X, T (&v)[K], T (&out)[
     }
   }
   if (!solve_barrier(X)) return false;
+  if (mag) {
+    m = 0;
+    for (int i = lane; i < X.vsize; i += 32) m = max(m, __ldcg(pm + i));
+    *mag = __reduce_max_sync(0xffffffffu, m);
+  }
   if (X.vsize <= 128) {
     // few blocks: every warp adds all partials itself, without another block synchronisation
     T t[K] = {};
@@ -1427,6 +1448,474 @@ __device__ __forceinline__ void spectral_rows_inv(const Geom& G, const PrecondAr
   end_units(X, units);
 }
 
+// ---- the spectral preconditioner in fixed point (power-of-two cell counts) -------------------
+//
+// z~ = Ahat^+ r~ for float64 solves, on the integer pipe (dg_fixed.cuh): the DFTs and the n x n
+// transforms of the three phases above, which held the float64 pipe for 60% of a solve, on complex
+// 64-bit integers.  A unit's lines are one block-floating-point array: every pass ORs the
+// magnitudes of what it writes, and the next one shifts by the few bits that keep its results
+// within 2^63 (inputs below 2^60; a radix-4 butterfly grows a component at most 4 sqrt(2)).  Only
+// the twiddle products round, one unit each; a float64 butterfly rounds every sum.
+//
+// Data and twiddles split at 32 bits, x = h 2^32 + l with a signed l (the low word as it is), w in
+// units of 2^-62: w x = 4 wh xh + (wh xl + wl xh) 2^-30, three multiply-adds per real product as
+// everywhere; |x| <= 2^62.5 and |w| <= 1 keep the second accumulator below 2^63.  The n x n
+// transforms, whose rows sum ten products, keep the 30-bit split and inputs below 2^60.
+struct Cll {
+  long long re, im;
+};
+
+// Bits of a magnitude: the high word with the sign folded in (0: below 2^32).
+__device__ __forceinline__ unsigned fx_high(long long v) {
+  const int h = int(v >> 32);
+  return unsigned(h ^ (h >> 31));
+}
+__device__ __forceinline__ unsigned fx_high(const Cll& v) { return fx_high(v.re) | fx_high(v.im); }
+__device__ __forceinline__ int fx_bits(unsigned high) { return high ? 64 - __clz(high) : 32; }
+
+// v / 2^s rounded to nearest (s > 0), v 2^-s (s <= 0).
+__device__ __forceinline__ long long fx_shift(long long v, int s) {
+  if (s > 62) return 0;
+  return s > 0 ? (v + (1ll << (s - 1))) >> s : v << -s;
+}
+// (a + b) / 2^s rounded, s >= 1; the sum may pass 2^63.
+__device__ __forceinline__ long long fx_half(long long a, long long b, int s) {
+  const long long h = (a >> 1) + (b >> 1) + (a & b & 1);
+  return s > 1 ? (h + (1ll << (s - 2))) >> (s - 1) : h;
+}
+__device__ __forceinline__ Cll fx_shift(const Cll& v, int s) { return Cll{fx_shift(v.re, s), fx_shift(v.im, s)}; }
+
+__device__ __forceinline__ Cfx fx_split(const Cll& v) { return Cfx{fx_split(v.re), fx_split(v.im)}; }
+// The 32-bit split.
+__device__ __forceinline__ fx fx_words(long long y) {
+  return fx{int(y >> 32) + int(unsigned(y) >> 31), int(unsigned(y))};
+}
+
+// A complex sum of products w x (Conj: conj(w) x), rounded by get().
+struct CfxAcc {
+  FxAcc r{0, 1ll << 29}, i{0, 1ll << 29};
+  template <bool Conj>
+  __device__ __forceinline__ void mac(const Cfx& w, const Cfx& x) {
+    const fx n = fx_neg(w.im);
+    fx_mac(r, w.re, x.re);
+    fx_mac(r, Conj ? w.im : n, x.im);
+    fx_mac(i, w.re, x.im);
+    fx_mac(i, Conj ? n : w.im, x.re);
+  }
+  __device__ __forceinline__ Cll get() const { return Cll{r.a1 + (r.a0 >> 30), i.a1 + (i.a0 >> 30)}; }
+};
+
+// w x (Conj: conj(w) x) of a twiddle in the 32-bit split.
+template <bool Conj>
+__device__ __forceinline__ Cll fx_cmul(const Cfx& w, const Cll& x) {
+  const fx xr = fx_words(x.re), xi = fx_words(x.im), n = fx{-w.im.h, -w.im.l};
+  FxAcc r{0, 1ll << 29}, i{0, 1ll << 29};
+  fx_mac(r, w.re, xr);
+  fx_mac(r, Conj ? w.im : n, xi);
+  fx_mac(i, w.re, xi);
+  fx_mac(i, Conj ? n : w.im, xr);
+  return Cll{(r.a1 << 2) + (r.a0 >> 30), (i.a1 << 2) + (i.a0 >> 30)};
+}
+
+__device__ __forceinline__ Cll operator+(const Cll& a, const Cll& b) { return Cll{a.re + b.re, a.im + b.im}; }
+__device__ __forceinline__ Cll operator-(const Cll& a, const Cll& b) { return Cll{a.re - b.re, a.im - b.im}; }
+// times -i (forward) or +i (inverse)
+template <bool Inv>
+__device__ __forceinline__ Cll fx_turn(const Cll& a) {
+  return Inv ? Cll{-a.im, a.re} : Cll{a.im, -a.re};
+}
+
+__device__ __forceinline__ Cfx ld_cfx(const Cfx* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return Cfx{fx{v.x, v.y}, fx{v.z, v.w}};
+}
+__device__ __forceinline__ Cll ld_cll(const Cll* p) {
+  const longlong2 v = __ldcg(reinterpret_cast<const longlong2*>(p));
+  return Cll{v.x, v.y};
+}
+__device__ __forceinline__ void st_cll(Cll* p, const Cll& v) {
+  __stcg(reinterpret_cast<longlong2*>(p), make_longlong2(v.re, v.im));
+}
+__device__ __forceinline__ Cll lds_cll(const Cll* p) {
+  const longlong2 v = *reinterpret_cast<const longlong2*>(p);
+  return Cll{v.x, v.y};
+}
+__device__ __forceinline__ void sts_cll(Cll* p, const Cll& v) {
+  *reinterpret_cast<longlong2*>(p) = make_longlong2(v.re, v.im);
+}
+
+// v, unknown to the compiler.
+__device__ __forceinline__ int opaque(int v) {
+  asm volatile("" : "+r"(v));
+  return v;
+}
+
+// The magnitudes a block's pass wrote, ORed into s_or[slot % 3] (the slot after next is cleared for
+// the pass that will use it); call before the pass's block synchronisation.
+__device__ __forceinline__ void fx_note(unsigned* s_or, int slot, unsigned high) {
+  high = __reduce_or_sync(0xffffffffu, high);
+  if ((threadIdx.x & 31) == 0 && high) atomicOr(&s_or[slot % 3], high);
+  if (threadIdx.x == 0) s_or[(slot + 1) % 3] = 0;
+}
+
+// DFTs of `count` lines of length L = 2^log2L >= 2 in shared memory, by the whole block.  Inv ==
+// false: decimation in time (bit-reversed input, natural output); Inv == true: conjugate twiddles and
+// decimation in frequency (natural input, bit-reversed output).  slot: the s_or slot that holds
+// the input's magnitudes; it is advanced to the output's.  Returns the bits shifted out (the
+// result times 2^returned is the DFT of the input).
+template <bool Inv>
+__device__ __forceinline__ int fx_fft_lines(Cll* s, int count, int L, int log2L, const Cfx* tw, unsigned* s_or,
+                                            int& slot) {
+  const int tid = threadIdx.x, nth = blockDim.x;
+  int total = 0;
+  // the shift that brings the pass's inputs below 2^60 (up as well as down)
+  auto next_shift = [&]() {
+    const unsigned m = s_or[slot % 3];
+    int sh = m ? fx_bits(m) - 60 : 0;
+    if (sh < 0 && (total != 0 || sh > -4)) sh = 0;  // up only before the first pass, if worthwhile
+    total += sh;
+    ++slot;
+    return sh;
+  };
+  auto radix2 = [&]() {  // span 1, every twiddle 1
+    const int sh = next_shift(), hl = L >> 1;
+    unsigned high = 0;
+    for (int t = tid; t < count * hl; t += nth) {
+      Cll* b = s + (t >> (log2L - 1)) * L + 2 * (t & (hl - 1));
+      Cll u = lds_cll(b), v = lds_cll(b + 1);
+      if (sh) {
+        u = fx_shift(u, sh);
+        v = fx_shift(v, sh);
+      }
+      const Cll x = u + v, y = u - v;
+      sts_cll(b, x);
+      sts_cll(b + 1, y);
+      high |= fx_high(x) | fx_high(y);
+    }
+    fx_note(s_or, slot, high);
+    __syncthreads();
+  };
+  const int q = L >> 2;
+  auto radix4 = [&](int h, int lh) {  // spans h and 2 h
+    const int sh = next_shift(), s4 = L / (4 * h);
+    unsigned high = 0;
+    for (int t = tid; t < count * q; t += nth) {
+      const int line = t >> (log2L - 2), tt = t & (q - 1);
+      const int grp = tt >> lh, pos = tt & (h - 1);
+      Cll* b = s + line * L + grp * 4 * h + pos;
+      Cll x0 = lds_cll(b), x1 = lds_cll(b + h), x2 = lds_cll(b + 2 * h), x3 = lds_cll(b + 3 * h);
+      if (sh) {
+        x0 = fx_shift(x0, sh);
+        x1 = fx_shift(x1, sh);
+        x2 = fx_shift(x2, sh);
+        x3 = fx_shift(x3, sh);
+      }
+      Cll y0, y1, y2, y3;
+      if constexpr (!Inv) {
+        if (h > 1) {
+          x1 = fx_cmul<false>(ld_cfx(tw + 2 * pos * s4), x1);
+          x2 = fx_cmul<false>(ld_cfx(tw + pos * s4), x2);
+          x3 = fx_cmul<false>(ld_cfx(tw + 3 * pos * s4), x3);
+        }
+        const Cll s1 = x0 + x1, s2 = x0 - x1, s3 = x2 + x3, s4v = fx_turn<false>(x2 - x3);
+        y0 = s1 + s3;
+        y2 = s1 - s3;
+        y1 = s2 + s4v;
+        y3 = s2 - s4v;
+      } else {
+        const Cll u0 = x0 + x2, u1 = x1 + x3, u2 = x0 - x2, u3 = fx_turn<true>(x1 - x3);
+        y0 = u0 + u1;
+        y1 = u0 - u1;
+        y2 = u2 + u3;
+        y3 = u2 - u3;
+        if (h > 1) {
+          y1 = fx_cmul<true>(ld_cfx(tw + 2 * pos * s4), y1);
+          y2 = fx_cmul<true>(ld_cfx(tw + pos * s4), y2);
+          y3 = fx_cmul<true>(ld_cfx(tw + 3 * pos * s4), y3);
+        }
+      }
+      sts_cll(b, y0);
+      sts_cll(b + h, y1);
+      sts_cll(b + 2 * h, y2);
+      sts_cll(b + 3 * h, y3);
+      high |= fx_high(y0) | fx_high(y1) | fx_high(y2) | fx_high(y3);
+    }
+    fx_note(s_or, slot, high);
+    __syncthreads();
+  };
+  if constexpr (!Inv) {
+    int lh = 0;
+    if (log2L & 1) {
+      radix2();
+      lh = 1;
+    }
+    for (; lh < log2L; lh += 2) radix4(1 << lh, lh);
+  } else {
+    int lh = log2L - 2;
+    for (; lh >= 0; lh -= 2) radix4(1 << lh, lh);
+    if (lh == -1) radix2();
+  }
+  return total;
+}
+
+// 2^60 / m for the significand 2^52 <= m < 2^53 of a float64, times 2^52 (a value in (2^59, 2^60]):
+// a float32 reciprocal and two Newton steps in integers, correct to about 2 units.
+__device__ __forceinline__ long long fx_recip(unsigned long long m) {
+  // D = m / 2^53 in [1/2, 1) as D 2^60; r0 ~ 1 / D in (1, 2] with 24 bits, as rh 2^-29
+  const long long D = (long long)(m << 7);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(0x3f000000u | unsigned((m >> 29) & 0x7fffffu))));
+  const unsigned rb = __float_as_uint(r);
+  int rh = int(((rb & 0x7fffffu) | 0x800000u) << 6) << ((rb >> 23) - 127);  // r 2^29, r in (1, 2]
+  const fx d{int(D >> 30), int(unsigned(D) & 0x3fffffffu)};
+  // e = 1 - D r0 in units of 2^-59 (D r0 2^59 = D 2^60 rh 2^30 / 2^61 ...)
+  const long long e = (1ll << 59) - ((long long)d.h * rh + (((long long)d.l * rh) >> 30));
+  long long R = ((long long)rh << 30) + 2 * (e >> 30) * rh + (((e & 0x3fffffffll) * rh) >> 29);
+  FxAcc s;
+  fx_mac(s, d, fx{int(R >> 30), int(unsigned(R) & 0x3fffffffu)});
+  const long long e1 = (1ll << 59) - (s.a1 + (s.a0 >> 30));
+  R += (e1 * (R >> 30)) >> 29;
+  return R;  // 2^59 / D = 2^112 / m
+}
+
+// Phase 1: S[kx][cy][a][j] as in spectral_rows_fwd.  r~ has its largest magnitude's biased exponent er
+// and enters below 2^57; every unit leaves its S in a scale of its own, noted in EU[W n + unit].
+template <int N>
+__device__ __forceinline__ void fx_rows_fwd(const Geom& G, const PrecondArgs<double>& P, const double* r, int er,
+                                            SolveCtx<double>& X, unsigned* s_or) {
+  const int Nx = G.Nx, Ny = G.Ny, W = Nx / 2 + 1;
+  Cll* L0 = reinterpret_cast<Cll*>(X.line0);
+  const int units = (Ny + 1) / 2 * N;
+  for (int u = next_unit(X, units); u < units; u = next_unit(X, units)) {
+    const int pr = u / N, a = u - pr * N;
+    const int cy0 = 2 * pr, cy1 = cy0 + 1;
+    const bool hasb = cy1 < Ny;
+    if (threadIdx.x < 3) s_or[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned high = 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < Nx * N; i += blockDim.x) {
+      const int cx = i / N, b = i - cx * N;
+      const double va = __ldcg(r + (((size_t)cy0 * Nx + cx) * N + a) * N + b);
+      const double vb = hasb ? __ldcg(r + (((size_t)cy1 * Nx + cx) * N + a) * N + b) : 0.0;
+      const Cll v{fx_from_bits(__double2hiint(va), __double2loint(va), er) >> 3,
+                  fx_from_bits(__double2hiint(vb), __double2loint(vb), er) >> 3};
+      sts_cll(L0 + b * Nx + dft_slot(cx, P.log2x), v);
+      high |= fx_high(v);
+    }
+    fx_note(s_or, 0, high);
+    __syncthreads();
+    int slot = 0;
+    const int shifted = P.log2x ? fx_fft_lines<false>(L0, N, Nx, P.log2x, P.ftwx, s_or, slot) : 0;
+    // the two real rows' spectra are halves of sums: below 2^60 after this shift
+    const int sh = max(1, fx_bits(s_or[slot % 3]) + 1 - 60);
+    if (threadIdx.x == 0) {
+      const int e = er - 1079 + shifted + sh - 1;
+      P.EU[W * N + u] = make_int2(e + 62, e);  // |S| < 2^62: n values below 2^60 in a unitary transform
+    }
+#pragma unroll 1
+    for (int k = threadIdx.x; k < W; k += blockDim.x) {
+      const int km = k == 0 ? 0 : Nx - k;
+      Cfx A[N], B[N];
+#pragma unroll
+      for (int b = 0; b < N; ++b) {
+        const Cll zk = lds_cll(L0 + b * Nx + k), zm = lds_cll(L0 + b * Nx + km);
+        A[b] = fx_split(Cll{fx_half(zk.re, zm.re, sh), fx_half(zk.im, -zm.im, sh)});
+        B[b] = fx_split(Cll{fx_half(zk.im, zm.im, sh), fx_half(zm.re, -zk.re, sh)});
+      }
+      // entry (b, j) at [(b N + j) W + k]: coalesced over the threads' k (the stride is opaque, so that
+      // the addresses of all entries are not kept in registers across the loop)
+      const Cfx* V = P.fVx + k;
+      const int vs = opaque(W);
+      Cll* Sa = reinterpret_cast<Cll*>(P.S) + (((size_t)k * Ny + cy0) * N + a) * N;
+      Cll* Sb = Sa + (size_t)N * N;
+#pragma unroll 1
+      for (int j = 0; j < N; ++j) {
+        CfxAcc ta, tb;
+#pragma unroll
+        for (int b = 0; b < N; ++b) {
+          const Cfx v = ld_cfx(V + (b * N + j) * vs);
+          ta.mac<true>(v, A[b]);
+          tb.mac<true>(v, B[b]);
+        }
+        st_cll(Sa + j, ta.get());
+        if (hasb) st_cll(Sb + j, tb.get());
+      }
+    }
+    __syncthreads();
+  }
+  end_units(X, units);
+}
+
+// The largest `top` of n units' scales, in every thread.
+__device__ __forceinline__ int fx_top(const int2* EU, int n) {
+  int top = -(1 << 28);
+  for (int i = threadIdx.x & 31; i < n; i += 32) top = max(top, __ldcg(EU + i).x);
+  return __reduce_max_sync(0xffffffffu, top);
+}
+
+// Phase 2, per unit (kx, j), as in spectral_cols.  Every unit leaves its S in a scale of its own, noted
+// in P.EU.
+template <int N>
+__device__ __forceinline__ void fx_cols(const Geom& G, const PrecondArgs<double>& P, SolveCtx<double>& X,
+                                        unsigned* s_or) {
+  const int Nx = G.Nx, Ny = G.Ny, W = Nx / 2 + 1;
+  Cll* L0 = reinterpret_cast<Cll*>(X.line0);
+  const int2* E1 = P.EU + W * N;
+  const int top = fx_top(E1, (Ny + 1) / 2 * N);  // S is brought to integers below 2^60 of it
+  const int e0 = top - 60 - P.log2x - P.log2y;   // (the inverse DFTs' 1 / (Nx Ny) included)
+  for (int u = next_unit(X, W * N); u < W * N; u = next_unit(X, W * N)) {
+    const int kx = u / N, j = u - kx * N;
+    Cll* Sk = reinterpret_cast<Cll*>(P.S) + (size_t)kx * Ny * N * N;
+    if (threadIdx.x < 3) s_or[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned high = 0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < Ny * N; i += blockDim.x) {
+      const int cy = i / N, a = i - cy * N;
+      const Cll v = fx_shift(ld_cll(Sk + ((size_t)cy * N + a) * N + j), top - 60 - __ldcg(E1 + (cy >> 1) * N + a).y);
+      sts_cll(L0 + a * Ny + dft_slot(cy, P.log2y), v);
+      high |= fx_high(v);
+    }
+    fx_note(s_or, 0, high);
+    __syncthreads();
+    int slot = 0;
+    int shifted = P.log2y ? fx_fft_lines<false>(L0, N, Ny, P.log2y, P.ftwy, s_or, slot) : 0;
+    const int sh = max(0, fx_bits(s_or[slot % 3]) - 60);
+    shifted += sh;
+    ++slot;
+    // 1 / (ly + lx) in units of 2^-p: p from the smallest non-zero sum, so that the factors are <= 1
+    const double lxj = P.lx[kx * N + j];
+    const double dmin = lxj + P.lymin[lxj == 0.0 ? 1 : 0];
+    const int p = (__double2hiint(dmin) >> 20) - 1023;
+    high = 0;
+#pragma unroll 1
+    for (int ky = threadIdx.x; ky < Ny; ky += blockDim.x) {
+      const Cfx* V = P.fVy + ky;
+      const int vs = opaque(Ny);
+      Cfx x[N];
+#pragma unroll
+      for (int a = 0; a < N; ++a) x[a] = fx_split(fx_shift(lds_cll(L0 + a * Ny + ky), sh));
+#pragma unroll 1
+      for (int i = 0; i < N; ++i) {
+        CfxAcc acc;
+#pragma unroll
+        for (int a = 0; a < N; ++a) acc.mac<true>(ld_cfx(V + (a * N + i) * vs), x[a]);
+        const double den = P.ly[ky * N + i] + lxj;
+        const int hi = __double2hiint(den);
+        // 2^p / den = 2^(p - e) 2^52 / m, den = m 2^(e - 52)
+        const long long q = fx_recip((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 |
+                                     (unsigned)__double2loint(den));
+        const int d = (hi >> 20) - 1023 - p;
+        // |y| < 2^62 (its high word of the 30-bit split would not fit): halved twice
+        const Cll yq = acc.get();
+        const Cfx y = fx_split(Cll{(yq.re + 2) >> 2, (yq.im + 2) >> 2});
+        const fx f = den == 0.0 ? fx{0, 0} : fx_split(q >> min(d, 63));
+        FxAcc re{0, 1ll << 29}, im{0, 1ll << 29};
+        fx_mac(re, f, y.re);
+        fx_mac(im, f, y.im);
+        // x is in registers: t takes its place
+        const Cfx t = fx_split(Cll{re.a1 + (re.a0 >> 30), im.a1 + (im.a0 >> 30)});
+        *reinterpret_cast<int4*>(L0 + i * Ny + ky) = make_int4(t.re.h, t.re.l, t.im.h, t.im.l);
+      }
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const int4 t = *reinterpret_cast<const int4*>(L0 + i * Ny + ky);
+        x[i] = Cfx{fx{t.x, t.y}, fx{t.z, t.w}};
+      }
+#pragma unroll 1
+      for (int a = 0; a < N; ++a) {
+        CfxAcc acc;
+#pragma unroll
+        for (int i = 0; i < N; ++i) acc.mac<false>(ld_cfx(V + (a * N + i) * vs), x[i]);
+        const Cll v = acc.get();
+        sts_cll(L0 + a * Ny + ky, v);
+        high |= fx_high(v);
+      }
+    }
+    fx_note(s_or, slot, high);
+    __syncthreads();
+    if (P.log2y) shifted += fx_fft_lines<true>(L0, N, Ny, P.log2y, P.ftwy, s_or, slot);
+    if (threadIdx.x == 0) {
+      // the factors are q 2^-60 = 2^p / den: the result counts in 2^(e0 + shifted - p)
+      const unsigned m = s_or[slot % 3];
+      const int e = e0 + shifted + 2 - p;
+      P.EU[u] = make_int2(m ? e + fx_bits(m) : -(1 << 28), e);
+    }
+    for (int i = threadIdx.x; i < Ny * N; i += blockDim.x) {
+      const int cy = i / N, a = i - cy * N;
+      st_cll(Sk + ((size_t)cy * N + a) * N + j, lds_cll(L0 + a * Ny + dft_slot(cy, P.log2y)));
+    }
+    __syncthreads();
+  }
+  end_units(X, W * N);
+}
+
+// Phase 3, as in spectral_rows_inv: the units' scales are brought to one, integers below 2^60.
+template <int N>
+__device__ __forceinline__ void fx_rows_inv(const Geom& G, const PrecondArgs<double>& P, SolveCtx<double>& X,
+                                            unsigned* s_or) {
+  const int Nx = G.Nx, Ny = G.Ny, W = Nx / 2 + 1;
+  Cll* L0 = reinterpret_cast<Cll*>(X.line0);
+  const int top = fx_top(P.EU, W * N);
+  const int units = (Ny + 1) / 2 * N;
+  for (int u = next_unit(X, units); u < units; u = next_unit(X, units)) {
+    const int pr = u / N, a = u - pr * N;
+    const int cy0 = 2 * pr, cy1 = cy0 + 1;
+    const bool hasb = cy1 < Ny;
+    if (threadIdx.x < 3) s_or[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned high = 0;
+#pragma unroll 1
+    for (int k = threadIdx.x; k < W; k += blockDim.x) {
+      const Cfx* V = P.fVx + k;
+      const int vs = opaque(W);
+      const Cll* Sa = reinterpret_cast<const Cll*>(P.S) + (((size_t)k * Ny + cy0) * N + a) * N;
+      const Cll* Sb = Sa + (size_t)N * N;
+      Cfx ta[N], tb[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const int sh = top - 60 - __ldcg(P.EU + k * N + j).y;
+        ta[j] = fx_split(fx_shift(ld_cll(Sa + j), sh));
+        tb[j] = hasb ? fx_split(fx_shift(ld_cll(Sb + j), sh)) : Cfx{fx{0, 0}, fx{0, 0}};
+      }
+      const bool mirror = k > 0 && 2 * k != Nx;  // Nx - k is a distinct bin
+#pragma unroll 1
+      for (int b = 0; b < N; ++b) {
+        CfxAcc ra, rb;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+          const Cfx v = ld_cfx(V + (b * N + j) * vs);
+          ra.mac<false>(v, ta[j]);
+          rb.mac<false>(v, tb[j]);
+        }
+        const Cll A = ra.get(), B = rb.get();
+        // Z = A + i B at k; at Nx - k the spectra of the real rows are conj(A), conj(B) (|A|, |B| < 2^62)
+        const Cll z{A.re - B.im, A.im + B.re};
+        sts_cll(L0 + b * Nx + k, z);
+        high |= fx_high(z);
+        if (mirror) {
+          const Cll c{A.re + B.im, B.re - A.im};
+          sts_cll(L0 + b * Nx + Nx - k, c);
+          high |= fx_high(c);
+        }
+      }
+    }
+    fx_note(s_or, 0, high);
+    __syncthreads();
+    int slot = 0;
+    const int e = top - 60 + (P.log2x ? fx_fft_lines<true>(L0, N, Nx, P.log2x, P.ftwx, s_or, slot) : 0);
+    for (int i = threadIdx.x; i < Nx * N; i += blockDim.x) {
+      const int cx = i / N, b = i - cx * N;
+      const Cll zv = lds_cll(L0 + b * Nx + dft_slot(cx, P.log2x));
+      __stcg(P.z + (((size_t)cy0 * Nx + cx) * N + a) * N + b, fx_to_double(zv.re, e));
+      if (hasb) __stcg(P.z + (((size_t)cy1 * Nx + cx) * N + a) * N + b, fx_to_double(zv.im, e));
+    }
+    __syncthreads();
+  }
+  end_units(X, units);
+}
+
 // z~ = Ahat^+ r~ (spectral preconditioner): the three phases and the sum r~ . z~ (in every block).
 template <typename TP, int N, typename TR>
 __device__ __forceinline__ bool pc_spectral(const Geom& G, const PrecondArgs<TP>& P, const TR* r, SolveCtx<TR>& X,
@@ -1561,7 +2050,7 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
           C, G, t, X,
           [&](size_t g, int k, bool interior) {
             const T zv = spec ? T(__ldcg(P->z + g))
-                         : P  ? fma(C.sw[k], T(__ldcg(P->uc + g / NN)), T(__ldcg(P->z + g)))
+                         : P  ? fma(C.sw[k], T(__ldcg(P->uc + unsigned(g) / NN)), T(__ldcg(P->z + g)))
                               : __ldcg(V.r + g);
             const T pv = first ? zv : fma(beta, __ldcg(pin + g), zv);
             if (interior) __stcg(pout + g, pv);
@@ -1662,6 +2151,103 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
   return it;
 }
 
+// The solve proper with the spectral preconditioner in fixed point: M^-1 = Ahat^+ makes the first CG
+// step length 1 up to rounding, so the iteration is y <- y + Ahat^+ r with the true residual
+// r = b - Ahat y after every step -- the stopping rule of cg_iterate, without the second operator
+// application, the dot products and the vector updates that find a step length of 1.  y starts in
+// V.p0 and ends in V.y; r, rr, mag (its largest magnitude word) belong to it, `fresh` says that they
+// were evaluated by the operator (not recycled).  Returns the number of preconditioner
+// applications; raises flags.
+template <int N>
+__device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, const Geom& G, const CgVectors<double>& V,
+                                                   const PrecondArgs<double>& P, const RhsSource<double>& Bsrc,
+                                                   SolveCtx<double>& X, double& rr, double rhob, unsigned mag,
+                                                   bool fresh, double tol2, int maxit, int& flags, double floor2,
+                                                   double* ay) {
+  __shared__ unsigned s_or[3];
+  const int ntiles = G.tilesX * G.tilesY;
+  const size_t ndof = (size_t)G.Nx * G.Ny * N * N;
+  double *yin = V.p0, *yout = V.y;
+  double yy = 0.0, rr_prev = -1.0;
+  int it = 0;
+  while (true) {
+    const bool met = rr <= tol2 * rhob;
+    if (fresh) {
+      if (met || rr == 0.0) break;
+      // stagnation at the float64 rounding floor of y (see CgArgs::floor2)
+      if (rr <= floor2 * yy && rr_prev >= 0.0 && rr > 0.25 * rr_prev) break;
+      rr_prev = rr;
+      if (it >= maxit || it > kMaxRestarts) {
+        flags |= kFlagNoconv;
+        break;
+      }
+    }
+    const bool step = !met;
+    const int er = int(mag >> 20);
+    if (step) {
+      // a finite non-zero rr bounds the largest residual by 2^+-537: every scale below is a normal number
+      if (!(rr <= 1.7976931348623157e308)) {
+        flags |= kFlagBreakdown;
+        break;
+      }
+      fx_rows_fwd<N>(G, P, V.r, er, X, s_or);
+      bool ok = solve_barrier(X);
+      if (ok) {
+        fx_cols<N>(G, P, X, s_or);
+        ok = solve_barrier(X);
+      }
+      if (ok) {
+        fx_rows_inv<N>(G, P, X, s_or);
+        ok = solve_barrier(X);
+      }
+      if (!ok) {
+        flags |= kFlagTimeout;
+        return it;
+      }
+      ++it;
+    }
+    double rt = 0.0, yt = 0.0;
+    mag = 0;
+    for (int t = X.vrank; t < ntiles; t += X.vsize) {
+      solve_apply<double, N>(
+          C, G, t, X,
+          [&](size_t g, int, bool interior) {
+            double y = __ldcg(yin + g);
+            if (step) y += __ldcg(P.z + g);
+            if (interior) {
+              __stcg(yout + g, y);
+              yt = fma(y, y, yt);
+            }
+            return y;
+          },
+          [&](size_t g, int k, double q) {
+            const double r = rhs_at<double, N>(C, Bsrc, g, k) - q;
+            __stcg(V.r + g, r);
+            if (ay) __stcg(ay + g, q);
+            rt = fma(r, r, rt);
+            mag = max(mag, fx_mag(r));
+          });
+    }
+    double v[2] = {rt, yt}, o[2];
+    if (!reduce_sums<2>(X, v, o, &mag)) {
+      flags |= kFlagTimeout;
+      return it;
+    }
+    rr = o[0];
+    yy = o[1];
+    fresh = true;
+    double* const t = yin;
+    yin = yout;
+    yout = t;
+  }
+  if (yin != V.y) {  // the last iterate is the other buffer
+    strided_pass<4>((size_t)X.vrank * blockDim.x + threadIdx.x, ndof, (size_t)X.vsize * blockDim.x,
+                    [&](size_t i) { return __ldcg(yin + i); }, [&](size_t i, double y) { __stcg(V.y + i, y); });
+    if (!solve_barrier(X)) flags |= kFlagTimeout;
+  }
+  return it;
+}
+
 // Removes the W-mean of psi = y / sqrt(W) from y (y -= m sqrt(W)): a preconditioner other
 // than W^-1 moves the iterates along the constants, the kernel of A.
 template <typename T, int N>
@@ -1673,12 +2259,12 @@ __device__ __forceinline__ bool project_mean(const Ops2D<T, N>& C, const Geom& G
   const size_t first = (size_t)X.vrank * blockDim.x + threadIdx.x;
   T s = T(0);
   strided_pass<4>(first, ndof, stride, [&](size_t i) { return __ldcg(y + i); },
-                  [&](size_t i, T v) { s = fma(C.sw[i % NN], v, s); });
+                  [&](size_t i, T v) { s = fma(C.sw[unsigned(i) % NN], v, s); });
   T m = T(0);
   if (!reduce_all(X, s, m)) return false;
   m = m / T(sumW);
   strided_pass<4>(first, ndof, stride, [&](size_t i) { return __ldcg(y + i); },
-                  [&](size_t i, T v) { __stcg(y + i, fma(-m, C.sw[i % NN], v)); });
+                  [&](size_t i, T v) { __stcg(y + i, fma(-m, C.sw[unsigned(i) % NN], v)); });
   return solve_barrier(X);
 }
 
@@ -1701,7 +2287,7 @@ struct CgArgs {
   int precond;          // kPrecondJacobi (W^-1: plain CG on the scaled system), kPrecondTwoLevel or kPrecondSpectral
   PrecondArgs<TP> pc;   // (TP = float: the preconditioner applied in float32)
   double* psi_out;      // if non-null: psi = y / sqrt(W) at the end
-  T* part;              // 6 * gridDim.x
+  T* part;              // 8 * gridDim.x
   SyncState* sync;
   SolveStatus* status;
   double tol2;
@@ -1782,8 +2368,15 @@ __device__ __forceinline__ void init_ctx(SolveCtx<T>& X, unsigned char* base, co
   __syncthreads();
 }
 
-// The whole Poisson solve on the (virtual) grid of X (context laid out by init_ctx).
-template <typename T, int N, typename TP = T>
+// Whether a float64 solve takes the fixed-point spectral path: the spectral preconditioner with its
+// fixed-point tables (power-of-two cell counts), run to a tolerance.
+__host__ __device__ __forceinline__ bool fx_spectral_solve(const PrecondArgs<double>& P, int precond, int fixed_iters) {
+  return precond == kPrecondSpectral && P.fVx && fixed_iters == 0;
+}
+
+// The whole Poisson solve on the (virtual) grid of X (context laid out by init_ctx).  Fxs: the
+// fixed-point spectral path (fx_spectral_solve), else CG.
+template <typename T, int N, typename TP = T, bool Fxs = false>
 __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, const CgArgs<T, TP>& A,
                                          SolveCtx<T>& X) {
   constexpr int NN = N * N;
@@ -1799,6 +2392,17 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
   int flags = 0, it = 0;
   T rr = T(0), rhob = T(0), rz = T(0);
 
+  // the fixed-point spectral path starts from y0 in p0
+  T* const y0v = Fxs ? A.v.p0 : A.v.y;
+  unsigned mag = 0;
+  auto reduce_rr = [&](T a, T b) {
+    T v[2] = {a, b}, o[2];
+    if (!reduce_sums<2>(X, v, o, Fxs ? &mag : nullptr)) return false;
+    rr = o[0];
+    rhob = o[1];
+    return true;
+  };
+
   // P0: W-mean of omega, in two passes (the second removes the rounding left by the first,
   // so that b carries no rounding-sized component along the kernel of A).
   T wbar = T(0);
@@ -1807,7 +2411,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
       T s = T(0);
       strided_pass<4>((size_t)X.vrank * blockDim.x + threadIdx.x, ndof, stride,
                       [&](size_t i) { return T(A.omega[i]); },
-                      [&](size_t i, T v) { s = fma(C.wq[i % NN], v - wbar, s); });
+                      [&](size_t i, T v) { s = fma(C.wq[unsigned(i) % NN], v - wbar, s); });
       T m = T(0);
       if (!reduce_all(X, s, m)) {
         flags |= kFlagTimeout;
@@ -1821,7 +2425,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
     T rrb = T(0), bbb = T(0);
     const RhsSource<T> src{A.omega, A.rhs, wbar};
     for (size_t g = (size_t)X.vrank * blockDim.x + threadIdx.x; g < ndof; g += stride) {
-      const int k = int(g % NN);
+      const int k = int(unsigned(g) % NN);
       T y0 = T(0), ax = T(0);
       if (A.xa) {
         y0 = T(A.ca) * T(A.xa[g]);
@@ -1831,14 +2435,15 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
         y0 = fma(T(A.cb), T(A.xb[g]), y0);
         ax = fma(T(A.cb), __ldcg(A.axb + g), ax);
       }
-      __stcg(A.v.y + g, y0);
+      __stcg(y0v + g, y0);
       const T b = rhs_at<T, N>(C, src, g, k);
       const T r = b - ax;
       __stcg(A.v.r + g, r);
       rrb = fma(r, r, rrb);
+      if constexpr (Fxs) mag = max(mag, fx_mag(r));
       bbb = fma(b, b, bbb);
     }
-    if (!reduce_all2(X, rrb, bbb, rr, rhob)) {
+    if (!reduce_rr(rrb, bbb)) {
       flags |= kFlagTimeout;
       goto finish;
     }
@@ -1852,7 +2457,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
             if (A.xa) v = A.ca * A.xa[g];
             if (A.xb) v = fma(A.cb, A.xb[g], v);
             T tv = A.x_unscaled ? T(v) * C.sw[k] : T(v);
-            if (interior) __stcg(A.v.y + g, tv);
+            if (interior) __stcg(y0v + g, tv);
             return tv;
           },
           [&](size_t g, int k, T qv) {
@@ -1860,10 +2465,11 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
             const T r = b - qv;
             __stcg(A.v.r + g, r);
             rrb = fma(r, r, rrb);
+            if constexpr (Fxs) mag = max(mag, fx_mag(r));
             bbb = fma(b, b, bbb);
           });
     }
-    if (!reduce_all2(X, rrb, bbb, rr, rhob)) {
+    if (!reduce_rr(rrb, bbb)) {
       flags |= kFlagTimeout;
       goto finish;
     }
@@ -1871,6 +2477,10 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
   if (rhob == T(0)) {
     for (size_t i = (size_t)X.vrank * blockDim.x + threadIdx.x; i < ndof; i += stride) __stcg(A.v.y + i, T(0));
     rr = T(0);
+  } else if constexpr (Fxs) {
+    it = fx_spectral_iterate<N>(C, G, A.v, A.pc, RhsSource<T>{A.omega, A.rhs, wbar}, X, rr, rhob, mag, !A.axa, A.tol2,
+                                  A.maxit, flags, A.floor2, A.ay);
+    if (!(flags & kFlagTimeout) && !project_mean<T, N>(C, G, A.v.y, A.sumW, X)) flags |= kFlagTimeout;
   } else {
     if (pc && !pc_apply<T, N, TP>(C, G, A.pc, A.v.r, X, rz)) {
       flags |= kFlagTimeout;
@@ -1884,7 +2494,7 @@ finish:
   if (A.psi_out && !(flags & kFlagTimeout)) {
     strided_pass<4>((size_t)X.vrank * blockDim.x + threadIdx.x, ndof, stride,
                     [&](size_t i) { return __ldcg(A.v.y + i); },
-                    [&](size_t i, T v) { A.psi_out[i] = double(v * C.isw[i % NN]); });
+                    [&](size_t i, T v) { A.psi_out[i] = double(v * C.isw[unsigned(i) % NN]); });
   }
   if (X.vrank == 0 && threadIdx.x == 0) {
     SolveStatus* st = A.status;
@@ -1900,15 +2510,13 @@ finish:
   }
 }
 
-// MinB: the blocks per SM the register budget is sized for.  The solves with the spectral
-// preconditioner are launched with MinB = 2 (up to 128 registers a thread: its V transforms
-// keep n complex values per row in registers, and its line buffers allow two blocks per SM on
-// large grids anyway).
-template <typename T, int N, typename TP = T, int MinB = (N == 5 ? 4 : 3)>
-__global__ void __launch_bounds__(kThreads, MinB) cg_kernel(const __grid_constant__ Ops2D<T, N> C, const Geom G,
+// Two blocks per SM and up to 128 registers a thread: the fixed-point operator and the spectral
+// transforms hold a line's or a wave number's n values in registers.
+template <typename T, int N, typename TP = T, bool Fxs = false>
+__global__ void __launch_bounds__(kThreads, 2) cg_kernel(const __grid_constant__ Ops2D<T, N> C, const Geom G,
                                                         const __grid_constant__ CgArgs<T, TP> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ T red[96];
+  __shared__ T red[112];
   __shared__ BarrierState bs;
   if (threadIdx.x == 0) bs = BarrierState{0, 0};
   const Ops2D<T, N>& Cs = stage_table(C, smem_raw);
@@ -1919,7 +2527,7 @@ __global__ void __launch_bounds__(kThreads, MinB) cg_kernel(const __grid_constan
   X.vrank = blockIdx.x;
   X.vsize = gridDim.x;
   X.cluster = A.cluster;
-  cg_solve<T, N, TP>(Cs, G, A, X);
+  cg_solve<T, N, TP, Fxs>(Cs, G, A, X);
 }
 
 // =========================================================================================
@@ -1945,8 +2553,8 @@ struct MixedArgs {
   CgVectors<float> v;  // inner solve: y = e, r, p0, p1, q
   int precond;         // kPrecondJacobi, kPrecondTwoLevel or kPrecondSpectral (inner float32 solve)
   PrecondArgs<float> pc;
-  double* partd;       // 6 * gridDim.x
-  float* partf;        // 6 * gridDim.x
+  double* partd;       // 8 * gridDim.x
+  float* partf;        // 8 * gridDim.x
   SyncState* sync;
   SolveStatus* status;
   double tol2, tol_in2;
@@ -1987,7 +2595,7 @@ __device__ __forceinline__ void mixed_residual(const Ops2D<double, N>& Cd, const
   if (from_x0 && A.axa) {  // Ahat y0 from the recycled products: a pointwise pass
     const size_t ndof = (size_t)G.Nx * G.Ny * NN;
     for (size_t g = (size_t)X.vrank * blockDim.x + threadIdx.x; g < ndof; g += (size_t)X.vsize * blockDim.x) {
-      const int k = int(g % NN);
+      const int k = int(unsigned(g) % NN);
       double y0 = 0.0, ax = 0.0;
       if (A.xa) {
         y0 = A.ca * A.xa[g];
@@ -2072,7 +2680,7 @@ __device__ __forceinline__ void mixed_solve(const Ops2D<double, N>& Cd, const Op
     double s = 0.0;
     strided_pass<4>((size_t)Xd.vrank * blockDim.x + threadIdx.x, ndof, stride,
                     [&](size_t i) { return A.omega[i]; },
-                    [&](size_t i, double v) { s = fma(Cd.wq[i % NN], v - wbar, s); });
+                    [&](size_t i, double v) { s = fma(Cd.wq[unsigned(i) % NN], v - wbar, s); });
     double m = 0.0;
     if (!reduce_all(Xd, s, m)) {
       flags |= kFlagTimeout;
@@ -2153,7 +2761,7 @@ finish:
   if (A.psi_out && !(flags & kFlagTimeout)) {
     strided_pass<4>((size_t)Xd.vrank * blockDim.x + threadIdx.x, ndof, stride,
                     [&](size_t i) { return __ldcg(A.y + i); },
-                    [&](size_t i, double v) { A.psi_out[i] = v * Cd.isw[i % NN]; });
+                    [&](size_t i, double v) { A.psi_out[i] = v * Cd.isw[unsigned(i) % NN]; });
   }
   if (Xd.vrank == 0 && threadIdx.x == 0) {
     SolveStatus* st = A.status;
@@ -2177,8 +2785,8 @@ __global__ void __launch_bounds__(kThreads, MinB) mixed_cg_kernel(const __grid_c
                                                            const __grid_constant__ MixedArgs A) {
   constexpr int NN = N * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double redd[96];
-  __shared__ float redf[96];
+  __shared__ double redd[112];
+  __shared__ float redf[128];
   __shared__ BarrierState bs;
   if (threadIdx.x == 0) bs = BarrierState{0, 0};
   const bool pc = A.precond == kPrecondTwoLevel;  // the cell blocks are staged
@@ -2292,7 +2900,7 @@ __host__ __device__ constexpr size_t batch_ops_bytes() {
 }
 
 template <int N>
-__device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int vrank, unsigned char* smem_all,
+__device__ __forceinline__ bool batch_step_body(BatchSim* Sp, const BatchGroup& grp, int vrank, unsigned char* smem_all,
                                            double* redd, float* redf, BarrierState* bs) {
   constexpr int NN = N * N;
   const BatchSim& S = *Sp;
@@ -2348,7 +2956,10 @@ __device__ __noinline__ bool batch_step(BatchSim* Sp, const BatchGroup& grp, int
     X.bs = bs;
     X.vrank = vrank;
     X.vsize = grp.nblocks;
-    cg_solve<double, N>(Cd, S.Gc, A, X);
+    if (fx_spectral_solve(S.pc, S.precond, S.fixed_iters))
+      cg_solve<double, N, double, true>(Cd, S.Gc, A, X);
+    else
+      cg_solve<double, N>(Cd, S.Gc, A, X);
   } else {
     MixedArgs A{};
     A.omega = S.omega[oc ^ 1];
@@ -2434,7 +3045,7 @@ __global__ void __launch_bounds__(kThreads) invariants_partial_kernel(const __gr
   __shared__ double red[32];
   double v = 0.0, e = 0.0, o = 0.0;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < ndof; i += (size_t)gridDim.x * blockDim.x) {
-    const int k = int(i % NN);
+    const int k = int(unsigned(i) % NN);
     const double w = omega[i];
     const double p = psi_scaled ? psi[i] * W.isw[k] : psi[i];
     const double ww = W.w[k] * w;
@@ -2459,7 +3070,7 @@ __global__ void scale_nodes_kernel(const __grid_constant__ NodeWeights<N> W, con
                                    double* __restrict__ y, size_t ndof, int inverse) {
   constexpr int NN = N * N;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < ndof; i += (size_t)gridDim.x * blockDim.x) {
-    const int k = int(i % NN);
+    const int k = int(unsigned(i) % NN);
     y[i] = x[i] * (inverse ? W.isw[k] : W.sw[k]);
   }
 }

@@ -13,7 +13,7 @@ int launch_rhs(const dg_grid* g, const RhsArgs& A, cudaStream_t st) {
   const bool gen = G.bc || (A.parts && A.parts != 7);
   auto kern = gen ? rhs_kernel<N, true> : rhs_kernel<N, false>;
   if (int rc = set_smem(kern, smem)) return rc;
-  kern<<<G.tilesX * G.tilesY, rhs_threads<N>(), smem, st>>>(fxrhs_of<N>(g), ops_of<double, N>(g), G, A);
+  kern<<<G.tilesX * G.tilesY, rhs_threads<N>(), smem, st>>>(fxrhs_of<N>(g), static_cast<const Ops2D<double, N>*>(g->d_opsd), G, A);
   CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
@@ -24,7 +24,7 @@ int launch_apply(const dg_grid* g, const double* x, double* y, int mode, cudaStr
   const size_t smem = fx_apply_bytes<N>(G.TY, G.TX);
   auto kern = mode == 0 ? apply_kernel<N, false> : apply_kernel<N, true>;
   if (int rc = set_smem(kern, smem)) return rc;
-  kern<<<G.tilesX * G.tilesY, kThreads, smem, st>>>(ops_of<double, N>(g), g->ks, G, x, y);
+  kern<<<G.tilesX * G.tilesY, kThreads, smem, st>>>(static_cast<const Ops2D<double, N>*>(g->d_opsd), g->ks, G, x, y);
   CUDA_TRY(cudaGetLastError());
   return DG_OK;
 }
@@ -69,17 +69,16 @@ int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_
   bool cluster = false;
   Geom G = solve_geom(g, false, &cluster);
   size_t smem = table_bytes<Ops2D<T, N>>() + cg_smem_bytes<T, N>(G.TY, G.TX, std::max(g->Nx, g->Ny), A.precond, pow2_grid(g));
+  if constexpr (std::is_same<TP, double>::value)
+    A.pc = pc_args(g, w);
+  else
+    A.pc = pc_args_f(g, w);
   auto kern = cg_kernel<T, N, TP>;
+  if constexpr (std::is_same<TP, double>::value)
+    if (fx_spectral_solve(A.pc, A.precond, A.fixed_iters)) kern = cg_kernel<T, N, TP, true>;
   if (int rc = set_smem(kern, smem)) return rc;
   int per_sm = 0;
   CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
-  if (A.precond == kPrecondSpectral && per_sm <= 2) {
-    // the spectral line buffers leave room for two blocks per SM: the variant whose register
-    // budget assumes two (no spills in the spectral transforms)
-    kern = cg_kernel<T, N, TP, 2>;
-    if (int rc = set_smem(kern, smem)) return rc;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
-  }
   if (per_sm < 1) return fail(DG_ERR_CUDA, "CG kernel does not fit on an SM (smem %zu B)", smem);
   int grid = std::min(per_sm * g->num_sms, G.tilesX * G.tilesY);
   grid = std::min(grid, w.grid_cap);
@@ -87,10 +86,6 @@ int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_
   A.ks = g->ks;
   A.sync = w.sync;
   A.status = w.status;
-  if constexpr (std::is_same<TP, double>::value)
-    A.pc = pc_args(g, w);
-  else
-    A.pc = pc_args_f(g, w);
   CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(SyncState), st));
   const bool tm = timed && timed->timing;
   if (tm)
