@@ -481,9 +481,9 @@ def main():
         ref.close()
         what = {"fp64": "float64 throughout (the headline path)",
                 "fp64pc32": "float64 throughout except the CG preconditioner, applied in float32",
-                "mixed64": "float64 bracket/viscous term/update, float32 inner PCG, float64 refinement residual",
-                "mixed": "bracket and viscous term in double-float on the float32 pipe, float32 inner PCG, "
-                         "float64 update and refinement residual"}
+                "mixed64": "as mixed",
+                "mixed": "fixed-point bracket and viscous term, float64 update; the solve by float32 inner PCG "
+                         "with float64 refinement, or by the fixed-point spectral solve where it applies"}
         for mname, mprec in (("fp64", dg.DG_FP64), ("fp64pc32", dg.DG_FP64_PC32), ("mixed64", dg.DG_MIXED64),
                              ("mixed", dg.DG_MIXED)):
             if mname == args.precision:

@@ -58,12 +58,16 @@ extern "C" {
                               /* compares against (conserves V only)                            */
 
 /* ---- precision modes ------------------------------------------------------------- */
-#define DG_FP64 0     /* everything in float64                                             */
+#define DG_FP64 0     /* float64 fields; operators and transforms in 64-bit fixed point      */
+                      /* (see dg_bracket), sums and updates in float64                      */
 #define DG_MIXED 1    /* inner CG in float32, float64 refinement and state; the bracket and  */
                       /* viscous term as in DG_FP64 (dg_bracket_mixed)                      */
-#define DG_MIXED64 2  /* the same as DG_MIXED (they differed in the bracket's arithmetic)   */
-#define DG_FP64_PC32 3 /* float64 everywhere except the CG preconditioner, applied in float32 */
+#define DG_MIXED64 2  /* the same as DG_MIXED                                               */
+#define DG_FP64_PC32 3 /* DG_FP64 with the CG preconditioner applied in float32              */
                        /* (a float32 copy of the cell block solve and the coarse DFT solve)   */
+/* With DG_PRECOND_SPECTRAL on a grid whose cell counts are powers of two a single simulation's
+ * tolerance-stopped solves take the fixed-point spectral solve of DG_FP64 in every mode: it is at
+ * least as exact and as fast as the float32 ones.                                             */
 
 typedef struct dg_grid dg_grid;
 typedef struct dg_sim dg_sim;
@@ -154,7 +158,10 @@ int dg_grid_set_tiles(dg_grid* g, int TY, int TX);
  * dg_spectral_symbol); z = A^+ r is a real 2D DFT of the n^2 node fields, n x n transforms per
  * wave vector, a division by the eigenvalue sums (the constant mode dropped) and the inverse
  * transforms.  CG then converges in one iteration in exact arithmetic (two or three in
- * floating point); the solution is returned with zero W-mean.  Its DFTs are radix-2 for cell
+ * floating point); the solution is returned with zero W-mean.  Where both cell counts are powers of
+ * two, a tolerance-stopped solve adds A^+ r to the iterate and evaluates the true residual until
+ * the tolerance is met -- CG with its step lengths, 1 up to rounding, set to 1 -- and the transforms
+ * run in 64-bit fixed point; iters counts the applications of A^+.  Its DFTs are radix-2 for cell
  * counts that are powers of two and direct sums otherwise (a side that is not a power of two
  * may have at most 256 cells).  Errors: DG_ERR_ARG (also for DG_PRECOND_TWOLEVEL and
  * DG_PRECOND_SPECTRAL on a Dirichlet grid: both use periodic DFTs; and for DG_PRECOND_SPECTRAL

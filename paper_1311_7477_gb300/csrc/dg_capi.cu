@@ -920,7 +920,10 @@ int sim_solve(dg_sim* s, const double* omega, const double* xa, double ca, const
   dg_grid* g = s->g;
   int rc;
   if (s->fixed_iters > 0) axa = axb = ay = nullptr;  // parity mode: the plain operator applications
-  if (s->precision == DG_FP64_PC32) {
+  // with the spectral preconditioner on power-of-two grids every precision takes the fixed-point
+  // solve: it is as exact as the float64 one and at least as fast as float32 sweeps
+  const bool fxs = fx_spectral_solve(pc_args(g, s->ws), g->precond, s->fixed_iters);
+  if (s->precision == DG_FP64_PC32 && !fxs) {
     CgArgs<double, float> A{};
     A.omega = omega;
     A.xa = xa;
@@ -940,7 +943,7 @@ int sim_solve(dg_sim* s, const double* omega, const double* xa, double ca, const
     A.fixed_iters = s->fixed_iters;
     A.sumW = g->Lx * g->Ly;
     rc = dispatch_n(g->n, [&](auto nc) { return launch_cg<double, decltype(nc)::value, float>(g, A, s->ws, st, s); });
-  } else if (s->precision != DG_FP64) {
+  } else if (s->precision != DG_FP64 && !fxs) {
     MixedArgs A{};
     A.omega = omega;
     A.xa = xa;

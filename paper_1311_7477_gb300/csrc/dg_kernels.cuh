@@ -551,7 +551,7 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
   const double cLx = A.visc * F.l.cx * fx_pow2(ul), cLy = A.visc * F.l.cy * fx_pow2(ul);
   const bool square = F.l.cx == F.l.cy;
   const int nin = nc * NN;
-#pragma unroll 2
+#pragma unroll 4
   for (int i = threadIdx.x; i < nin; i += blockDim.x) {
     const int c = i / NN, k = i - (i / NN) * NN;
     const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
@@ -563,6 +563,10 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
       A.omega_out[g] = J;
       continue;
     }
+    // the node's other fields, loaded before they are needed
+    const double base = A.omega_base[g];
+    const double h0 = A.nhist > 0 ? A.hist[0][g] : 0.0, h1 = A.nhist > 1 ? A.hist[1][g] : 0.0,
+                 h2 = A.nhist > 2 ? A.hist[2][g] : 0.0;
     double R = -J;
     if (viscous) {  // + D Delta_h omega, since -Delta_h = lx + ly
       const long long lx = reinterpret_cast<const long long*>(sB)[o], ly = reinterpret_cast<const long long*>(sC)[o];
@@ -572,9 +576,11 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
         R = fma(-cLx, fx_to_double(lx), fma(-cLy, fx_to_double(ly), R));
     }
     double incr = A.c_new * R;
-    for (int m = 0; m < A.nhist; ++m) incr = fma(A.c_hist[m], A.hist[m][g], incr);
+    if (A.nhist > 0) incr = fma(A.c_hist[0], h0, incr);
+    if (A.nhist > 1) incr = fma(A.c_hist[1], h1, incr);
+    if (A.nhist > 2) incr = fma(A.c_hist[2], h2, incr);
     if (A.R_out) A.R_out[g] = R;
-    A.omega_out[g] = fma(A.dt, incr, A.omega_base[g]);
+    A.omega_out[g] = fma(A.dt, incr, base);
   }
   __syncthreads();
 }
@@ -2163,15 +2169,20 @@ __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, co
                                                    const PrecondArgs<double>& P, const RhsSource<double>& Bsrc,
                                                    SolveCtx<double>& X, double& rr, double rhob, unsigned mag,
                                                    bool fresh, double tol2, int maxit, int& flags, double floor2,
-                                                   double* ay) {
+                                                   double sumW, double* ay, SolveStatus* st) {
   __shared__ unsigned s_or[3];
   const int ntiles = G.tilesX * G.tilesY;
   const size_t ndof = (size_t)G.Nx * G.Ny * N * N;
   double *yin = V.p0, *yout = V.y;
-  double yy = 0.0, rr_prev = -1.0;
+  double yy = 0.0, sy = 0.0, rr_prev = -1.0;
   int it = 0;
   while (true) {
     const bool met = rr <= tol2 * rhob;
+    if (X.vrank == 0 && threadIdx.x == 0 && it < kRefineHistory) {
+      st->hist_rr[it] = rr / rhob;
+      st->hist_it[it] = 1;
+      st->hist_len = it + 1;
+    }
     if (fresh) {
       if (met || rr == 0.0) break;
       // stagnation at the float64 rounding floor of y (see CgArgs::floor2)
@@ -2206,17 +2217,18 @@ __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, co
       }
       ++it;
     }
-    double rt = 0.0, yt = 0.0;
+    double rt = 0.0, yt = 0.0, st_ = 0.0;
     mag = 0;
     for (int t = X.vrank; t < ntiles; t += X.vsize) {
       solve_apply<double, N>(
           C, G, t, X,
-          [&](size_t g, int, bool interior) {
+          [&](size_t g, int k, bool interior) {
             double y = __ldcg(yin + g);
             if (step) y += __ldcg(P.z + g);
             if (interior) {
               __stcg(yout + g, y);
               yt = fma(y, y, yt);
+              st_ = fma(C.sw[k], y, st_);
             }
             return y;
           },
@@ -2228,21 +2240,27 @@ __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, co
             mag = max(mag, fx_mag(r));
           });
     }
-    double v[2] = {rt, yt}, o[2];
-    if (!reduce_sums<2>(X, v, o, &mag)) {
+    double v[3] = {rt, yt, st_}, o[3];
+    if (!reduce_sums<3>(X, v, o, &mag)) {
       flags |= kFlagTimeout;
       return it;
     }
     rr = o[0];
     yy = o[1];
+    sy = o[2];
     fresh = true;
     double* const t = yin;
     yin = yout;
     yout = t;
   }
-  if (yin != V.y) {  // the last iterate is the other buffer
+  // the W-mean of psi = y / sqrt(W) comes out (y -= m sqrt(W), as project_mean); the transforms drop
+  // the constant, so what is left is usually below the rounding of y and the pass is skipped
+  const double m = sy / sumW;
+  const bool project = m * m * sumW > ldexp(yy, -108);
+  if (yin != V.y || project) {
     strided_pass<4>((size_t)X.vrank * blockDim.x + threadIdx.x, ndof, (size_t)X.vsize * blockDim.x,
-                    [&](size_t i) { return __ldcg(yin + i); }, [&](size_t i, double y) { __stcg(V.y + i, y); });
+                    [&](size_t i) { return __ldcg(yin + i); },
+                    [&](size_t i, double y) { __stcg(V.y + i, project ? fma(-m, C.sw[unsigned(i) % (N * N)], y) : y); });
     if (!solve_barrier(X)) flags |= kFlagTimeout;
   }
   return it;
@@ -2432,8 +2450,14 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
         ax = T(A.ca) * __ldcg(A.axa + g);
       }
       if (A.xb) {
-        y0 = fma(T(A.cb), T(A.xb[g]), y0);
-        ax = fma(T(A.cb), __ldcg(A.axb + g), ax);
+        const T xb = T(A.xb[g]), axb = __ldcg(A.axb + g);
+        if (A.cb == -1.0 && A.xa) {  // the stepper's 2 psi^k - psi^{k-1}: one rounding
+          y0 = fma(T(A.ca), T(A.xa[g]), -xb);
+          ax = fma(T(A.ca), __ldcg(A.axa + g), -axb);
+        } else {
+          y0 = fma(T(A.cb), xb, y0);
+          ax = fma(T(A.cb), axb, ax);
+        }
       }
       __stcg(y0v + g, y0);
       const T b = rhs_at<T, N>(C, src, g, k);
@@ -2479,8 +2503,7 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
     rr = T(0);
   } else if constexpr (Fxs) {
     it = fx_spectral_iterate<N>(C, G, A.v, A.pc, RhsSource<T>{A.omega, A.rhs, wbar}, X, rr, rhob, mag, !A.axa, A.tol2,
-                                  A.maxit, flags, A.floor2, A.ay);
-    if (!(flags & kFlagTimeout) && !project_mean<T, N>(C, G, A.v.y, A.sumW, X)) flags |= kFlagTimeout;
+                                  A.maxit, flags, A.floor2, A.sumW, A.ay, A.status);
   } else {
     if (pc && !pc_apply<T, N, TP>(C, G, A.pc, A.v.r, X, rz)) {
       flags |= kFlagTimeout;
@@ -2504,14 +2527,16 @@ finish:
     st->last_flags = flags;
     st->flags |= flags;
     st->nsolves += 1;
-    st->last_sweeps = 0;
+    st->last_sweeps = Fxs ? it : 0;
     st->last_rho = double(rr);
     st->last_rhob = double(rhob);
   }
 }
 
 // Two blocks per SM and up to 128 registers a thread: the fixed-point operator and the spectral
-// transforms hold a line's or a wave number's n values in registers.
+// transforms hold a line's or a wave number's n values in registers (blocks of 384 and 512 threads with
+// 80 and 64 registers are no faster: 1024^2 cells, n = 5 4148 / 4102 / 4153 us per solve, 32^2, n = 3
+// 65 / 76 / 83).
 template <typename T, int N, typename TP = T, bool Fxs = false>
 __global__ void __launch_bounds__(kThreads, 2) cg_kernel(const __grid_constant__ Ops2D<T, N> C, const Geom G,
                                                         const __grid_constant__ CgArgs<T, TP> A) {
@@ -2864,30 +2889,72 @@ struct BatchArgs {
   int* error;                // first error flag of any group
 };
 
+// The arguments of a batched pass live in shared memory: as local variables of these functions they
+// held the registers that the passes need (a stand-alone kernel reads them from the constant bank).
 template <int N>
 __device__ __noinline__ void batch_rhs(const BatchSim& S, const FxRhs<N>& F, int oc, int p0, int r1, int r2, int rfree,
                                        int vrank, int vsize, unsigned char* smem) {
-  RhsArgs A{};
-  A.psi = S.psi[p0];
-  A.omega_in = S.omega[oc];
-  A.omega_base = S.omega[oc];
-  A.omega_out = S.omega[oc ^ 1];
-  A.R_out = S.R[rfree];
-  A.hist[0] = S.R[r1];
-  A.hist[1] = S.R[r2];
-  A.c_new = 23.0 / 12.0;
-  A.c_hist[0] = -16.0 / 12.0;
-  A.c_hist[1] = 5.0 / 12.0;
-  A.nhist = 2;
-  A.dt = S.dt;
-  A.visc = S.D;
-  A.psi_scaled = 1;
-  const int nt = S.Gr.tilesX * S.Gr.tilesY;
+  __shared__ RhsArgs A;
+  __shared__ Geom G;
+  if (threadIdx.x == 0) {
+    RhsArgs a{};
+    a.psi = S.psi[p0];
+    a.omega_in = S.omega[oc];
+    a.omega_base = S.omega[oc];
+    a.omega_out = S.omega[oc ^ 1];
+    a.R_out = S.R[rfree];
+    a.hist[0] = S.R[r1];
+    a.hist[1] = S.R[r2];
+    a.c_new = 23.0 / 12.0;
+    a.c_hist[0] = -16.0 / 12.0;
+    a.c_hist[1] = 5.0 / 12.0;
+    a.nhist = 2;
+    a.dt = S.dt;
+    a.visc = S.D;
+    a.psi_scaled = 1;
+    A = a;
+    G = S.Gr;
+  }
+  __syncthreads();
+  const int nt = G.tilesX * G.tilesY;
   const Ops2D<double, N>& C = *static_cast<const Ops2D<double, N>*>(S.ops_d);
-  if (S.Gr.bc)
-    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, true>(F, C, S.Gr, A, t, smem);
+  if (G.bc)
+    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, true>(F, C, G, A, t, smem);
   else
-    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, false>(F, C, S.Gr, A, t, smem);
+    for (int t = vrank; t < nt; t += vsize) rhs_tile<N, false>(F, C, G, A, t, smem);
+}
+
+template <int N, bool Fxs>
+__device__ __noinline__ void batch_solve(const Ops2D<double, N>& C, const Geom& G, const CgArgs<double>& A,
+                                         unsigned char* smem, double* red, BarrierState* bs, int vrank, int vsize) {
+  SolveCtx<double> X;
+  init_ctx<double, N>(X, smem, G, A.pc.Bt, A.precond == kPrecondTwoLevel, max(G.Nx, G.Ny));
+  X.red = red;
+  X.bs = bs;
+  X.vrank = vrank;
+  X.vsize = vsize;
+  cg_solve<double, N, double, Fxs>(C, G, A, X);
+}
+
+template <int N>
+__device__ __noinline__ void batch_mixed(const Ops2D<double, N>& Cd, const Ops2D<float, N>& Cf, const OpsK<df, N>& Ck,
+                                         const Geom& G, const MixedArgs& A, unsigned char* smem, double* redd,
+                                         float* redf, BarrierState* bs, int vrank, int vsize) {
+  const bool pc = A.precond == kPrecondTwoLevel;  // the cell blocks are staged
+  const int Lmax = max(G.Nx, G.Ny);
+  SolveCtx<float> Xf;
+  init_ctx<float, N>(Xf, smem, G, A.pc.Bt, pc, Lmax);
+  Xf.red = redf;
+  Xf.bs = bs;
+  Xf.vrank = vrank;
+  Xf.vsize = vsize;
+  SolveCtx<double> Xd;
+  init_ctx<double, N>(Xd, smem + (pc ? align16(sizeof(float) * N * N * N * N) : 0), G, (const double*)nullptr, false, Lmax);
+  Xd.red = redd;
+  Xd.bs = bs;
+  Xd.vrank = vrank;
+  Xd.vsize = vsize;
+  mixed_solve<N>(Cd, Cf, Ck, G, A, Xf, Xd);
 }
 
 // One AB3 step of simulation S on a group.  Returns false after a barrier timeout.
@@ -2902,7 +2969,9 @@ __host__ __device__ constexpr size_t batch_ops_bytes() {
 template <int N>
 __device__ __forceinline__ bool batch_step_body(BatchSim* Sp, const BatchGroup& grp, int vrank, unsigned char* smem_all,
                                            double* redd, float* redf, BarrierState* bs) {
-  constexpr int NN = N * N;
+  __shared__ CgArgs<double> s_cg;
+  __shared__ MixedArgs s_mixed;
+  __shared__ Geom s_g;
   const BatchSim& S = *Sp;
   // a simulation that has reached its step limit sits the step out (every block of the
   // group reads the same step index: it was written before the group's last barrier)
@@ -2917,14 +2986,9 @@ __device__ __forceinline__ bool batch_step_body(BatchSim* Sp, const BatchGroup& 
   if (!grid_barrier(grp.sync, bs, grp.nblocks)) return false;
   // the solve's tables (the barrier has synchronised the block: the RHS table is no longer read)
   const Ops2D<double, N>& Cd = stage_table(*static_cast<const Ops2D<double, N>*>(S.ops_d), smem_all);
-  const Ops2D<float, N>& Cf =
-      stage_table(*static_cast<const Ops2D<float, N>*>(S.ops_f), smem_all + table_bytes<Ops2D<double, N>>());
-  const OpsK<df, N>& Ck = stage_table(*static_cast<const OpsK<df, N>*>(S.ops_k),
-                                      smem_all + table_bytes<Ops2D<double, N>>() + table_bytes<Ops2D<float, N>>());
-  const bool pc = S.precond == kPrecondTwoLevel;  // the cell blocks are staged
-  const int Lmax = max(S.Gc.Nx, S.Gc.Ny);
   // the initial residual from the kept operator products (as in the single-simulation stepper)
   const bool rec = S.fixed_iters == 0 && __ldcg(&Sp->apsi_ok[p0]) && __ldcg(&Sp->apsi_ok[p1]);
+  const bool fxs = fx_spectral_solve(S.pc, S.precond, S.fixed_iters);
   if (S.precision == 0) {
     CgArgs<double> A{};
     A.omega = S.omega[oc ^ 1];
@@ -2950,16 +3014,15 @@ __device__ __forceinline__ bool batch_step_body(BatchSim* Sp, const BatchGroup& 
     A.fixed_iters = S.fixed_iters;
     A.sumW = S.sumW;
     A.ks = S.ks;
-    SolveCtx<double> X;
-    init_ctx<double, N>(X, smem, S.Gc, S.pc.Bt, pc, Lmax);
-    X.red = redd;
-    X.bs = bs;
-    X.vrank = vrank;
-    X.vsize = grp.nblocks;
-    if (fx_spectral_solve(S.pc, S.precond, S.fixed_iters))
-      cg_solve<double, N, double, true>(Cd, S.Gc, A, X);
+    if (threadIdx.x == 0) {
+      s_cg = A;
+      s_g = S.Gc;
+    }
+    __syncthreads();
+    if (fxs)
+      batch_solve<N, true>(Cd, s_g, s_cg, smem, redd, bs, vrank, grp.nblocks);
     else
-      cg_solve<double, N>(Cd, S.Gc, A, X);
+      batch_solve<N, false>(Cd, s_g, s_cg, smem, redd, bs, vrank, grp.nblocks);
   } else {
     MixedArgs A{};
     A.omega = S.omega[oc ^ 1];
@@ -2990,19 +3053,16 @@ __device__ __forceinline__ bool batch_step_body(BatchSim* Sp, const BatchGroup& 
     A.sumW = S.sumW;
     A.ks = S.ks;
     A.precise_apply = S.precise_apply;
-    SolveCtx<float> Xf;
-    init_ctx<float, N>(Xf, smem, S.Gc, S.pcf.Bt, pc, Lmax);
-    Xf.red = redf;
-    Xf.bs = bs;
-    Xf.vrank = vrank;
-    Xf.vsize = grp.nblocks;
-    SolveCtx<double> Xd;
-    init_ctx<double, N>(Xd, smem + (pc ? align16(sizeof(float) * NN * NN) : 0), S.Gc, (const double*)nullptr, false, Lmax);
-    Xd.red = redd;
-    Xd.bs = bs;
-    Xd.vrank = vrank;
-    Xd.vsize = grp.nblocks;
-    mixed_solve<N>(Cd, Cf, Ck, S.Gc, A, Xf, Xd);
+    const Ops2D<float, N>& Cf =
+        stage_table(*static_cast<const Ops2D<float, N>*>(S.ops_f), smem_all + table_bytes<Ops2D<double, N>>());
+    const OpsK<df, N>& Ck = stage_table(*static_cast<const OpsK<df, N>*>(S.ops_k),
+                                        smem_all + table_bytes<Ops2D<double, N>>() + table_bytes<Ops2D<float, N>>());
+    if (threadIdx.x == 0) {
+      s_mixed = A;
+      s_g = S.Gc;
+    }
+    __syncthreads();
+    batch_mixed<N>(Cd, Cf, Ck, s_g, s_mixed, smem, redd, redf, bs, vrank, grp.nblocks);
   }
   // every block has finished the solve before the rings move
   if (!grid_barrier(grp.sync, bs, grp.nblocks)) return false;
