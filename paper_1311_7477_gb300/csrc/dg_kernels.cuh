@@ -288,12 +288,13 @@ struct FxRhs {
   FxScale l;       // the Laplacian's
 };
 
-// Shared memory of one right-hand-side tile: five arrays over the box, or the float64 fallback on
-// single cells, whichever is larger.
+// Shared memory of one right-hand-side tile: five arrays over the box, or the float64 fallback's on
+// the tile (up to 72 KB, three blocks per SM) or on single cells, whichever is larger.
 template <int N>
 __host__ __device__ constexpr size_t rhs_smem_bytes(int TY, int TX) {
   const size_t a = (size_t)(TY + 2) * (TX + 2) * 5 * fx_cell<N>() * 8;
-  const size_t b = rhs_smem_values<double, N>(1, 1) * 8;
+  size_t b = rhs_smem_values<double, N>(TY, TX) * 8;
+  if (b > 72 * 1024) b = rhs_smem_values<double, N>(1, 1) * 8;
   return a > b ? a : b;
 }
 
