@@ -1,17 +1,22 @@
-"""The fixed-point right-hand side where it can go wrong: tile edges and remainders for every n,
-anisotropic cells, the parts the tables do not cover (a jump penalty), and values outside the
-fixed-point range, which the float64 tile takes.
+"""The fixed-point kernels where they can go wrong: tile edges and remainders for every n,
+anisotropic cells, the parts the tables do not cover (a jump penalty), values outside the
+fixed-point range, which the float64 tile takes; and the spectral solve on the shortest, the
+unequal and the odd-power lines of its integer DFTs.
 
 Bars: 1e-12 in relative L2 against the float64 oracle, as for the float64 evaluation: one rounding of
 2^-60 of a tile's largest value per term against the oracle's own 2^-53.  Fields are i.i.d. normal,
-so no value is more than a few bits below its tile's largest.
+so no value is more than a few bits below its tile's largest.  The spectral solve is held to the bar of
+two backward-stable solutions (test_gpu_spectral.solve_bar) and, scaled by a power of two, to the
+same bits.
 """
 import numpy as np
 import pytest
 
 from oracle.operators import Operators
+from oracle.solver import Spectral, poisson_rhs
 from oracle.tables import Grid as OGrid
 from tests.test_gpu_parity import bracket_scale, dev, host, rel_l2
+from tests.test_gpu_spectral import solve_bar
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -71,3 +76,56 @@ def test_bracket_outside_the_fixed_point_range(dg, n):
         assert np.array_equal(np.isfinite(got), np.isfinite(want))
         ok = np.isfinite(want)
         assert rel_l2(got[ok], ref[ok], scale) < 1e-12
+
+
+@pytest.mark.parametrize("Nx,Ny,n", [(1, 1, 4), (1, 4, 3), (2, 1, 5), (2, 2, 1), (8, 4, 2), (16, 8, 3), (32, 64, 4),
+                                     (128, 2, 5), (4, 256, 2), (64, 32, 5)])
+@pytest.mark.parametrize("field", ["noise", "point", "mode"])
+def test_spectral_solve(dg, Nx, Ny, n, field):
+    Lx, Ly = 1.5, 2.0
+    g = dg.Grid(Nx, Ny, n, Lx, Ly)
+    g.set_precond("spectral")
+    og = OGrid(Nx, Ny, n, Lx, Ly)
+    o = Operators(og)
+    w = np.random.default_rng(Nx + n).standard_normal(g.shape)
+    if field == "point":
+        w = np.zeros(g.shape)
+        w[Ny // 2, Nx // 2, 0, n - 1] = 1.0
+    if field == "mode":
+        X, Y = og.mesh()
+        w = np.cos(2 * np.pi * X / Lx) * np.cos(2 * np.pi * Y / Ly) + 1e-9 * w
+    ref = Spectral(o)(poisson_rhs(o, w))
+    out = []
+    for k in (0, 300, -300):
+        psi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+        rc, it, relres = dg.dg_poisson_solve(g, dev(np.ldexp(w, k)), psi, 1e-10, 50)
+        assert it <= 2 and relres <= 1e-10
+        out.append(np.ldexp(host(psi), -k))
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+    assert rel_l2(out[0], ref) < solve_bar(o, Lx, Ly)
+
+
+def test_spectral_solve_batched(dg):
+    """Float64 members with the spectral preconditioner: batched steps against the same steps alone
+    (the sums run over other block counts)."""
+    def make():
+        out = []
+        for Nx, Ny, n in ((32, 16, 3), (16, 64, 5), (8, 8, 2)):
+            g = dg.Grid(Nx, Ny, n)
+            g.set_precond("spectral")
+            X, Y = OGrid(Nx, Ny, n).mesh()
+            w = np.sin(X) * np.cos(2 * Y) + 0.3 * np.cos(X + Y)
+            out.append((g, dg.Sim(g, dev(w), D=1e-3, dt=1e-3, cg_tol=1e-11)))
+        return out
+    alone, members = make(), make()
+    b = dg.Batch(3)
+    for _, s in members:
+        b.admit(s)
+    b.step(4)
+    assert b.status()["rc"] == 0
+    for (g, s), (_, t) in zip(alone, members):
+        s.step(6)  # two start-up steps on admission, four batched
+        f = [torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(4)]
+        s.get(f[0], f[1])
+        t.get(f[2], f[3])
+        assert rel_l2(host(f[2]), host(f[0])) < 1e-11 and rel_l2(host(f[3]), host(f[1])) < 1e-10
