@@ -251,7 +251,7 @@ int dg_poisson_solve(dg_grid* g, const double* omega, double* psi, double tol, i
  * since creating one allocates.  The paper has no counterpart; this is an interface choice.
  * It takes the grid as plain parameters (Nx, Ny, n, Lx, Ly, tau as in dg_grid_create) and
  * keeps all its scratch (CG vectors, partial sums, barrier and status words) in one
- * file-scope device array of about 2.8 MB that every GPU loading the library holds until
+ * file-scope device array of about 2.9 MB that every GPU loading the library holds until
  * the process exits.  Grids are limited to Nx*Ny*n*n <= 65536 values; larger ones are
  * rejected with DG_ERR_ARG.  It calls no cudaMalloc, cudaFree or other allocating routine.
  * Every call looks up the array's device address on the current device

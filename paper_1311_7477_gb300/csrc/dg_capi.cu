@@ -1538,7 +1538,7 @@ int dg_sim_invariants(dg_sim* s, double out[3], void* stream) {
 // framework -- this entry point runs the same persistent CG kernel as dg_poisson_solve but
 // keeps every scratch vector, the per-block partial sums, the grid barrier and the status
 // word in one file-scope __device__ array of fixed size.  Each GPU that loads the library
-// holds that array (about 2.8 MB) until the process exits.
+// holds that array (about 2.9 MB) until the process exits.
 // ---------------------------------------------------------------------------------------
 namespace {
 

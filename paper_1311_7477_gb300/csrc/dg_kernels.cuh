@@ -2428,9 +2428,12 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
   if (A.rhs == nullptr && !A.keep_mean) {
     for (int pass = 0; pass < 2; ++pass) {
       T s = T(0);
-      strided_pass<4>((size_t)X.vrank * blockDim.x + threadIdx.x, ndof, stride,
-                      [&](size_t i) { return T(A.omega[i]); },
-                      [&](size_t i, T v) { s = fma(C.wq[unsigned(i) % NN], v - wbar, s); });
+      const size_t first = (size_t)X.vrank * blockDim.x + threadIdx.x;
+      auto ld = [&](size_t i) { return T(A.omega[i]); };
+      if (pass == 0)  // (the float64 pipe bounds these passes: no subtraction of 0)
+        strided_pass<4>(first, ndof, stride, ld, [&](size_t i, T v) { s = fma(C.wq[unsigned(i) % NN], v, s); });
+      else
+        strided_pass<4>(first, ndof, stride, ld, [&](size_t i, T v) { s = fma(C.wq[unsigned(i) % NN], v - wbar, s); });
       T m = T(0);
       if (!reduce_all(X, s, m)) {
         flags |= kFlagTimeout;
