@@ -344,8 +344,10 @@ __device__ __forceinline__ T sum_partials(const T* p, int G, int stride, T* bcas
 // ---- grid barrier for persistent cooperative kernels -----------------------------------
 
 struct alignas(8) SyncState {
-  unsigned int count;   // arrivals since the launch, modulo 2^32
-  int error;            // read together with count (one 64-bit load)
+  // arrivals since the launch, modulo 2^32, in the high half (a carry out of it is lost), the error
+  // in the low half.  Every access while a kernel runs is of the whole word: in the memory model a
+  // release and an acquire of different widths do not synchronise.
+  unsigned long long word;
   unsigned int ticket;  // work-unit tickets of the dynamically scheduled phases (next_unit)
   unsigned int pad;
 };
@@ -363,8 +365,8 @@ constexpr unsigned long long kSpinCap = 1ull << 23;
 
 // The nblk blocks of a (virtual) grid meet here: all blocks of a cooperative launch, or the
 // blocks of one group of a batched launch.  Returns false if any block raised an error.
-// One release-add per block on a counter that only grows, and acquire-polls of the counter itself
-// with the error word beside it: a barrier costs one trip to L2 for the add and one for the poll that sees the
+// One release-add per block on a counter that only grows, and acquire-polls of the counter and the
+// error in one word: a barrier costs one trip to L2 for the add and one for the poll that sees the
 // last arrival (a counter that the last block resets before it opens a second word cost three
 // more, and the full fences around them).
 __device__ __forceinline__ bool grid_barrier(SyncState* s, BarrierState* bs, unsigned int nblk) {
@@ -372,15 +374,15 @@ __device__ __forceinline__ bool grid_barrier(SyncState* s, BarrierState* bs, uns
   if (threadIdx.x == 0) {
     const unsigned int target = bs->target + nblk;
     bs->target = target;
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(&s->count), "r"(1u) : "memory");
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(&s->word), "l"(1ull << 32) : "memory");
     unsigned long long spins = 0, v;
     int err;
     while (true) {
-      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(s) : "memory");
-      err = int(v >> 32);
-      if (err || int(unsigned(v) - target) >= 0) break;
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&s->word) : "memory");
+      err = int(unsigned(v));
+      if (err || int(unsigned(v >> 32) - target) >= 0) break;
       if (++spins > kSpinCap) {
-        atomicCAS(&s->error, 0, kFlagTimeout);
+        atomicOr(&s->word, (unsigned long long)kFlagTimeout);
         err = kFlagTimeout;
         break;
       }
