@@ -2163,21 +2163,23 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
 // step length 1 up to rounding, so the iteration is y <- y + Ahat^+ r with the true residual
 // r = b - Ahat y after every step -- the stopping rule of cg_iterate, without the second operator
 // application, the dot products and the vector updates that find a step length of 1.  y starts in
-// V.p0 and ends in V.y; r, rr, mag (its largest magnitude word) belong to it, `fresh` says that they
-// were evaluated by the operator (not recycled).  Returns the number of preconditioner
-// applications; raises flags.
+// V.p0 and ends in V.y; r, rr, mag (its largest magnitude word) belong to it.  Whatever rr says, the
+// pass that evaluates the true residual runs at least once: it also leaves the operator product of y
+// in ay and the sums that take the W-mean out.  Returns the number of preconditioner applications;
+// raises flags.
 template <int N>
 __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, const Geom& G, const CgVectors<double>& V,
                                                    const PrecondArgs<double>& P, const RhsSource<double>& Bsrc,
                                                    SolveCtx<double>& X, double& rr, double rhob, unsigned mag,
-                                                   bool fresh, double tol2, int maxit, int& flags, double floor2,
-                                                   double sumW, double* ay, SolveStatus* st) {
+                                                   double tol2, int maxit, int& flags, double floor2, double sumW,
+                                                   double* ay, SolveStatus* st) {
   __shared__ unsigned s_or[3];
   const int ntiles = G.tilesX * G.tilesY;
   const size_t ndof = (size_t)G.Nx * G.Ny * N * N;
   double *yin = V.p0, *yout = V.y;
   double yy = 0.0, sy = 0.0, rr_prev = -1.0;
   int it = 0;
+  bool fresh = false;  // rr is the residual that the pass below evaluated
   while (true) {
     const bool met = rr <= tol2 * rhob;
     if (X.vrank == 0 && threadIdx.x == 0 && it < kRefineHistory) {
@@ -2195,7 +2197,7 @@ __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, co
         break;
       }
     }
-    const bool step = !met;
+    const bool step = !met && it < maxit;  // (maxit = 0: y0 is evaluated alone)
     const int er = int(mag >> 20);
     if (step) {
       // a finite non-zero rr bounds the largest residual by 2^+-537: every scale below is a normal number
@@ -2507,8 +2509,8 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
     for (size_t i = (size_t)X.vrank * blockDim.x + threadIdx.x; i < ndof; i += stride) __stcg(A.v.y + i, T(0));
     rr = T(0);
   } else if constexpr (Fxs) {
-    it = fx_spectral_iterate<N>(C, G, A.v, A.pc, RhsSource<T>{A.omega, A.rhs, wbar}, X, rr, rhob, mag, !A.axa, A.tol2,
-                                  A.maxit, flags, A.floor2, A.sumW, A.ay, A.status);
+    it = fx_spectral_iterate<N>(C, G, A.v, A.pc, RhsSource<T>{A.omega, A.rhs, wbar}, X, rr, rhob, mag, A.tol2,
+                                A.maxit, flags, A.floor2, A.sumW, A.ay, A.status);
   } else {
     if (pc && !pc_apply<T, N, TP>(C, G, A.pc, A.v.r, X, rz)) {
       flags |= kFlagTimeout;

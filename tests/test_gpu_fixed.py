@@ -129,3 +129,55 @@ def test_spectral_solve_batched(dg):
         s.get(f[0], f[1])
         t.get(f[2], f[3])
         assert rel_l2(host(f[2]), host(f[0])) < 1e-11 and rel_l2(host(f[3]), host(f[1])) < 1e-10
+
+
+def _steady(Nx, Ny, n):
+    X, Y = OGrid(Nx, Ny, n).mesh()
+    return 2 * np.sin(X) * np.sin(Y)
+
+
+@pytest.mark.parametrize("maxit", [0, 50])
+def test_spectral_solve_of_an_accepted_guess(dg, maxit):
+    """A guess that meets the tolerance, plus a constant: no application, and the constant goes.  The
+    mean left is that of one rounding (2^-53) of each value, here held to ten times that."""
+    Nx, Ny, n = 32, 16, 4
+    g = dg.Grid(Nx, Ny, n)
+    g.set_precond("spectral")
+    W = OGrid(Nx, Ny, n).weights()
+    w = _steady(Nx, Ny, n)
+    psi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+    dg.dg_poisson_solve(g, dev(w), psi, 1e-11)
+    good = host(psi).copy()
+    psi += 3.0
+    rc, it, relres = dg.dg_poisson_solve(g, dev(w), psi, 1e-7, maxit=maxit)
+    assert it == 0 and relres <= 1e-7
+    got = host(psi)
+    assert abs(np.sum(W * got) / np.sum(W * np.ones(g.shape))) < 10 * 2.0 ** -53 * 4
+    assert rel_l2(got, good) < 1e-14
+    # not converged and no application allowed: the guess without its mean, and the error
+    psi = dev(0.5 * good + 3.0)
+    rc, it, relres = dg.dg_poisson_solve(g, dev(w), psi, 1e-7, maxit=0, check=False)
+    assert rc == dg.DG_ERR_NOCONV and it == 0 and abs(relres - 0.5) < 1e-6
+    assert rel_l2(host(psi), 0.5 * good) < 1e-14
+
+
+def test_accepted_guess_leaves_its_operator_product(dg):
+    """Solves that accept their guess, after a state was set over unrelated fields: the next solve
+    starts from the products that these left, so one application is enough."""
+    Nx, Ny, n = 32, 32, 3
+    g = dg.Grid(Nx, Ny, n)
+    g.set_precond("spectral")
+    noise = np.random.default_rng(5).standard_normal(g.shape)
+    s = dg.Sim(g, dev(1e3 * noise), D=0.0, dt=1e-7, cg_tol=1e-10)
+    s.step(4)
+    w = _steady(Nx, Ny, n)
+    psi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+    dg.dg_poisson_solve(g, dev(w), psi, 1e-12)
+    z = dev(np.zeros(g.shape))
+    s.set_state(4, dev(w), psi, psi, z, z)
+    s.set_cg(1e-4, 100)
+    s.step(3)
+    assert s.status().cg_iters_last == 0
+    s.set_cg(1e-10, 100)
+    s.step(1)
+    assert s.status().cg_iters_last <= 1
