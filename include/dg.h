@@ -67,7 +67,8 @@ extern "C" {
                        /* (a float32 copy of the cell block solve and the coarse DFT solve)   */
 /* With DG_PRECOND_SPECTRAL on a grid whose cell counts are powers of two a single simulation's
  * tolerance-stopped solves take the fixed-point spectral solve of DG_FP64 in every mode: it is at
- * least as exact and as fast as the float32 ones.                                             */
+ * least as exact and as fast as the float32 ones.  Where its lines do not fit in shared memory (16 n
+ * max(Nx, Ny) bytes, at most about 210 KB) DG_MIXED and DG_MIXED64 keep their float32 sweeps.  */
 
 typedef struct dg_grid dg_grid;
 typedef struct dg_sim dg_sim;

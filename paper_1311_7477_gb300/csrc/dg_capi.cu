@@ -505,7 +505,15 @@ int build_spectral(dg_grid* g) {
     if (int rc = upload(lam, lh)) return rc;
     return upload(lamf, lh);
   };
-  const bool fixed = P.log2x >= 0 && P.log2y >= 0;
+  // the fixed-point solve's lines hold 16-byte values; where they do not fit beside the operator table
+  // and the static shared memory (16 KB cover both), the grid goes without its tables, and so the mixed
+  // modes without that solve: their float32 sweeps need half the room (a side of 4096 cells with n = 4
+  // or 5: 262 and 328 KB against 131 and 164)
+  int dev = 0, optin = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const size_t room = pc_line_bytes<double, N>(kPrecondSpectral, std::max(g->Nx, g->Ny), true) + 16 * 1024;
+  const bool fixed = P.log2x >= 0 && P.log2y >= 0 && room <= (size_t)optin;
   if (int rc = line(O.kx, g->Nx, g->Nx / 2 + 1, &P.Vx, &P.lx, &P.Vxf, &P.lxf, fixed ? &P.fVx : nullptr, &P.ftwx, nullptr))
     return rc;
   return line(O.ky, g->Ny, g->Ny, &P.Vy, &P.ly, &P.Vyf, &P.lyf, fixed ? &P.fVy : nullptr, &P.ftwy, P.lymin);
@@ -920,8 +928,8 @@ int sim_solve(dg_sim* s, const double* omega, const double* xa, double ca, const
   dg_grid* g = s->g;
   int rc;
   if (s->fixed_iters > 0) axa = axb = ay = nullptr;  // parity mode: the plain operator applications
-  // with the spectral preconditioner on power-of-two grids every precision takes the fixed-point
-  // solve: it is as exact as the float64 one and at least as fast as float32 sweeps
+  // with the spectral preconditioner on power-of-two grids whose lines fit (build_spectral) every
+  // precision takes the fixed-point solve: as exact as the float64 one, as fast as float32 sweeps
   const bool fxs = fx_spectral_solve(pc_args(g, s->ws), g->precond, s->fixed_iters);
   if (s->precision == DG_FP64_PC32 && !fxs) {
     CgArgs<double, float> A{};

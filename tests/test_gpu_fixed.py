@@ -13,7 +13,7 @@ import numpy as np
 import pytest
 
 from oracle.operators import Operators
-from oracle.solver import Spectral, poisson_rhs
+from oracle.solver import Spectral, poisson_rhs, rounding_floor2
 from oracle.tables import Grid as OGrid
 from tests.test_gpu_parity import bracket_scale, dev, host, rel_l2
 from tests.test_gpu_spectral import solve_bar
@@ -181,3 +181,28 @@ def test_accepted_guess_leaves_its_operator_product(dg):
     s.set_cg(1e-10, 100)
     s.step(1)
     assert s.status().cg_iters_last <= 1
+
+
+@pytest.mark.parametrize("Nx,Ny,n", [(4096, 2, 4), (1, 4096, 5)])
+@pytest.mark.parametrize("mode", ["mixed", "mixed64"])
+def test_mixed_steps_on_lines_too_long_for_the_fixed_point_solve(dg, Nx, Ny, n, mode):
+    """The mixed modes on a side whose 16-byte lines exceed shared memory: their float32 sweeps.  The
+    residual of the initial solve and of a step is measured with the oracle's operator; the bar is
+    the tolerance and the float64 rounding floor of the residual."""
+    g = dg.Grid(Nx, Ny, n)
+    g.set_precond("spectral")
+    og = OGrid(Nx, Ny, n)
+    o = Operators(og)
+    X, Y = og.mesh()
+    w = np.sin(3 * X) * np.cos(Y) + 0.3 * np.cos(5 * X + 2 * Y) + 0.2 * np.sin(7 * Y) + 0.2 * np.sin(4 * X)
+    s = dg.Sim(g, dev(w), D=0.0, dt=1e-6, precision={"mixed": dg.DG_MIXED, "mixed64": dg.DG_MIXED64}[mode], cg_tol=1e-8)
+    om, ps = (torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(2))
+    for k in range(2):
+        s.step(k)
+        assert s.status().status == 0
+        s.get(om, ps)
+        p, b = host(ps), poisson_rhs(o, host(om))
+        r = b - o.A(p)
+        norm = lambda v: np.sqrt(np.sum(v * v / o.W2))
+        floor = np.sqrt(rounding_floor2(o) * np.sum(o.W2 * p * p))
+        assert norm(r) <= 1e-8 * norm(b) + 2 * floor
