@@ -1481,6 +1481,11 @@ __device__ __forceinline__ unsigned fx_high(long long v) {
 __device__ __forceinline__ unsigned fx_high(const Cll& v) { return fx_high(v.re) | fx_high(v.im); }
 __device__ __forceinline__ int fx_bits(unsigned high) { return high ? 64 - __clz(high) : 32; }
 
+// The magnitudes of a complex value, ORed: as many bits as the larger one.
+__device__ __forceinline__ unsigned long long fx_mag64(const Cll& v) {
+  return (unsigned long long)(llabs(v.re) | llabs(v.im));
+}
+
 // v / 2^s rounded to nearest (s > 0), v 2^-s (s <= 0).
 __device__ __forceinline__ long long fx_shift(long long v, int s) {
   if (s > 62) return 0;
@@ -1667,7 +1672,7 @@ __device__ __forceinline__ int fx_fft_lines(Cll* s, int count, int L, int log2L,
 }
 
 // 2^60 / m for the significand 2^52 <= m < 2^53 of a float64, times 2^52 (a value in (2^59, 2^60]):
-// a float32 reciprocal and two Newton steps in integers, correct to about 2 units.
+// a float32 reciprocal and two Newton steps in integers, correct to 4 units.
 __device__ __forceinline__ long long fx_recip(unsigned long long m) {
   // D = m / 2^53 in [1/2, 1) as D 2^60; r0 ~ 1 / D in (1, 2] with 24 bits, as rh 2^-29
   const long long D = (long long)(m << 7);
@@ -1763,7 +1768,10 @@ __device__ __forceinline__ int fx_top(const int2* EU, int n) {
 }
 
 // Phase 2, per unit (kx, j), as in spectral_cols.  Every unit leaves its S in a scale of its own, noted
-// in P.EU.
+// in P.EU.  Its quotients y / (ly + lx), each formed from its own 60-bit significand, share a scale that
+// a quotient by the smallest sum would fill.  Where the unit's content lies in high eigenvalues only,
+// up to 2^27 times the smallest, they come out that much below: the unit is then done again in a finer
+// scale (its input is still in S).
 template <int N>
 __device__ __forceinline__ void fx_cols(const Geom& G, const PrecondArgs<double>& P, SolveCtx<double>& X,
                                         unsigned* s_or) {
@@ -1775,80 +1783,90 @@ __device__ __forceinline__ void fx_cols(const Geom& G, const PrecondArgs<double>
   for (int u = next_unit(X, W * N); u < W * N; u = next_unit(X, W * N)) {
     const int kx = u / N, j = u - kx * N;
     Cll* Sk = reinterpret_cast<Cll*>(P.S) + (size_t)kx * Ny * N * N;
-    if (threadIdx.x < 3) s_or[threadIdx.x] = 0;
-    __syncthreads();
-    unsigned high = 0;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < Ny * N; i += blockDim.x) {
-      const int cy = i / N, a = i - cy * N;
-      const Cll v = fx_shift(ld_cll(Sk + ((size_t)cy * N + a) * N + j), top - 60 - __ldcg(E1 + (cy >> 1) * N + a).y);
-      sts_cll(L0 + a * Ny + dft_slot(cy, P.log2y), v);
-      high |= fx_high(v);
-    }
-    fx_note(s_or, 0, high);
-    __syncthreads();
-    int slot = 0;
-    int shifted = P.log2y ? fx_fft_lines<false>(L0, N, Ny, P.log2y, P.ftwy, s_or, slot) : 0;
-    const int sh = max(0, fx_bits(s_or[slot % 3]) - 60);
-    shifted += sh;
-    ++slot;
-    // 1 / (ly + lx) in units of 2^-p: p from the smallest non-zero sum, so that the factors are <= 1
     const double lxj = P.lx[kx * N + j];
-    const double dmin = lxj + P.lymin[lxj == 0.0 ? 1 : 0];
-    const int p = (__double2hiint(dmin) >> 20) - 1023;
-    high = 0;
-#pragma unroll 1
-    for (int ky = threadIdx.x; ky < Ny; ky += blockDim.x) {
-      const Cfx* V = P.fVy + ky;
-      const int vs = opaque(Ny);
-      Cfx x[N];
-#pragma unroll
-      for (int a = 0; a < N; ++a) x[a] = fx_split(fx_shift(lds_cll(L0 + a * Ny + ky), sh));
-#pragma unroll 1
-      for (int i = 0; i < N; ++i) {
-        CfxAcc acc;
-#pragma unroll
-        for (int a = 0; a < N; ++a) acc.mac<true>(ld_cfx(V + (a * N + i) * vs), x[a]);
-        const double den = P.ly[ky * N + i] + lxj;
-        const int hi = __double2hiint(den);
-        // 2^p / den = 2^(p - e) 2^52 / m, den = m 2^(e - 52)
-        const long long q = fx_recip((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 |
-                                     (unsigned)__double2loint(den));
-        const int d = (hi >> 20) - 1023 - p;
-        // |y| < 2^62 (its high word of the 30-bit split would not fit): halved twice
-        const Cll yq = acc.get();
-        const Cfx y = fx_split(Cll{(yq.re + 2) >> 2, (yq.im + 2) >> 2});
-        const fx f = den == 0.0 ? fx{0, 0} : fx_split(q >> min(d, 63));
-        FxAcc re{0, 1ll << 29}, im{0, 1ll << 29};
-        fx_mac(re, f, y.re);
-        fx_mac(im, f, y.im);
-        // x is in registers: t takes its place
-        const Cfx t = fx_split(Cll{re.a1 + (re.a0 >> 30), im.a1 + (im.a0 >> 30)});
-        *reinterpret_cast<int4*>(L0 + i * Ny + ky) = make_int4(t.re.h, t.re.l, t.im.h, t.im.l);
-      }
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        const int4 t = *reinterpret_cast<const int4*>(L0 + i * Ny + ky);
-        x[i] = Cfx{fx{t.x, t.y}, fx{t.z, t.w}};
-      }
-#pragma unroll 1
-      for (int a = 0; a < N; ++a) {
-        CfxAcc acc;
-#pragma unroll
-        for (int i = 0; i < N; ++i) acc.mac<false>(ld_cfx(V + (a * N + i) * vs), x[i]);
-        const Cll v = acc.get();
-        sts_cll(L0 + a * Ny + ky, v);
+    // the smallest non-zero sum is 2^p (1 .. 2): quotients of values below 2^62 are below 2^(62 - p)
+    int qtop = 62 - ((__double2hiint(lxj + P.lymin[lxj == 0.0 ? 1 : 0]) >> 20) - 1023);
+    int slot, shifted;
+    for (int pass = 0;; ++pass) {
+      if (threadIdx.x < 3) s_or[threadIdx.x] = 0;
+      __syncthreads();
+      unsigned high = 0;
+#pragma unroll 4
+      for (int i = threadIdx.x; i < Ny * N; i += blockDim.x) {
+        const int cy = i / N, a = i - cy * N;
+        const Cll v = fx_shift(ld_cll(Sk + ((size_t)cy * N + a) * N + j), top - 60 - __ldcg(E1 + (cy >> 1) * N + a).y);
+        sts_cll(L0 + a * Ny + dft_slot(cy, P.log2y), v);
         high |= fx_high(v);
       }
+      fx_note(s_or, 0, high);
+      __syncthreads();
+      slot = 0;
+      shifted = P.log2y ? fx_fft_lines<false>(L0, N, Ny, P.log2y, P.ftwy, s_or, slot) : 0;
+      const int bits = fx_bits(s_or[slot % 3]), sh = max(0, bits - 60);
+      shifted += sh;
+      ++slot;
+      high = 0;
+#pragma unroll 1
+      for (int ky = threadIdx.x; ky < Ny; ky += blockDim.x) {
+        const Cfx* V = P.fVy + ky;
+        const int vs = opaque(Ny);
+        Cfx x[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) x[a] = fx_split(fx_shift(lds_cll(L0 + a * Ny + ky), sh));
+#pragma unroll 1
+        for (int i = 0; i < N; ++i) {
+          CfxAcc acc;
+#pragma unroll
+          for (int a = 0; a < N; ++a) acc.mac<true>(ld_cfx(V + (a * N + i) * vs), x[a]);
+          const Cll y = acc.get();  // |y| < 2^62
+          const double den = P.ly[ky * N + i] + lxj;
+          const unsigned long long m = fx_mag64(y);
+          Cfx t{fx{0, 0}, fx{0, 0}};
+          if (den != 0.0 && m) {
+            // den = r 2^(e - 52) and q = 2^112 / r: y / den = y q 2^(-60 - e) = t 2^(qtop - 60)
+            const int hi = __double2hiint(den), by = 64 - __clzll((long long)m);
+            const fx q = fx_split(fx_recip((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 |
+                                           (unsigned)__double2loint(den)));
+            const Cfx w = fx_split(fx_shift(y, by - 60));
+            FxAcc re{0, 1ll << 29}, im{0, 1ll << 29};
+            fx_mac(re, q, w.re);
+            fx_mac(im, q, w.im);
+            t = fx_split(fx_shift(Cll{re.a1 + (re.a0 >> 30), im.a1 + (im.a0 >> 30)}, qtop - by + (hi >> 20) - 1023));
+          }
+          // x is in registers: t takes its place
+          *reinterpret_cast<int4*>(L0 + i * Ny + ky) = make_int4(t.re.h, t.re.l, t.im.h, t.im.l);
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const int4 t = *reinterpret_cast<const int4*>(L0 + i * Ny + ky);
+          x[i] = Cfx{fx{t.x, t.y}, fx{t.z, t.w}};
+        }
+#pragma unroll 1
+        for (int a = 0; a < N; ++a) {
+          CfxAcc acc;
+#pragma unroll
+          for (int i = 0; i < N; ++i) acc.mac<false>(ld_cfx(V + (a * N + i) * vs), x[i]);
+          const Cll v = acc.get();
+          sts_cll(L0 + a * Ny + ky, v);
+          high |= fx_high(v);
+        }
+      }
+      fx_note(s_or, slot, high);
+      __syncthreads();
+      // t and V t have the same norm: with `lost` bits missing, t 2^(lost - 5) stays below 2^60.  (Below
+      // 2^32 the bits are not known: a second time may show that more are missing.)  With 20 of them
+      // gone an application still gains 12 digits; a closer line would redo units of ordinary
+      // fields (32^2 cells, n = 3, a steady state and noise: 13 missing; 71.8 us a step, 74.0 with 12)
+      const int lost = min(bits, 60) - fx_bits(s_or[slot % 3]);
+      if (lost <= 20 || pass == 3) break;
+      qtop -= lost - 5;
+      __syncthreads();  // every thread has read s_or
     }
-    fx_note(s_or, slot, high);
-    __syncthreads();
     if (P.log2y) shifted += fx_fft_lines<true>(L0, N, Ny, P.log2y, P.ftwy, s_or, slot);
     if (threadIdx.x == 0) {
-      // the factors are q 2^-60 = 2^p / den: the result counts in 2^(e0 + shifted - p)
-      const unsigned m = s_or[slot % 3];
-      const int e = e0 + shifted + 2 - p;
-      P.EU[u] = make_int2(m ? e + fx_bits(m) : -(1 << 28), e);
+      // values below 2^32, zeros among them, count as 2^32: their magnitudes are not noted
+      const int e = e0 + shifted + qtop - 60;
+      P.EU[u] = make_int2(e + fx_bits(s_or[slot % 3]), e);
     }
     for (int i = threadIdx.x; i < Ny * N; i += blockDim.x) {
       const int cy = i / N, a = i - cy * N;

@@ -206,3 +206,49 @@ def test_mixed_steps_on_lines_too_long_for_the_fixed_point_solve(dg, Nx, Ny, n, 
         norm = lambda v: np.sqrt(np.sum(v * v / o.W2))
         floor = np.sqrt(rounding_floor2(o) * np.sum(o.W2 * p * p))
         assert norm(r) <= 1e-8 * norm(b) + 2 * floor
+
+
+def _line_mode(dg, N, n, L, k, branch):
+    """A real eigenvector of the scaled 1D operator of a line as node values (N, n) of the field (the
+    scaled one over sqrt(w)), and its eigenvalue."""
+    lam, V = dg.spectral_symbol(N, n, L, k)
+    u = np.real(np.exp(2j * np.pi * (k * np.arange(N) % N) / N)[:, None] * V[None, :, branch])
+    return u / np.sqrt(np.polynomial.legendre.leggauss(n)[1]), lam[branch]
+
+
+@pytest.mark.parametrize("Nx,Ny,n", [(4, 1024, 5), (4, 2048, 5), (2, 4096, 3), (1024, 4, 5), (2, 16, 4)])
+def test_spectral_solve_of_high_modes(dg, Nx, Ny, n):
+    """Single eigenmodes of the highest branch along the long side, with quotients up to 2^27 below those
+    of the line's smooth modes: solved in one application or two."""
+    Lx, Ly = 1.5, 2.0
+    g = dg.Grid(Nx, Ny, n, Lx, Ly)
+    g.set_precond("spectral")
+    bar = solve_bar(Operators(OGrid(Nx, Ny, n, Lx, Ly)), Lx, Ly)
+    N, L = max((Nx, Lx), (Ny, Ly))
+    for k in sorted({0, 1, 3, N // 4, N // 2 - 1, N // 2}):
+        u, lam = _line_mode(dg, N, n, L, k, n - 1)
+        u /= np.abs(u).max()
+        w = np.empty(g.shape)
+        w[:] = u[None, :, None, :] if Nx > Ny else u[:, None, :, None]
+        psi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+        rc, it, relres = dg.dg_poisson_solve(g, dev(w), psi, 1e-10, 50)
+        assert it <= 2 and relres <= 1e-10, k
+        assert rel_l2(host(psi), w / lam) < bar, k
+
+
+def test_spectral_solve_of_a_high_and_a_small_smooth_mode(dg):
+    """A mode of the highest branch along the long lines, and a smooth one across them that is small in
+    the right-hand side and larger in the solution."""
+    Nx, Ny, n, Lx = 1024, 16, 5, 1.0
+    g = dg.Grid(Nx, Ny, n, Lx, 16 * Lx)
+    g.set_precond("spectral")
+    hi, lam = _line_mode(dg, Nx, n, Lx, 1, n - 1)
+    lo, mu = _line_mode(dg, Ny, n, 16 * Lx, 1, 0)
+    hi, lo = hi / np.abs(hi).max(), lo / np.abs(lo).max()
+    for s in (-28, -29, -30):
+        w = hi[None, :, None, :] + 2.0 ** s * lo[:, None, :, None]
+        ref = hi[None, :, None, :] / lam + 2.0 ** s / mu * lo[:, None, :, None]
+        psi = torch.zeros(g.shape, dtype=torch.float64, device="cuda")
+        rc, it, relres = dg.dg_poisson_solve(g, dev(w), psi, 1e-12, 50)
+        assert it <= 2 and relres <= 1e-12, s
+        assert rel_l2(host(psi), ref) < 1e-5, s
