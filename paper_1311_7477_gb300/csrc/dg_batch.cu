@@ -35,14 +35,22 @@ __global__ void __launch_bounds__(kThreads) batch_kernel(const __grid_constant__
   if (!ok && threadIdx.x == 0) atomicCAS(A.error, 0, kFlagTimeout);
 }
 
-int batch_kernel_occupancy(size_t smem, int* per_sm) {
+int batch_smem_limit(size_t* limit, size_t* all) {
   int dev = 0, optin = 0;
   CUDA_TRY(cudaGetDevice(&dev));
   CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   cudaFuncAttributes fa;
   CUDA_TRY(cudaFuncGetAttributes(&fa, batch_kernel));
-  if (smem + fa.sharedSizeBytes > (size_t)optin)
-    return fail(DG_ERR_ARG, "batch needs %zu B of shared memory per block (max %d)", smem + fa.sharedSizeBytes, optin);
+  *all = (size_t)optin;
+  *limit = *all - fa.sharedSizeBytes;
+  return DG_OK;
+}
+
+int batch_kernel_occupancy(size_t smem, int* per_sm) {
+  size_t limit = 0, all = 0;
+  if (int rc = batch_smem_limit(&limit, &all)) return rc;
+  if (smem > limit)
+    return fail(DG_ERR_ARG, "batch needs %zu B of shared memory per block (max %zu)", smem + all - limit, all);
   if (int rc = set_smem(batch_kernel, smem)) return rc;
   CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, batch_kernel, kThreads, smem));
   return DG_OK;

@@ -1702,6 +1702,9 @@ namespace {
 // Tiles of a simulation inside a batch: the batch's choice for its n, else the built-in ones
 // (a small grid's blocks are few in a batch group, so its tiles are not split further as for a
 // whole-GPU solve).
+// The fixed-point operator stages a tile's results beside its box, more than the box and its face
+// traces in float64 take from 8 x 8 cells on (n = 5, 20 x 20: 257 and 178 KB).  A solve tile that
+// fits the latter way is accepted: it is split until it fits the former.
 void batch_geoms(const dg_batch* b, const dg_grid* g, Geom* Gr, Geom* Gc) {
   int rty, rtx, cty, ctx;
   default_tiles(g->n, rty, rtx, cty, ctx);
@@ -1715,6 +1718,16 @@ void batch_geoms(const dg_batch* b, const dg_grid* g, Geom* Gr, Geom* Gc) {
   }
   *Gr = geom_of(g, rty, rtx);
   *Gc = geom_of(g, cty, ctx);
+  size_t limit = 0, all = 0;
+  if (batch_smem_limit(&limit, &all)) return;  // reported by batch_kernel_occupancy
+  dispatch_n(g->n, [&](auto nc) {
+    constexpr int N = decltype(nc)::value;
+    const size_t ops = batch_ops_bytes<N>(), bt = g->precond == kPrecondTwoLevel ? N * N * N * N : 0;
+    if (ops + 4 * bt + 8 * cg_tile_values<double, N>(Gc->TY, Gc->TX) > all) return DG_OK;  // refused
+    while (ops + 8 * bt + cg_tile_bytes<double, N>(Gc->TY, Gc->TX) + 32 > limit && Gc->TY * Gc->TX > 1)
+      *Gc = Gc->TX >= Gc->TY ? geom_of(g, Gc->TY, (Gc->TX + 1) / 2) : geom_of(g, (Gc->TY + 1) / 2, Gc->TX);
+    return DG_OK;
+  });
 }
 
 BatchSim make_batch_sim(const dg_batch* bt, dg_sim* s) {

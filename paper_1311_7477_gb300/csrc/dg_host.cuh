@@ -371,7 +371,9 @@ int launch_scale(const dg_grid* g, const double* x, double* y, int inverse, cuda
 int launch_invariants_final(const double* part, int nparts, double* out, cudaStream_t st);
 // the capped-barrier self-test kernel; returns the CUDA error of the launch
 cudaError_t launch_barrier_selftest(SyncState* s, int* out, cudaStream_t st);
-// the batched persistent kernel: occupancy for smem bytes of dynamic shared memory, launch
+// the batched persistent kernel: the dynamic shared memory a block may have (and all of it, static
+// included), occupancy for smem bytes of it, launch
+int batch_smem_limit(size_t* limit, size_t* all);
 int batch_kernel_occupancy(size_t smem, int* per_sm);
 int batch_kernel_launch(const BatchArgs& A, int grid, size_t smem, cudaStream_t st);
 

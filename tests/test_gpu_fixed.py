@@ -252,3 +252,40 @@ def test_spectral_solve_of_a_high_and_a_small_smooth_mode(dg):
         rc, it, relres = dg.dg_poisson_solve(g, dev(w), psi, 1e-12, 50)
         assert it <= 2 and relres <= 1e-12, s
         assert rel_l2(host(psi), ref) < 1e-5, s
+
+
+@pytest.mark.parametrize("n,tile", [(4, (26, 25)), (5, (20, 21))])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("precond", ["jacobi", "twolevel"])
+def test_batch_with_large_solve_tiles(dg, n, tile, prec, precond):
+    """Solve tiles that fit shared memory with their face traces, but not with the fixed-point results
+    beside the box: accepted, and the steps agree with those on the built-in tiles to the bar of the
+    batched tests for solves stopped by a tolerance (1e-8)."""
+    out = []
+    for t in (tile, (0, 0)):
+        g = dg.Grid(30, 28, n)
+        g.set_precond(precond)
+        X, Y = OGrid(30, 28, n).mesh()
+        s = dg.Sim(g, dev(np.sin(X) * np.cos(2 * Y) + 0.3 * np.cos(X + Y)), D=1e-3, dt=1e-3, cg_tol=1e-12,
+                   precision=dg.DG_FP64 if prec == "fp64" else dg.DG_MIXED)
+        b = dg.Batch(1)
+        b.set_tiles(n, cg=t)
+        b.admit(s)
+        b.step(2)
+        assert b.status()["rc"] == 0
+        f = [torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(2)]
+        s.get(*f)
+        out.append([host(x) for x in f])
+    for a, c in zip(*out):
+        assert rel_l2(a, c) < 1e-8
+
+
+def test_batch_refuses_tiles_that_never_fitted(dg):
+    g = dg.Grid(32, 32, 5)
+    s = dg.Sim(g, dev(np.random.default_rng(0).standard_normal(g.shape)), dt=1e-6)
+    b = dg.Batch(1)
+    b.set_tiles(5, cg=(28, 28))
+    b.admit(s)
+    with pytest.raises(dg.DGError) as e:
+        b.step(1)
+    assert e.value.code == dg.DG_ERR_ARG
