@@ -15,7 +15,7 @@ import pytest
 from oracle.operators import Operators
 from oracle.solver import Spectral, poisson_rhs, rounding_floor2
 from oracle.tables import Grid as OGrid
-from tests.test_gpu_parity import bracket_scale, dev, host, rel_l2
+from tests.test_gpu_parity import RHO_D, bracket_scale, dev, host, rel_l2
 from tests.test_gpu_spectral import solve_bar
 
 pytestmark = pytest.mark.gpu
@@ -289,3 +289,48 @@ def test_batch_refuses_tiles_that_never_fitted(dg):
     with pytest.raises(dg.DGError) as e:
         b.step(1)
     assert e.value.code == dg.DG_ERR_ARG
+
+
+@pytest.mark.parametrize("N,n", [(640, 4), (512, 5)])
+def test_pointwise_bracket_of_resolved_fields(dg, N, n):
+    """J++ alone on fields whose derivatives are far below the range of their rows.  The bar is the
+    float64 rounding of the two factors: each derivative is off by about 2^-53 rho_D / h |f|, and
+    |f| ~ |f_x| here; four times that."""
+    g = dg.Grid(N, N, n)
+    og = OGrid(N, N, n)
+    o = Operators(og)
+    X, Y = og.mesh()
+    f, h = np.sin(X) * np.cos(Y) + 0.2 * np.cos(2 * Y), np.cos(X - Y) + 0.3 * np.sin(2 * X)
+    J = torch.empty(g.shape, dtype=torch.float64, device="cuda")
+    dg.dg_bracket_parts(g, dev(f), dev(h), J, 1)
+    assert rel_l2(host(J), o.bracket_parts(f, h)[0]) < 4 * 2.0 ** -53 * RHO_D[n] / og.hx
+
+
+@pytest.mark.parametrize("Nx,Ny,n", SHAPES)
+@pytest.mark.parametrize("bc", ["periodic", "dirichlet"])
+def test_pointwise_bracket(dg, Nx, Ny, n, bc):
+    """J++ alone, in a bracket and in a step with viscosity; it changes sign with its arguments' order
+    and vanishes on equal ones, bitwise; its result scales with powers of two."""
+    Lx, Ly, D = 1.5, 2.0, 0.05
+    g = dg.Grid(Nx, Ny, n, Lx, Ly, bc=bc)
+    o = Operators(OGrid(Nx, Ny, n, Lx, Ly), bc=bc)
+    psi, w, z = np.random.default_rng(Nx + n).standard_normal((3, Ny, Nx, n, n))
+    scale = bracket_scale(o, psi, w)
+    J = torch.empty(g.shape, dtype=torch.float64, device="cuda")
+
+    def jpp(a, b):
+        dg.dg_bracket_parts(g, dev(a), dev(b), J, 1)
+        return host(J).copy()
+    a = jpp(psi, w)
+    assert rel_l2(a, o.bracket_parts(psi, w)[0], scale) < 1e-12
+    assert np.array_equal(jpp(w, psi), -a) and not jpp(psi, psi).any()
+    assert np.array_equal(jpp(np.ldexp(psi, 200), np.ldexp(w, -100)), np.ldexp(a, 100))
+    s = dg.Sim(g, dev(np.zeros(g.shape)), D=D, dt=1e-6)
+    s.set_bracket("naive")
+    s.set_state(5, dev(w), dev(psi), dev(psi), dev(z), dev(z))
+    s.set_cg(1e-30, 10, fixed_iters=1)
+    s.step(1)
+    b = [torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(5)]
+    s.get_state(*b)
+    lap = D * o.laplacian(w)
+    assert rel_l2(host(b[3]), lap - o.bracket_parts(psi, w)[0], scale + np.linalg.norm(lap.ravel())) < 1e-12
