@@ -245,6 +245,86 @@ __host__ __device__ constexpr int fx_cell() {
   return (N * N) | 1;
 }
 
+// How far below a tile's largest value its cells may lie in fixed point, in bits.  Errors there are
+// relative to the tile's largest value, in float64 to the values around the node.  Away from a cell 2^s
+// times the others they pass those of the float64 tile at s = 6 (operators) and, for the bracket, whose
+// two fields' bits add up, at s = 4, 4, 4, 3, 2 for n = 1..5, and double with each bit: at 8 bits
+// they are 3.5 times and 15 to 80 times the float64 tile's.  A tile with a cell further down, its eight
+// neighbours too (the zero line of a field does not count), is left to float64: the tail of a compact
+// vortex, the foot of a thin shear layer.  Such a tile takes four times as long; what it takes to
+// find out costs the others 1 to 5% (1000^2 cells, n = 4: 704 -> 714 us; 501 x 373, n = 3: 69 -> 72;
+// Laplacian, 500 x 300, n = 5: 70.5 -> 72.2).
+constexpr int kFxRange = 8;
+
+// The smallest non-zero magnitude word of what a thread staged, less 1 (zeros wrap around to the largest).
+__device__ __forceinline__ unsigned fx_low(unsigned low, double v) { return min(low, fx_mag(v) - 1u); }
+// The bits between the largest and the smallest non-zero value, from their magnitude words.
+__device__ __forceinline__ int fx_spread(unsigned mag, unsigned low) {
+  return mag ? max(1, int(mag >> 20)) - max(1, int((low + 1u) >> 20)) : 0;
+}
+
+// Whether a cell of the tile lies more than kFxRange bits below the largest value ef, eg of the staged
+// fields f, g: the bits of both added, or (alone) those of g.  f may be null: g alone, on a box without
+// corners.  e: one or two words per box cell of scratch.  In every thread, after a block synchronisation.
+template <int N>
+__device__ __noinline__ bool fx_far(const TileBox& B, const double* f, const double* g, int ef, int eg, bool alone,
+                                    int* e) {
+  constexpr int CS = fx_cell<N>();
+  const int BWe = B.TXe + 2, BHe = B.TYe + 2, nb = BWe * BHe;
+  const unsigned mw = magic_of(BWe);
+  for (int u = threadIdx.x; u < (f ? 2 : 1) * nb; u += blockDim.x) {
+    const int c = u < nb ? u : u - nb;
+    const int br = quot(c, mw), bc = c - br * BWe;
+    const bool corner = (br == 0 || br == BHe - 1) && (bc == 0 || bc == BWe - 1);
+    unsigned m = 0;
+    if (f || !corner) {
+      const double* v = (u < nb ? g : f) + (br * B.BW + bc) * CS;
+      for (int k = 0; k < N * N; ++k) m = max(m, fx_mag(v[k]));
+    }
+    e[u] = m ? max(1, int(m >> 20)) : 0;
+  }
+  __syncthreads();
+  bool far = false;
+  for (int c = threadIdx.x; c < B.TYe * B.TXe; c += blockDim.x) {
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    int mg = 0, mf = 0;
+    for (int y = 0; y < 3; ++y)
+      for (int x = 0; x < 3; ++x) {
+        const int o = (ry + y) * BWe + rx + x;
+        mg = max(mg, e[o]);
+        if (f) mf = max(mf, e[nb + o]);
+      }
+    if (mg && alone) far |= eg - mg > kFxRange;
+    if (mg && mf) far |= ef - mf + eg - mg > kFxRange;
+  }
+  return __syncthreads_or(far);
+}
+
+// A quick look at the converted tile before that one: whether a cell has no node near the largest values
+// among the middle nodes of itself and its eight neighbours.  (The zero lines of resolved fields, which most
+// tiles that come here have, end here.)  In every thread, after a block synchronisation.
+template <int N>
+__device__ __forceinline__ bool fx_lonely(const TileBox& B, const fx* f, const fx* g) {
+  constexpr int CS = fx_cell<N>();
+  bool lonely = false;
+  for (int c = threadIdx.x; c < B.TYe * B.TXe; c += blockDim.x) {
+    const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
+    const int o = (ry * B.BW + rx) * CS + N / 2 * (N + 1);
+    int least = 64;
+#pragma unroll
+    for (int y = 0; y < 3; ++y)
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        const int i = o + (y * B.BW + x) * CS;
+        // high words of the largest values lie in 2^29 .. 2^30
+        const int hg = g[i].h, hf = f ? f[i].h : 1 << 29;
+        least = min(least, __clz(hg ^ (hg >> 31)) + __clz(hf ^ (hf >> 31)) - 4);
+      }
+    lonely |= least > kFxRange;
+  }
+  return __syncthreads_or(lonely);
+}
+
 // The factors of the fixed-point LDG operators, 1 / hx^2 and 1 / hy^2.  ok: they lie in the range the
 // fixed-point path covers.  stiff, lap: device tables (FxTable<n>) that replace fx_stiff and fx_lap
 // on grids with a jump penalty tau != 0, else null.
@@ -299,8 +379,8 @@ __host__ __device__ constexpr size_t rhs_smem_bytes(int TY, int TX) {
 }
 
 // The tile in float64: for tiles whose values the fixed-point scale cannot hold (infinities, NaN,
-// products near the ends of the float64 range).  It needs more shared memory per cell than the
-// fixed-point tile, so it runs on sub-tiles that fit.
+// products near the ends of the float64 range, cells far below the others: kFxRange).  It needs more
+// shared memory per cell than the fixed-point tile, so it runs on sub-tiles that fit.
 template <int N>
 __device__ __noinline__ void rhs_tile_float(const Ops2D<double, N>& C, const Geom& G, const RhsArgs& A, int tile,
                                             unsigned char* smem) {
@@ -332,7 +412,7 @@ __device__ __noinline__ void rhs_tile_float(const Ops2D<double, N>& C, const Geo
 // field's derivatives are kept, and multiplied after a shift that fills 60 bits.  Returns the
 // two fields' shifts, by which the result's unit is finer.  (Smooth fields, 512^2 cells, n = 5, against
 // long double: relative error 6.9e-12 without the shifts, 3.2e-15 with; the float64 tile 1.9e-13.  1000^2
-// cells, n = 5: 1029 us, 1267 through the phases of the whole J.)
+// cells, n = 4: 603 us, 745 through the phases of the whole J.)
 template <int N>
 __device__ __noinline__ int fx_jpp(const Geom& G, const TileBox& B, fx* sF, fx* sG, fx* sA, fx* sB, fx* sC,
                                    unsigned (*s_mag)[16]) {
@@ -414,7 +494,7 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
                                          const RhsArgs& A, int tile, unsigned char* smem) {
   constexpr int NN = N * N;
   constexpr int CS = fx_cell<N>();
-  __shared__ unsigned s_mag[2][16];
+  __shared__ unsigned s_mag[4][16];
   static_assert(rhs_threads<N>() <= 512 && kThreads <= 512, "warps of s_mag");
   __shared__ fx s_isw[NN];
   constexpr FxTable<N> D = fx_deriv<N>();
@@ -428,71 +508,86 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
   fx* sB = sA + boxc * CS;  // g_x, then h1, then lx g
   fx* sC = sB + boxc * CS;  // h2, then ly g
 
-  // stage the two fields and their largest magnitudes
-  {
-    double* rF = reinterpret_cast<double*>(sF);
-    double* rG = reinterpret_cast<double*>(sG);
-    unsigned mf = 0, mg = 0;
-    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
-    const int rowlen = BWe * NN, total = BHe * rowlen;
-    const unsigned mrow = magic_of(rowlen);
-#pragma unroll 4
-    for (int i = threadIdx.x; i < total; i += blockDim.x) {
-      const int br = quot(i, mrow);
-      const int j = i - br * rowlen;
-      const int bc = j / NN, k = j - bc * NN;
-      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
-      const int o = (br * BW + bc) * CS + k;
-      if (Gen && G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)) {
-        rF[o] = 0.0;
-        rG[o] = 0.0;
-        continue;
-      }
-      const size_t g = ((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k;
-      const double f = A.psi[g], w = A.omega_in[g];
-      rF[o] = f;
-      rG[o] = w;
-      mf = max(mf, fx_mag(f));
-      mg = max(mg, fx_mag(w));
-    }
-    mf = __reduce_max_sync(0xffffffffu, mf);
-    mg = __reduce_max_sync(0xffffffffu, mg);
-    if (A.psi_scaled && threadIdx.x < NN) s_isw[threadIdx.x] = F.isw[threadIdx.x];
-    if ((threadIdx.x & 31) == 0) {
-      s_mag[0][threadIdx.x >> 5] = mf;
-      s_mag[1][threadIdx.x >> 5] = mg;
-    }
-  }
-  __syncthreads();
-  const int nw = int(blockDim.x >> 5), lane = threadIdx.x & 31;
-  const unsigned mf = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[0][lane] : 0u);
-  const unsigned mg = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[1][lane] : 0u);
-  const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
-  // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any)
-  const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
-  int uj = uf + ug + 2 * D.e + 60;
-  const int ul = ug + (F.l.lap ? static_cast<const FxTable<N>*>(F.l.lap)->e : Lp.e);
   const bool viscous = A.visc != 0.0 && !A.bracket_only;
-  // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
-  const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.l.ok && abs(ul) <= 600));
-  if (!covered) {
-    __syncthreads();  // the staging is reused
-    rhs_tile_float<N>(C, G, A, tile, smem);
-    return;
-  }
-  for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
-    const fx f = sF[i], w = sG[i];  // raw bits: {low, high} words
-    long long x = fx_from_bits(unsigned(f.l), unsigned(f.h), ef);
-    if (A.psi_scaled) {
-      const int k = i % CS;
-      FxAcc s;
-      fx_mac(s, s_isw[k < NN ? k : 0], fx_split(x));
-      x = fx_round(s);
+  const int nw = int(blockDim.x >> 5), lane = threadIdx.x & 31;
+  int uj, ul;  // units of the products and of the viscous term, 2^uj and 2^ul
+  for (bool again = false;; again = true) {
+    // stage the two fields and their largest and smallest magnitudes
+    {
+      double* rF = reinterpret_cast<double*>(sF);
+      double* rG = reinterpret_cast<double*>(sG);
+      unsigned mf = 0, mg = 0, nf = ~0u, ng = ~0u;
+      const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+      const int rowlen = BWe * NN, total = BHe * rowlen;
+      const unsigned mrow = magic_of(rowlen);
+#pragma unroll 4
+      for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int br = quot(i, mrow);
+        const int j = i - br * rowlen;
+        const int bc = j / NN, k = j - bc * NN;
+        const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+        const int o = (br * BW + bc) * CS + k;
+        if (Gen && G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)) {
+          rF[o] = 0.0;
+          rG[o] = 0.0;
+          continue;
+        }
+        const size_t g = ((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k;
+        const double f = A.psi[g], w = A.omega_in[g];
+        rF[o] = f;
+        rG[o] = w;
+        mf = max(mf, fx_mag(f));
+        mg = max(mg, fx_mag(w));
+        nf = fx_low(nf, f);
+        ng = fx_low(ng, w);
+      }
+      mf = __reduce_max_sync(0xffffffffu, mf);
+      mg = __reduce_max_sync(0xffffffffu, mg);
+      nf = __reduce_min_sync(0xffffffffu, nf);
+      ng = __reduce_min_sync(0xffffffffu, ng);
+      if (A.psi_scaled && threadIdx.x < NN) s_isw[threadIdx.x] = F.isw[threadIdx.x];
+      if ((threadIdx.x & 31) == 0) {
+        s_mag[0][threadIdx.x >> 5] = mf;
+        s_mag[1][threadIdx.x >> 5] = mg;
+        s_mag[2][threadIdx.x >> 5] = nf;
+        s_mag[3][threadIdx.x >> 5] = ng;
+      }
     }
-    sF[i] = fx_split(x);
-    sG[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), eg));
+    __syncthreads();
+    const unsigned mf = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[0][lane] : 0u);
+    const unsigned mg = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[1][lane] : 0u);
+    const unsigned nf = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[2][lane] : ~0u);
+    const unsigned ng = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[3][lane] : ~0u);
+    const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
+    // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any)
+    const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
+    uj = uf + ug + 2 * D.e + 60;
+    ul = ug + (F.l.lap ? static_cast<const FxTable<N>*>(F.l.lap)->e : Lp.e);
+    // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
+    const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.l.ok && abs(ul) <= 600));
+    if (!covered || (again && fx_far<N>(B, reinterpret_cast<const double*>(sF), reinterpret_cast<const double*>(sG), ef,
+                                        eg, viscous, reinterpret_cast<int*>(sA)))) {
+      __syncthreads();  // the staging is reused
+      rhs_tile_float<N>(C, G, A, tile, smem);
+      return;
+    }
+    for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
+      const fx f = sF[i], w = sG[i];  // raw bits: {low, high} words
+      long long x = fx_from_bits(unsigned(f.l), unsigned(f.h), ef);
+      if (A.psi_scaled) {
+        const int k = i % CS;
+        FxAcc s;
+        fx_mac(s, s_isw[k < NN ? k : 0], fx_split(x));
+        x = fx_round(s);
+      }
+      sF[i] = fx_split(x);
+      sG[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), eg));
+    }
+    __syncthreads();
+    // values far apart (kFxRange), and perhaps a cell of nothing else: the tile is staged again, to look at
+    // its cells themselves
+    if (again || fx_spread(mf, nf) + fx_spread(mg, ng) <= kFxRange || !fx_lonely<N>(B, sF, sG)) break;
   }
-  __syncthreads();
 
   // Which parts enter (Eq. J): J = s (c0 J++ + J+x + Jx+) with J+x = D_x(f g_y) - D_y(f g_x),
   // Jx+ = D_y(f_x g) - D_x(f_y g).
@@ -669,13 +764,15 @@ __global__ void __launch_bounds__(rhs_threads<N>(), rhs_blocks<N>()) rhs_kernel(
 // One tile of an LDG operator on a float64 field in fixed point (dg_fixed.cuh).
 // =========================================================================================
 
-// Shared memory of the pass: the staged box and the two directions' results on the tile.
+// Shared memory of the pass: the staged box and the two directions' results on the tile (or, before
+// them, fx_far's word per box cell).
 template <int N>
 __host__ __device__ constexpr size_t fx_apply_bytes(int TY, int TX) {
-  return ((size_t)(TY + 2) * (TX + 2) + 2 * (size_t)TY * TX) * fx_cell<N>() * 8;
+  const size_t box = (size_t)(TY + 2) * (TX + 2), q = 2 * (size_t)TY * TX * fx_cell<N>() * 8;
+  return box * fx_cell<N>() * 8 + (q > 4 * box ? q : (4 * box + 7) / 8 * 8);
 }
 
-// The lines of the tile in float64, for tiles the fixed-point scale cannot hold.
+// The lines of the tile in float64, for tiles the fixed-point scale cannot hold or not well enough.
 template <int N>
 __device__ __noinline__ void apply_lines_float(const Op1D<double, N>& ox, const Op1D<double, N>& oy, const Geom& G,
                                                const TileBox& B, const double* sU, double* qx, double* qy) {
@@ -707,8 +804,10 @@ __device__ __noinline__ void apply_lines_float(const Op1D<double, N>& ox, const 
 
 // Stages u = load(g, k, interior) on the tile and its plus-shaped halo, applies the operator (Lap:
 // -Delta_h, else W^-1/2 A W^-1/2; ox, oy its float64 form) and hands (g, k, q) of the tile's nodes
-// to out.  smem: fx_apply_bytes<N>(G.TY, G.TX).
-template <int N, bool Lap, class LoadF, class OutF>
+// to out.  Local: tiles with cells far below the others (kFxRange) go to float64.  The solves do
+// without: there errors count against the norm of the whole field, and 2^-60 of a tile's largest
+// value is below 2^-53 of its norm.  smem: fx_apply_bytes<N>(G.TY, G.TX).
+template <int N, bool Lap, bool Local, class LoadF, class OutF>
 __device__ __forceinline__ void fx_tile_apply(const Op1D<double, N>& ox, const Op1D<double, N>& oy, const FxScale& S,
                                               const Geom& G, int tile, void* smem, LoadF&& load, OutF&& out) {
   constexpr int NN = N * N;
@@ -720,43 +819,63 @@ __device__ __forceinline__ void fx_tile_apply(const Op1D<double, N>& ox, const O
   fx* sU = static_cast<fx*>(smem);
   long long* qx = reinterpret_cast<long long*>(sU + boxc * CS);
   long long* qy = qx + G.TY * G.TX * CS;
-  unsigned m = 0;
-  {
-    double* rU = reinterpret_cast<double*>(sU);
-    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
-    const int rowlen = BWe * NN, total = BHe * rowlen;
-    const unsigned mrow = magic_of(rowlen);
-#pragma unroll 4
-    for (int i = threadIdx.x; i < total; i += blockDim.x) {
-      const int br = quot(i, mrow);
-      const int j = i - br * rowlen;
-      const int bc = j / NN, k = j - bc * NN;
-      const bool rowhalo = (br == 0) || (br == BHe - 1), colhalo = (bc == 0) || (bc == BWe - 1);
-      if (rowhalo && colhalo) continue;  // the 5-cell operators never read the corners
-      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
-      const int o = (br * BW + bc) * CS + k;
-      double v = 0.0;  // Dirichlet: zero outside
-      if (!(G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)))
-        v = load(((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k, k, !(rowhalo || colhalo));
-      rU[o] = v;
-      m = max(m, fx_mag(v));
-    }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) s_mag[threadIdx.x >> 5] = m;
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  m = __reduce_max_sync(0xffffffffu, lane < int(blockDim.x >> 5) ? s_mag[lane] : 0u);
+  const int lane = threadIdx.x & 31, nw = int(blockDim.x >> 5);
   const FxTable<N>* tab = static_cast<const FxTable<N>*>(Lap ? S.lap : S.stiff);
-  const int em = max(1, int(m >> 20)), uq = m ? em - 1082 + (tab ? tab->e : O.e) : 0;
-  const bool covered = S.ok && em < 2047 && abs(uq) <= 600;
-  const int nc = B.TYe * B.TXe;
-  if (covered) {
+  int uq;
+  bool covered;
+  for (bool again = false;; again = true) {
+    unsigned m = 0, low = ~0u;
+    {
+      double* rU = reinterpret_cast<double*>(sU);
+      const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+      const int rowlen = BWe * NN, total = BHe * rowlen;
+      const unsigned mrow = magic_of(rowlen);
+#pragma unroll 4
+      for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int br = quot(i, mrow);
+        const int j = i - br * rowlen;
+        const int bc = j / NN, k = j - bc * NN;
+        const bool rowhalo = (br == 0) || (br == BHe - 1), colhalo = (bc == 0) || (bc == BWe - 1);
+        const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+        const int o = (br * BW + bc) * CS + k;
+        if (rowhalo && colhalo) {  // the 5-cell operators never read the corners
+          if constexpr (Local) rU[o] = 0.0;
+          continue;
+        }
+        double v = 0.0;  // Dirichlet: zero outside
+        if (!(G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)))
+          v = load(((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k, k, !(rowhalo || colhalo));
+        rU[o] = v;
+        m = max(m, fx_mag(v));
+        if constexpr (Local) low = fx_low(low, v);
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if constexpr (Local) low = __reduce_min_sync(0xffffffffu, low);
+      if ((threadIdx.x & 31) == 0) {
+        s_mag[threadIdx.x >> 5] = m;
+        if constexpr (Local) s_mag[16 + (threadIdx.x >> 5)] = low;
+      }
+    }
+    __syncthreads();
+    m = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[lane] : 0u);
+    const int em = max(1, int(m >> 20));
+    uq = m ? em - 1082 + (tab ? tab->e : O.e) : 0;
+    covered = S.ok && em < 2047 && abs(uq) <= 600;
+    if constexpr (Local) {
+      low = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[16 + lane] : ~0u);
+      if (covered && again)
+        covered = !fx_far<N>(B, nullptr, reinterpret_cast<const double*>(sU), 0, em, true, reinterpret_cast<int*>(qx));
+    }
+    if (!covered) break;
     for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
       const fx w = sU[i];  // raw bits: {low, high} words
       sU[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), em));
     }
     __syncthreads();
+    if (!Local || again || fx_spread(m, low) <= kFxRange || !fx_lonely<N>(B, nullptr, sU)) break;
+  }
+  const int nc = B.TYe * B.TXe;
+  if (covered) {
     const unsigned mnc = magic_of(nc);
     if (tab) fx_lines_table<N>(tab, B, sU, qx, qy, G.TX, 0);
     for (int u = threadIdx.x; u < (tab ? 0 : 2 * nc * N); u += blockDim.x) {
@@ -819,7 +938,7 @@ __global__ void __launch_bounds__(kThreads, 4) apply_kernel(const Ops2D<double, 
     if (threadIdx.x < N * N) s_sw[threadIdx.x] = C->sw[threadIdx.x];
     __syncthreads();
   }
-  fx_tile_apply<N, Lap>(
+  fx_tile_apply<N, Lap, true>(
       Lap ? C->lx : C->kx, Lap ? C->ly : C->ky, S, G, blockIdx.x, smem_raw,
       [&](size_t g, int k, bool) { return Lap ? x[g] : x[g] * s_sw[k]; },
       [&](size_t g, int k, double q) { y[g] = Lap ? -q : q * s_sw[k]; });
@@ -1170,7 +1289,7 @@ template <typename T, int N, class LoadF, class OutF>
 __device__ __forceinline__ void solve_apply(const Ops2D<T, N>& C, const Geom& G, int tile, SolveCtx<T>& X,
                                             LoadF&& load, OutF&& out) {
   if constexpr (std::is_same<T, double>::value) {
-    fx_tile_apply<N, false>(C.kx, C.ky, X.ks, G, tile, X.sU, load, out);
+    fx_tile_apply<N, false, false>(C.kx, C.ky, X.ks, G, tile, X.sU, load, out);
   } else {
     if (X.kdf) {
       SolveCtx<df> W;

@@ -334,3 +334,70 @@ def test_pointwise_bracket(dg, Nx, Ny, n, bc):
     s.get_state(*b)
     lap = D * o.laplacian(w)
     assert rel_l2(host(b[3]), lap - o.bracket_parts(psi, w)[0], scale + np.linalg.norm(lap.ravel())) < 1e-12
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("bc", ["periodic", "dirichlet"])
+@pytest.mark.parametrize("bits", [5, 8, 9, 20, 45, 70, 300])
+def test_cells_far_below_their_tile(dg, n, bc, bits):
+    """A cell 2^bits times the others, or others that are that much smaller: away from it the operators'
+    results are those without it, to the bar of the other fields (1e-12 of the local scale; 2^-53 and
+    the table of errors at the range's end, 80 at most, leave a hundredfold)."""
+    Nx, Ny, Lx, Ly, D = 19, 17, 1.5, 2.0, 0.05
+    g = dg.Grid(Nx, Ny, n, Lx, Ly, bc=bc)
+    g.set_tiles(16 if n < 3 else 8, 16 if n < 3 else 8)  # (not the small tiles of a small grid)
+    o = Operators(OGrid(Nx, Ny, n, Lx, Ly), bc=bc)
+    f, h = np.random.default_rng(n).standard_normal((2, Ny, Nx, n, n))
+    out = torch.empty(g.shape, dtype=torch.float64, device="cuda")
+    cy, cx = 6, 9
+    dy, dx = np.abs(np.arange(Ny) - cy), np.abs(np.arange(Nx) - cx)
+    away = np.maximum(dy[:, None], dx[None, :]) >= 2
+    lap = o.laplacian(h)
+    J, scale = o.bracket(f, h), bracket_scale(o, f, h)
+    Jp = o.bracket_parts(f, h)[0]
+
+    def check(got, want, k, scale=0.0):
+        assert rel_l2(np.ldexp(host(got), k)[away], want[away], scale) < 1e-12
+
+    for up in (True, False):  # the cell raised, or the rest lowered (into subnormal products at 300)
+        def spiked(u):
+            v = u.copy() if up else np.ldexp(u, -bits)
+            v[cy, cx] = np.ldexp(u[cy, cx], bits) if up else u[cy, cx]
+            return dev(v), 0 if up else bits
+        F, k = spiked(f)
+        H, _ = spiked(h)
+        for a, b, m in ((F, dev(h), k), (dev(f), H, k), (F, H, 2 * k)):
+            dg.dg_bracket(g, a, b, out)
+            check(out, J, m, scale)
+            dg.dg_bracket_parts(g, a, b, out, 1)
+            check(out, Jp, m, scale)
+        for mode, want in ((0, o.A(h)), (1, lap)):
+            dg.dg_laplace_apply(g, H, out, mode=mode)
+            check(out, want, k)
+        # a step's right-hand side, J and the viscous term, from the spiked vorticity
+        s = dg.Sim(g, dev(np.zeros(g.shape)), D=D, dt=1e-6)
+        z = dev(np.zeros(g.shape))
+        s.set_state(5, H, dev(f), dev(f), z, z)
+        s.set_cg(1e-30, 10, fixed_iters=1)
+        s.step(1)
+        b = [torch.empty(g.shape, dtype=torch.float64, device="cuda") for _ in range(5)]
+        s.get_state(*b)
+        check(b[3], D * lap - J, k, scale)
+
+
+def test_zero_far_from_a_compact_field(dg):
+    """A field of a few cells: exactly zero where its stencils do not reach."""
+    Nx, Ny, n = 40, 24, 4
+    g = dg.Grid(Nx, Ny, n)
+    f, h = np.random.default_rng(1).standard_normal((2, Ny, Nx, n, n))
+    h[:10], h[13:], h[:, :20], h[:, 23:] = 0, 0, 0, 0
+    out = torch.empty(g.shape, dtype=torch.float64, device="cuda")
+    dg.dg_bracket(g, dev(f), dev(h), out)
+    J = host(out).copy()
+    assert np.abs(J[9:14, 19:24]).max() > 0
+    J[8:15, 18:25] = 0
+    assert not J.any()
+    dg.dg_laplace_apply(g, dev(h), out, mode=1)
+    q = host(out).copy()
+    q[8:15, 18:25] = 0
+    assert not q.any()
