@@ -191,7 +191,8 @@ int dg_spectral_symbol(int N, int n, double L, double tau, int k, double* lam, d
  * eps32 times the row-sum bound of the scaled operator exceeds 5% of the smallest non-zero
  * eigenvalue of -Delta on the box (there a float32 apply is wrong by O(1) on the smoothest
  * modes and the sweeps of a solve from a poor guess contract slowly), else 0.  The choice
- * changes the inner iterates only, not what the solve converges to.
+ * changes the inner iterates only, not what the solve converges to.  (The fixed-point spectral
+ * solve has no inner iterates: there the mode has no effect.)
  * dg_grid_get_compensated_apply returns the mode in use.  Errors: DG_ERR_ARG.
  */
 int dg_grid_set_compensated_apply(dg_grid* g, int mode);
@@ -384,7 +385,9 @@ int dg_sim_set_cg(dg_sim* s, double tol, int maxit, int fixed_iters);
  * dg_sim_set_refinement -- DG_MIXED / DG_MIXED64: each float32 inner CG sweep stops when its
  * residual has fallen by tol_in (0 < tol_in < 1), or by half the factor still missing to the
  * CG tolerance if that is looser; at most max_sweeps >= 1 float64 refinement sweeps per solve
- * (the float64 residual must reach the CG tolerance of dg_sim_create / dg_sim_set_cg).
+ * (the float64 residual must reach the CG tolerance of dg_sim_create / dg_sim_set_cg).  Where a
+ * single simulation takes the fixed-point spectral solve (see DG_MIXED), max_sweeps caps its
+ * applications of A^+, and tol_in and the inner iteration cap of dg_sim_set_cg have no use.
  * Defaults: tol_in = 1e-4, max_sweeps = 40.
  */
 int dg_sim_set_refinement(dg_sim* s, double tol_in, int max_sweeps);

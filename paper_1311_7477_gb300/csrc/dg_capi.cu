@@ -990,6 +990,8 @@ int sim_solve(dg_sim* s, const double* omega, const double* xa, double ca, const
     A.floor2 = g->floor2;
     A.keep_mean = g->bc;
     A.maxit = s->fixed_iters > 0 ? std::max(s->maxit, s->fixed_iters) : s->maxit;
+    // the mixed modes' maxit caps a sweep's inner iterations; here an application stands for a sweep
+    if (s->precision == DG_MIXED || s->precision == DG_MIXED64) A.maxit = s->max_sweeps;
     A.fixed_iters = s->fixed_iters;
     A.sumW = g->Lx * g->Ly;
     rc = dispatch_n(g->n, [&](auto nc) { return launch_cg<double, decltype(nc)::value>(g, A, s->ws, st, s); });

@@ -401,3 +401,21 @@ def test_zero_far_from_a_compact_field(dg):
     q = host(out).copy()
     q[8:15, 18:25] = 0
     assert not q.any()
+
+
+@pytest.mark.parametrize("mode", ["mixed", "mixed64"])
+def test_mixed_caps_on_the_fixed_point_solve(dg, mode):
+    """The inner iteration cap of a mixed simulation is no cap on the solve's applications (several are
+    needed here, to the rounding floor below an unreachable tolerance); its sweep cap is."""
+    g = dg.Grid(32, 32, 4)
+    g.set_precond("spectral")
+    w = np.random.default_rng(3).standard_normal(g.shape)
+    s = dg.Sim(g, dev(w), D=0.0, dt=1e-7, precision={"mixed": dg.DG_MIXED, "mixed64": dg.DG_MIXED64}[mode], cg_tol=1e-10)
+    s.set_cg(1e-18, 1)
+    s.step(2)
+    info = s.status()
+    assert info.status == 0 and info.cg_iters_last > 1
+    s.set_refinement(1e-4, 1)
+    s.step(1)
+    info = s.status(check=False)
+    assert info.status == dg.DG_ERR_NOCONV and info.cg_iters_last == 1
