@@ -1279,17 +1279,18 @@ __device__ __forceinline__ void cg_tile_apply(const Tab& C, const Geom& G, int t
   __syncthreads();
 }
 
-// One tile pass of the solve's operator, (g, k, q) handed to out: a float64 solve in fixed point
-// (fx_tile_apply), a float32 one in float32 or -- with the compensated apply enabled -- in
+// One tile pass of the solve's operator, (g, k, u, q) handed to out: a float64 solve in fixed point
+// (fx_tile_apply; u is loaded again, own(g)), a float32 one in float32 or -- with the compensated apply enabled -- in
 // double-float arithmetic on the same float32 values, the result rounded to float32.  A float32 evaluation of Ahat u has an absolute error of about
 // eps32 |Ahat| |u|, which on the smoothest modes of a fine grid (eigenvalue ~1 against
 // |Ahat| ~ 1e7 at 1024^2 cells, n = 5) is as large as Ahat u itself; the double-float apply
 // brings it down to ~eps32^2 |Ahat| |u|.
-template <typename T, int N, class LoadF, class OutF>
+template <typename T, int N, class LoadF, class OwnF, class OutF>
 __device__ __forceinline__ void solve_apply(const Ops2D<T, N>& C, const Geom& G, int tile, SolveCtx<T>& X,
-                                            LoadF&& load, OutF&& out) {
+                                            LoadF&& load, OwnF&& own, OutF&& out) {
   if constexpr (std::is_same<T, double>::value) {
-    fx_tile_apply<N, false, false>(C.kx, C.ky, X.ks, G, tile, X.sU, load, out);
+    fx_tile_apply<N, false, false>(C.kx, C.ky, X.ks, G, tile, X.sU, load,
+                                   [&](size_t g, int k, T q) { out(g, k, own(g), q); });
   } else {
     if (X.kdf) {
       SolveCtx<df> W;
@@ -1301,10 +1302,10 @@ __device__ __forceinline__ void solve_apply(const Ops2D<T, N>& C, const Geom& G,
       cg_tile_apply<df, N>(
           *static_cast<const OpsK<df, N>*>(X.kdf), G, tile, W,
           [&](size_t g, int k, bool interior) { return df(load(g, k, interior)); },
-          [&](size_t g, int k, df, df q) { out(g, k, to_float(q)); });
+          [&](size_t g, int k, df u, df q) { out(g, k, u.hi, to_float(q)); });
       return;
     }
-    cg_tile_apply<T, N>(C, G, tile, X, load, [&](size_t g, int k, T, T q) { out(g, k, q); });
+    cg_tile_apply<T, N>(C, G, tile, X, load, out);
   }
 }
 
@@ -2214,9 +2215,8 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
       T rt = T(0), yt = T(0);
       for (int t = X.vrank; t < ntiles; t += X.vsize) {
         solve_apply<T, N>(
-            C, G, t, X, [&](size_t g, int, bool) { return __ldcg(V.y + g); },
-            [&](size_t g, int k, T qv) {
-              const T yv = __ldcg(V.y + g);
+            C, G, t, X, [&](size_t g, int, bool) { return __ldcg(V.y + g); }, [&](size_t g) { return __ldcg(V.y + g); },
+            [&](size_t g, int k, T yv, T qv) {
               const T r = rhs_at<T, N>(C, Bsrc, g, k) - qv;
               __stcg(V.r + g, r);
               if (ay) __stcg(ay + g, qv);
@@ -2271,9 +2271,10 @@ __device__ __forceinline__ int cg_iterate(const Ops2D<T, N>& C, const Geom& G, c
             if (interior) __stcg(pout + g, pv);
             return pv;
           },
-          [&](size_t g, int, T qv) {  // p of the tile: written above, by this block
+          [&](size_t g) { return __ldcg(pout + g); },  // written above, by this block
+          [&](size_t g, int, T pv, T qv) {
             __stcg(V.q + g, qv);
-            pq = fma(__ldcg(pout + g), qv, pq);
+            pq = fma(pv, qv, pq);
           });
     }
     T pqs = T(0);
@@ -2443,7 +2444,8 @@ __device__ __forceinline__ int fx_spectral_iterate(const Ops2D<double, N>& C, co
             }
             return y;
           },
-          [&](size_t g, int k, double q) {
+          [](size_t) { return 0.0; },
+          [&](size_t g, int k, double, double q) {
             const double r = rhs_at<double, N>(C, Bsrc, g, k) - q;
             __stcg(V.r + g, r);
             if (ay) __stcg(ay + g, q);
@@ -2698,7 +2700,8 @@ __device__ __forceinline__ void cg_solve(const Ops2D<T, N>& C, const Geom& G, co
             if (interior) __stcg(y0v + g, tv);
             return tv;
           },
-          [&](size_t g, int k, T qv) {
+          [](size_t) { return T(0); },
+          [&](size_t g, int k, T, T qv) {
             const T b = rhs_at<T, N>(C, RhsSource<T>{A.omega, A.rhs, wbar}, g, k);
             const T r = b - qv;
             __stcg(A.v.r + g, r);
@@ -2871,8 +2874,8 @@ __device__ __forceinline__ void mixed_residual(const Ops2D<double, N>& Cd, const
           if (interior) __stcg(A.y + g, v);
           return v;
         },
-        [&](size_t g, int k, double qv) {
-          const double yv = __ldcg(A.y + g);
+        [&](size_t g) { return __ldcg(A.y + g); },
+        [&](size_t g, int k, double yv, double qv) {
           const double b = Cd.sw[k] * (A.omega[g] - wbar);
           const double r = b - qv;
           if (A.ay) __stcg(A.ay + g, qv);
