@@ -1801,7 +1801,7 @@ size_t batch_smem_for(const dg_batch* b, const dg_sim* s) {
     constexpr int N = decltype(nc)::value;
     const size_t rhs = rhs_smem_bytes<N>(Gr.TY, Gr.TX);
     const size_t sol = s->precision == DG_FP64 ? cg_smem_bytes<double, N>(Gc.TY, Gc.TX, Lmax, g->precond, pow2_grid(g))
-                                               : mixed_smem_bytes<N>(Gc.TY, Gc.TX, Lmax, g->precond, pow2_grid(g));
+                                               : mixed_smem_bytes<N>(Gc, Lmax, g->precond, pow2_grid(g), false);
     out = batch_ops_bytes<N>() + std::max(rhs, sol);
     return DG_OK;
   });

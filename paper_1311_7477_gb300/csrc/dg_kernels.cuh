@@ -2810,6 +2810,7 @@ struct MixedArgs {
   int precise_apply;
   int keep_mean;       // homogeneous Dirichlet: b = sqrt(W) omega (no mean removed)
   FxScale ks;          // factors of the fixed-point operator (float64 residuals)
+  bool half;           // the residuals' tiles are half the solve's (launch_mixed)
 };
 
 // The operator tables a mixed solve stages in shared memory: float64 (residuals), float32
@@ -2819,9 +2820,24 @@ __host__ __device__ constexpr size_t mixed_ops_bytes() {
   return table_bytes<Ops2D<double, N>>() + table_bytes<Ops2D<float, N>>() + table_bytes<OpsK<df, N>>();
 }
 
+// The tiles of the float64 residuals: the solve's, or (half) half of them.
+__host__ __device__ inline Geom residual_geom(Geom G, bool half) {
+  if (half) {
+    if (G.TX >= G.TY)
+      G.TX = (G.TX + 1) / 2;
+    else
+      G.TY = (G.TY + 1) / 2;
+    G.tilesX = (G.Nx + G.TX - 1) / G.TX;
+    G.tilesY = (G.Ny + G.TY - 1) / G.TY;
+  }
+  return G;
+}
+
 template <int N>
-__host__ __device__ constexpr size_t mixed_smem_bytes(int TY, int TX, int Lmax, int kind, bool pow2) {
-  size_t t = cg_tile_bytes<double, N>(TY, TX);
+inline size_t mixed_smem_bytes(const Geom& G, int Lmax, int kind, bool pow2, bool half) {
+  const int TY = G.TY, TX = G.TX;
+  const Geom R = residual_geom(G, half);
+  size_t t = fx_apply_bytes<N>(R.TY, R.TX);
   const size_t w = cg_tile_values<df, N>(TY, TX) * 8, l = pc_line_bytes<float, N>(kind, Lmax, pow2);
   t = t > w ? t : w;
   return (kind == kPrecondTwoLevel ? align16(sizeof(float) * N * N * N * N) : 0) + align16(t > l ? t : l);
@@ -2935,7 +2951,7 @@ __device__ __forceinline__ void mixed_solve(const Ops2D<double, N>& Cd, const Op
     double yy = 0.0;
     {
       double r2 = 0.0, b2 = 0.0, y2 = 0.0;
-      mixed_residual<N>(Cd, G, A, wbar, pass == 0, Xd, r2, b2, y2);
+      mixed_residual<N>(Cd, residual_geom(G, A.half), A, wbar, pass == 0, Xd, r2, b2, y2);
       if (!reduce_all3(Xd, r2, b2, y2, rr, bb, yy)) {
         flags |= kFlagTimeout;
         goto finish;

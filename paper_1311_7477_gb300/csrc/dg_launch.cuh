@@ -111,8 +111,12 @@ template <int N>
 int launch_mixed(const dg_grid* g, MixedArgs A, const Workspace& w, cudaStream_t st, dg_sim* timed) {
   bool cluster = false;
   Geom G = solve_geom(g, true, &cluster);
+  // four blocks per SM where there are tiles for them: of 8 x 8 cells at n = 5 the float64 residuals take
+  // 45.6 KB, which leaves three, so they run on half tiles there (two-level, 512^2 cells: 47.6 ms on
+  // whole tiles, 43.5 on half ones; 128^2, which has no tiles for a fourth block: 4.85 and 5.03)
+  A.half = N == 5 && G.tilesX * G.tilesY > 3 * g->num_sms;
   auto smem_of = [&](const Geom& Gx) {
-    return mixed_ops_bytes<N>() + mixed_smem_bytes<N>(Gx.TY, Gx.TX, std::max(g->Nx, g->Ny), A.precond, pow2_grid(g));
+    return mixed_ops_bytes<N>() + mixed_smem_bytes<N>(Gx, std::max(g->Nx, g->Ny), A.precond, pow2_grid(g), A.half);
   };
   size_t smem = smem_of(G);
   auto kern = mixed_cg_kernel<N>;
