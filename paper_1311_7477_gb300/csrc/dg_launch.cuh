@@ -64,6 +64,19 @@ int launch_solve(Kern kern, bool cluster, int grid, size_t smem, cudaStream_t st
   return DG_OK;
 }
 
+// The blocks that a solve can use: one per tile, and one per unit of the longer lines' direct spectral
+// DFTs, which take longer than the barriers of a few more blocks.  (One float64 solve on tiles alone and
+// so: 100^2 cells, n = 3 618 and 510 us; 160^2, n = 2 911 and 823; mixed 475 and 411.  Units of the
+// shorter lines are no reason: 60 x 200, n = 2, mixed 293 on 100 blocks, 365 on 200.)  A cluster has one
+// block per tile.
+template <int N>
+int solve_units(const dg_grid* g, const Geom& G, int precond, bool cluster = false) {
+  const int tiles = G.tilesX * G.tilesY;
+  if (precond != kPrecondSpectral || pow2_grid(g) || cluster) return tiles;
+  const int rows = (g->Ny + 1) / 2 * N, cols = (g->Nx / 2 + 1) * N;
+  return std::max(tiles, g->Nx > g->Ny ? rows : g->Nx < g->Ny ? cols : std::max(rows, cols));
+}
+
 template <typename T, int N, typename TP>
 int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_t st, dg_sim* timed) {
   bool cluster = false;
@@ -80,7 +93,7 @@ int launch_cg(const dg_grid* g, CgArgs<T, TP> A, const Workspace& w, cudaStream_
   int per_sm = 0;
   CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
   if (per_sm < 1) return fail(DG_ERR_CUDA, "CG kernel does not fit on an SM (smem %zu B)", smem);
-  int grid = std::min(per_sm * g->num_sms, G.tilesX * G.tilesY);
+  int grid = std::min(per_sm * g->num_sms, solve_units<N>(g, G, A.precond));
   grid = std::min(grid, w.grid_cap);
   A.part = reinterpret_cast<T*>(w.part);
   A.ks = g->ks;
@@ -129,7 +142,7 @@ int launch_mixed(const dg_grid* g, MixedArgs A, const Workspace& w, cudaStream_t
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
   }
   if (per_sm < 1) return fail(DG_ERR_CUDA, "mixed CG kernel does not fit on an SM (smem %zu B)", smem);
-  int grid = std::min(per_sm * g->num_sms, G.tilesX * G.tilesY);
+  int grid = std::min(per_sm * g->num_sms, solve_units<N>(g, G, A.precond, cluster));
   grid = std::min(grid, w.grid_cap);
   A.rf = w.rf;
   A.v = CgVectors<float>{w.fe, w.fr, w.fp0, w.fp1, w.fq};
