@@ -248,13 +248,13 @@ __host__ __device__ constexpr int fx_cell() {
 // How far below a tile's largest value its cells may lie in fixed point, in bits.  Errors there are
 // relative to the tile's largest value, in float64 to the values around the node.  Away from a cell 2^s
 // times the others they pass those of the float64 tile at s = 6 (operators) and, for the bracket, whose
-// two fields' bits add up, at s = 4, 4, 4, 3, 2 for n = 1..5, and double with each bit: at 8 bits
-// they are 3.5 times and 15 to 80 times the float64 tile's.  A tile with a cell further down, its eight
-// neighbours too (the zero line of a field does not count), is left to float64: the tail of a compact
-// vortex, the foot of a thin shear layer.  Such a tile takes four times as long; what it takes to
-// find out costs the others 1 to 5% (1000^2 cells, n = 4: 704 -> 714 us; 501 x 373, n = 3: 69 -> 72;
-// Laplacian, 500 x 300, n = 5: 70.5 -> 72.2).
-constexpr int kFxRange = 8;
+// two fields' bits add up, at s = 4, 4, 4, 3, 2 for n = 1..5, and double with each bit: at 14 bits they
+// are still below 1e-12 of the values around the node.  A tile with a cell further down, its eight
+// neighbours too (the zero line of a field does not count), is left to float64: the tail of a narrow
+// vortex.  Such a tile takes four times as long (at a limit of 8 bits the whole far field of a
+// Gaussian of a tenth of the box would be such tiles, at 14 a third; where zero lines of
+// proportional fields cross, up to 13 bits occur).
+constexpr int kFxRange = 14;
 
 // The smallest non-zero magnitude word of what a thread staged, less 1 (zeros wrap around to the largest).
 __device__ __forceinline__ unsigned fx_low(unsigned low, double v) { return min(low, fx_mag(v) - 1u); }
@@ -300,27 +300,25 @@ __device__ __noinline__ bool fx_far(const TileBox& B, const double* f, const dou
   return __syncthreads_or(far);
 }
 
-// A quick look at the converted tile before that one: whether a cell has no node near the largest values
-// among the middle nodes of itself and its eight neighbours.  (The zero lines of resolved fields, which most
-// tiles that come here have, end here.)  In every thread, after a block synchronisation.
+// A quick look before that one: whether a cell has no node near the largest values among the middle
+// nodes of itself and its eight neighbours.  (The zero lines of resolved fields, which most tiles that
+// come here have, end here.)  In every thread, after a block synchronisation.
 template <int N>
-__device__ __forceinline__ bool fx_lonely(const TileBox& B, const fx* f, const fx* g) {
+__device__ __forceinline__ bool fx_lonely(const TileBox& B, const double* f, const double* g, int ef, int eg) {
   constexpr int CS = fx_cell<N>();
   bool lonely = false;
   for (int c = threadIdx.x; c < B.TYe * B.TXe; c += blockDim.x) {
     const int ry = quot(c, B.mTXe), rx = c - ry * B.TXe;
     const int o = (ry * B.BW + rx) * CS + N / 2 * (N + 1);
-    int least = 64;
+    int top = 0;
 #pragma unroll
     for (int y = 0; y < 3; ++y)
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
         const int i = o + (y * B.BW + x) * CS;
-        // high words of the largest values lie in 2^29 .. 2^30
-        const int hg = g[i].h, hf = f ? f[i].h : 1 << 29;
-        least = min(least, __clz(hg ^ (hg >> 31)) + __clz(hf ^ (hf >> 31)) - 4);
+        top = max(top, ((__double2hiint(g[i]) >> 20) & 0x7ff) + (f ? (__double2hiint(f[i]) >> 20) & 0x7ff : 0));
       }
-    lonely |= least > kFxRange;
+    lonely |= eg + (f ? ef : 0) - top > kFxRange;
   }
   return __syncthreads_or(lonely);
 }
@@ -510,84 +508,82 @@ __device__ __forceinline__ void rhs_tile(const FxRhs<N>& F, const Ops2D<double, 
 
   const bool viscous = A.visc != 0.0 && !A.bracket_only;
   const int nw = int(blockDim.x >> 5), lane = threadIdx.x & 31;
-  int uj, ul;  // units of the products and of the viscous term, 2^uj and 2^ul
-  for (bool again = false;; again = true) {
-    // stage the two fields and their largest and smallest magnitudes
-    {
-      double* rF = reinterpret_cast<double*>(sF);
-      double* rG = reinterpret_cast<double*>(sG);
-      unsigned mf = 0, mg = 0, nf = ~0u, ng = ~0u;
-      const int BWe = B.TXe + 2, BHe = B.TYe + 2;
-      const int rowlen = BWe * NN, total = BHe * rowlen;
-      const unsigned mrow = magic_of(rowlen);
+  // stage the two fields and their largest and smallest magnitudes
+  {
+    double* rF = reinterpret_cast<double*>(sF);
+    double* rG = reinterpret_cast<double*>(sG);
+    unsigned mf = 0, mg = 0, nf = ~0u, ng = ~0u;
+    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+    const int rowlen = BWe * NN, total = BHe * rowlen;
+    const unsigned mrow = magic_of(rowlen);
 #pragma unroll 4
-      for (int i = threadIdx.x; i < total; i += blockDim.x) {
-        const int br = quot(i, mrow);
-        const int j = i - br * rowlen;
-        const int bc = j / NN, k = j - bc * NN;
-        const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
-        const int o = (br * BW + bc) * CS + k;
-        if (Gen && G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)) {
-          rF[o] = 0.0;
-          rG[o] = 0.0;
-          continue;
-        }
-        const size_t g = ((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k;
-        const double f = A.psi[g], w = A.omega_in[g];
-        rF[o] = f;
-        rG[o] = w;
-        mf = max(mf, fx_mag(f));
-        mg = max(mg, fx_mag(w));
-        nf = fx_low(nf, f);
-        ng = fx_low(ng, w);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int br = quot(i, mrow);
+      const int j = i - br * rowlen;
+      const int bc = j / NN, k = j - bc * NN;
+      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+      const int o = (br * BW + bc) * CS + k;
+      if (Gen && G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)) {
+        rF[o] = 0.0;
+        rG[o] = 0.0;
+        continue;
       }
-      mf = __reduce_max_sync(0xffffffffu, mf);
-      mg = __reduce_max_sync(0xffffffffu, mg);
-      nf = __reduce_min_sync(0xffffffffu, nf);
-      ng = __reduce_min_sync(0xffffffffu, ng);
-      if (A.psi_scaled && threadIdx.x < NN) s_isw[threadIdx.x] = F.isw[threadIdx.x];
-      if ((threadIdx.x & 31) == 0) {
-        s_mag[0][threadIdx.x >> 5] = mf;
-        s_mag[1][threadIdx.x >> 5] = mg;
-        s_mag[2][threadIdx.x >> 5] = nf;
-        s_mag[3][threadIdx.x >> 5] = ng;
-      }
+      const size_t g = ((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k;
+      const double f = A.psi[g], w = A.omega_in[g];
+      rF[o] = f;
+      rG[o] = w;
+      mf = max(mf, fx_mag(f));
+      mg = max(mg, fx_mag(w));
+      nf = fx_low(nf, f);
+      ng = fx_low(ng, w);
     }
-    __syncthreads();
-    const unsigned mf = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[0][lane] : 0u);
-    const unsigned mg = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[1][lane] : 0u);
-    const unsigned nf = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[2][lane] : ~0u);
-    const unsigned ng = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[3][lane] : ~0u);
-    const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
-    // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any)
-    const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
-    uj = uf + ug + 2 * D.e + 60;
-    ul = ug + (F.l.lap ? static_cast<const FxTable<N>*>(F.l.lap)->e : Lp.e);
-    // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
-    const bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.l.ok && abs(ul) <= 600));
-    if (!covered || (again && fx_far<N>(B, reinterpret_cast<const double*>(sF), reinterpret_cast<const double*>(sG), ef,
-                                        eg, viscous, reinterpret_cast<int*>(sA)))) {
-      __syncthreads();  // the staging is reused
-      rhs_tile_float<N>(C, G, A, tile, smem);
-      return;
+    mf = __reduce_max_sync(0xffffffffu, mf);
+    mg = __reduce_max_sync(0xffffffffu, mg);
+    nf = __reduce_min_sync(0xffffffffu, nf);
+    ng = __reduce_min_sync(0xffffffffu, ng);
+    if (A.psi_scaled && threadIdx.x < NN) s_isw[threadIdx.x] = F.isw[threadIdx.x];
+    if ((threadIdx.x & 31) == 0) {
+      s_mag[0][threadIdx.x >> 5] = mf;
+      s_mag[1][threadIdx.x >> 5] = mg;
+      s_mag[2][threadIdx.x >> 5] = nf;
+      s_mag[3][threadIdx.x >> 5] = ng;
     }
-    for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
-      const fx f = sF[i], w = sG[i];  // raw bits: {low, high} words
-      long long x = fx_from_bits(unsigned(f.l), unsigned(f.h), ef);
-      if (A.psi_scaled) {
-        const int k = i % CS;
-        FxAcc s;
-        fx_mac(s, s_isw[k < NN ? k : 0], fx_split(x));
-        x = fx_round(s);
-      }
-      sF[i] = fx_split(x);
-      sG[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), eg));
-    }
-    __syncthreads();
-    // values far apart (kFxRange), and perhaps a cell of nothing else: the tile is staged again, to look at
-    // its cells themselves
-    if (again || fx_spread(mf, nf) + fx_spread(mg, ng) <= kFxRange || !fx_lonely<N>(B, sF, sG)) break;
   }
+  __syncthreads();
+  const unsigned mf = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[0][lane] : 0u);
+  const unsigned mg = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[1][lane] : 0u);
+  const unsigned nf = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[2][lane] : ~0u);
+  const unsigned ng = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[3][lane] : ~0u);
+  const int ef = max(1, int(mf >> 20)), eg = max(1, int(mg >> 20));
+  // units of the fixed-point fields, 2^uf and 2^ug (of an all-zero field: any), of the products and of the
+  // viscous term
+  const int uf = mf ? ef - 1082 + (A.psi_scaled ? F.ei : 0) : 0, ug = mg ? eg - 1082 : 0;
+  int uj = uf + ug + 2 * D.e + 60;
+  const int ul = ug + (F.l.lap ? static_cast<const FxTable<N>*>(F.l.lap)->e : Lp.e);
+  // magnitudes below 2^63: units within 2^+-600 keep every result and factor a normal number
+  bool covered = F.ok && ef < 2047 && eg < 2047 && abs(uj) <= 600 && (!viscous || (F.l.ok && abs(ul) <= 600));
+  if (covered && fx_spread(mf, nf) + fx_spread(mg, ng) > kFxRange) {
+    const double *rF = reinterpret_cast<const double*>(sF), *rG = reinterpret_cast<const double*>(sG);
+    if (fx_lonely<N>(B, rF, rG, ef, eg)) covered = !fx_far<N>(B, rF, rG, ef, eg, viscous, reinterpret_cast<int*>(sA));
+  }
+  if (!covered) {
+    __syncthreads();  // the staging is reused
+    rhs_tile_float<N>(C, G, A, tile, smem);
+    return;
+  }
+  for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
+    const fx f = sF[i], w = sG[i];  // raw bits: {low, high} words
+    long long x = fx_from_bits(unsigned(f.l), unsigned(f.h), ef);
+    if (A.psi_scaled) {
+      const int k = i % CS;
+      FxAcc s;
+      fx_mac(s, s_isw[k < NN ? k : 0], fx_split(x));
+      x = fx_round(s);
+    }
+    sF[i] = fx_split(x);
+    sG[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), eg));
+  }
+  __syncthreads();
 
   // Which parts enter (Eq. J): J = s (c0 J++ + J+x + Jx+) with J+x = D_x(f g_y) - D_y(f g_x),
   // Jx+ = D_y(f_x g) - D_x(f_y g).
@@ -821,61 +817,55 @@ __device__ __forceinline__ void fx_tile_apply(const Op1D<double, N>& ox, const O
   long long* qy = qx + G.TY * G.TX * CS;
   const int lane = threadIdx.x & 31, nw = int(blockDim.x >> 5);
   const FxTable<N>* tab = static_cast<const FxTable<N>*>(Lap ? S.lap : S.stiff);
-  int uq;
-  bool covered;
-  for (bool again = false;; again = true) {
-    unsigned m = 0, low = ~0u;
-    {
-      double* rU = reinterpret_cast<double*>(sU);
-      const int BWe = B.TXe + 2, BHe = B.TYe + 2;
-      const int rowlen = BWe * NN, total = BHe * rowlen;
-      const unsigned mrow = magic_of(rowlen);
+  unsigned m = 0, low = ~0u;
+  {
+    double* rU = reinterpret_cast<double*>(sU);
+    const int BWe = B.TXe + 2, BHe = B.TYe + 2;
+    const int rowlen = BWe * NN, total = BHe * rowlen;
+    const unsigned mrow = magic_of(rowlen);
 #pragma unroll 4
-      for (int i = threadIdx.x; i < total; i += blockDim.x) {
-        const int br = quot(i, mrow);
-        const int j = i - br * rowlen;
-        const int bc = j / NN, k = j - bc * NN;
-        const bool rowhalo = (br == 0) || (br == BHe - 1), colhalo = (bc == 0) || (bc == BWe - 1);
-        const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
-        const int o = (br * BW + bc) * CS + k;
-        if (rowhalo && colhalo) {  // the 5-cell operators never read the corners
-          if constexpr (Local) rU[o] = 0.0;
-          continue;
-        }
-        double v = 0.0;  // Dirichlet: zero outside
-        if (!(G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)))
-          v = load(((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k, k, !(rowhalo || colhalo));
-        rU[o] = v;
-        m = max(m, fx_mag(v));
-        if constexpr (Local) low = fx_low(low, v);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int br = quot(i, mrow);
+      const int j = i - br * rowlen;
+      const int bc = j / NN, k = j - bc * NN;
+      const bool rowhalo = (br == 0) || (br == BHe - 1), colhalo = (bc == 0) || (bc == BWe - 1);
+      const int gy = B.ty0 + br - 1, gx = B.tx0 + bc - 1;
+      const int o = (br * BW + bc) * CS + k;
+      if (rowhalo && colhalo) {  // the 5-cell operators never read the corners
+        if constexpr (Local) rU[o] = 0.0;
+        continue;
       }
-      m = __reduce_max_sync(0xffffffffu, m);
-      if constexpr (Local) low = __reduce_min_sync(0xffffffffu, low);
-      if ((threadIdx.x & 31) == 0) {
-        s_mag[threadIdx.x >> 5] = m;
-        if constexpr (Local) s_mag[16 + (threadIdx.x >> 5)] = low;
-      }
+      double v = 0.0;  // Dirichlet: zero outside
+      if (!(G.bc && (gy < 0 || gy >= G.Ny || gx < 0 || gx >= G.Nx)))
+        v = load(((size_t)wrap_index(gy, G.Ny) * G.Nx + wrap_index(gx, G.Nx)) * NN + k, k, !(rowhalo || colhalo));
+      rU[o] = v;
+      m = max(m, fx_mag(v));
+      if constexpr (Local) low = fx_low(low, v);
     }
-    __syncthreads();
-    m = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[lane] : 0u);
-    const int em = max(1, int(m >> 20));
-    uq = m ? em - 1082 + (tab ? tab->e : O.e) : 0;
-    covered = S.ok && em < 2047 && abs(uq) <= 600;
-    if constexpr (Local) {
-      low = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[16 + lane] : ~0u);
-      if (covered && again)
-        covered = !fx_far<N>(B, nullptr, reinterpret_cast<const double*>(sU), 0, em, true, reinterpret_cast<int*>(qx));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if constexpr (Local) low = __reduce_min_sync(0xffffffffu, low);
+    if ((threadIdx.x & 31) == 0) {
+      s_mag[threadIdx.x >> 5] = m;
+      if constexpr (Local) s_mag[16 + (threadIdx.x >> 5)] = low;
     }
-    if (!covered) break;
+  }
+  __syncthreads();
+  m = __reduce_max_sync(0xffffffffu, lane < nw ? s_mag[lane] : 0u);
+  const int em = max(1, int(m >> 20)), uq = m ? em - 1082 + (tab ? tab->e : O.e) : 0;
+  bool covered = S.ok && em < 2047 && abs(uq) <= 600;
+  if constexpr (Local) {
+    low = __reduce_min_sync(0xffffffffu, lane < nw ? s_mag[16 + lane] : ~0u);
+    const double* rU = reinterpret_cast<const double*>(sU);
+    if (covered && fx_spread(m, low) > kFxRange && fx_lonely<N>(B, nullptr, rU, 0, em))
+      covered = !fx_far<N>(B, nullptr, rU, 0, em, true, reinterpret_cast<int*>(qx));
+  }
+  const int nc = B.TYe * B.TXe;
+  if (covered) {
     for (int i = threadIdx.x; i < boxc * CS; i += blockDim.x) {
       const fx w = sU[i];  // raw bits: {low, high} words
       sU[i] = fx_split(fx_from_bits(unsigned(w.l), unsigned(w.h), em));
     }
     __syncthreads();
-    if (!Local || again || fx_spread(m, low) <= kFxRange || !fx_lonely<N>(B, nullptr, sU)) break;
-  }
-  const int nc = B.TYe * B.TXe;
-  if (covered) {
     const unsigned mnc = magic_of(nc);
     if (tab) fx_lines_table<N>(tab, B, sU, qx, qy, G.TX, 0);
     for (int u = threadIdx.x; u < (tab ? 0 : 2 * nc * N); u += blockDim.x) {

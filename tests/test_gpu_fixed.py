@@ -341,8 +341,8 @@ def test_pointwise_bracket(dg, Nx, Ny, n, bc):
 @pytest.mark.parametrize("bits", [5, 8, 9, 20, 45, 70, 300])
 def test_cells_far_below_their_tile(dg, n, bc, bits):
     """A cell 2^bits times the others, or others that are that much smaller: away from it the operators'
-    results are those without it, to the bar of the other fields (1e-12 of the local scale; 2^-53 and
-    the table of errors at the range's end, 80 at most, leave a hundredfold)."""
+    results are those without it, to the bar of the other fields, 1e-12 of the local scale (2^12 times
+    2^-53 where the fixed-point range ends)."""
     Nx, Ny, Lx, Ly, D = 19, 17, 1.5, 2.0, 0.05
     g = dg.Grid(Nx, Ny, n, Lx, Ly, bc=bc)
     g.set_tiles(16 if n < 3 else 8, 16 if n < 3 else 8)  # (not the small tiles of a small grid)
