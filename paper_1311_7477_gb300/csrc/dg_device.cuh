@@ -362,11 +362,12 @@ struct BarrierState {
 // Waits of a block at the barrier give up after this many polls (~1 s with the sleep
 // below) and raise kFlagTimeout; every later barrier then returns false at once.
 constexpr unsigned long long kSpinCap = 1ull << 23;
-// An acquire drops the SM's L1 lines, those of the blocks still at work on it too.  After the polls of
-// a short wait (about 10 us) a block therefore polls without, and acquires once at the end.  (Phases of
+// An acquire drops the SM's L1 lines, those of the blocks still at work on it too.  After the polls of a
+// short wait (about 40 us) a block therefore polls without, and acquires once at the end.  (Phases of
 // long units with tables in L1: two-level solve, mixed, 1000 x 300 cells, n = 1, 68.4 ms with an acquire
-// in every poll, 35.9 so; spectral, mixed, 160^2, n = 5, 2.33 and 2.01 ms.)
-constexpr unsigned long long kAcquirePolls = 16;
+// in every poll, 36.2 so; spectral, mixed, 160^2, n = 5, 2.33 and 1.93 ms.  After 16 polls already: ten
+// steps of 32^2, n = 3 take 725 us, 717 so.)
+constexpr unsigned long long kAcquirePolls = 64;
 
 // The nblk blocks of a (virtual) grid meet here: all blocks of a cooperative launch, or the
 // blocks of one group of a batched launch.  Returns false if any block raised an error.
