@@ -468,15 +468,16 @@ __device__ __noinline__ int fx_jpp(const Geom& G, const TileBox& B, fx* sF, fx* 
 // One tile of the right-hand side in fixed point (smem: rhs_smem_bytes<N>(G.TY, G.TX)).
 //
 // What bounds it: the integer pipe (60% busy with the multiply-adds on 512^2 cells, n = 5) and the
-// synchronisations between phases; the float64 pipe only does the update (8%).  Per bracket, before
-// (the same phases in float64) and now: 1000^2 cells, n = 4 2396 and 695 us; 1000^2, n = 5 4.8 ms and
-// 1223 us; 100^2, n = 4 38.9 and 16.4 us; 501 x 373, n = 3 158 (in double-float) and 72 us.  A thread computes a whole line of a cell (its n nodes along x or y):
+// synchronisations between phases; the float64 pipe only does the update (8%).  Per bracket, in float64
+// (the same phases) and now: 1000^2 cells, n = 4 2396 and 710 us; 1000^2, n = 5 4.8 ms and 1.21 ms;
+// 100^2, n = 4 38.9 and 16.4 us; 501 x 373, n = 3 158 (in double-float) and 74 us.  A thread computes a
+// whole line of a cell (its n nodes along x or y):
 // it reads the n values of the line and the neighbours' once, evaluates their face traces itself
 // (as many multiply-adds as evaluating each trace once and storing it, one phase and 12 n arrays
 // less), and takes its coefficients from the constant bank.  Phases (a block synchronisation after
 // each):
-//   stage f = psi and g = omega with their halo ring, find the tile's largest magnitudes,
-//   convert to fixed point;
+//   stage f = psi and g = omega with their halo ring, find the tile's largest and smallest magnitudes
+//   (and, where they are far apart, whether a cell is too far down: kFxRange), convert to fixed point;
 //   x-lines of rows [-1, TYe]:  f_x, g_x, h2 = f_x g - f g_x;
 //   y-lines of columns [-1, TXe]:  f_y, g_y, J++ = f_x g_y - f_y g_x, h1 = f g_y - f_y g;
 //   x-lines of the tile: D_x h1 (over f); y-lines: J++ + D_y h2;   [viscous: lx g, ly g]

@@ -1,13 +1,12 @@
 """The mixed-precision paths against the FP64 oracle.
 
-DG_MIXED evaluates the bracket and the viscous term in double-float arithmetic on the float32
-pipe (dg_bracket_mixed: each value the unevaluated sum of two floats, about 48 significant
-bits) and solves the Poisson equation by float64 refinement sweeps around a float32 inner
-PCG; DG_MIXED64 keeps the bracket in float64.  State, update and invariants are float64.
+DG_MIXED and DG_MIXED64 evaluate the bracket and the viscous term as DG_FP64 does (in 64-bit fixed
+point; dg_bracket_mixed is dg_bracket) and solve the Poisson equation by float64 refinement sweeps
+around a float32 inner PCG, or by the fixed-point spectral solve where it applies.  State, update
+and invariants are float64.
 
-Bars: the double-float bracket matches the oracle to 1e-12 in relative L2 (its rounding is
-about 2^-46 of the terms that cancel in J, against 2^-52 for float64) and keeps J(f, f) = 0
-bitwise; one step of either mode from an identical state is within 1e-10 of the oracle's step
+Bars: the bracket matches the oracle to 1e-12 in relative L2 and keeps J(f, f) = 0 bitwise;
+one step of either mode from an identical state is within 1e-10 of the oracle's step
 (the target of the mixed-precision pattern), with psi meeting the float64 solver tolerance on
 the oracle's own operator.
 """
